@@ -22,10 +22,17 @@
 // K.Q^T MMAs and TMEM owner, warp 14 = issuer of the P.V and sum MMAs (one
 // thread each; two issuers because a single thread's issue rate, not the tensor
 // pipe, bounded the loop), warps 2-13 = three softmax groups of four warps.
-// The groups take the tiles in turn (tile i belongs to group i % 3; a thread is
-// one cache position, TMEM lane quarter = warp % 4, and works through all N
-// columns of its tile), so the latencies of one tile (TMEM load, barrier,
-// hand-over) hide behind the exponentials of the two tiles the other groups are
+// The softmax stage has two organisations.  With a bf16 cache all three groups work on
+// every tile, each on a third of the columns (a thread is one cache position, TMEM lane
+// quarter = warp % 4), and tiles go through in pairs: one vote on the guard, one fence and
+// one hand-over to the P.V issuer for 256 positions, while the products of the pair before
+// and the K.Q^T of the next run beside.  (Handed over one by one, a tile costs about 2.1 k
+// cycles of which the exponentials are 0.4 k; in pairs the stream is bound by HBM at 80 rows
+// too: 72B-shaped layer of 32K positions 29.5 us against 30.0, 128K positions x 4 at 80
+// rows 321 us against 331 in turns.)
+// With an fp8 cache of up to 64 rows the groups take the tiles in turn (tile i belongs to
+// group i % 3, a thread works through all N columns of its tile), so the latencies of one
+// tile hide behind the exponentials of the two tiles the other groups are
 // on; S^T has a TMEM buffer per tile in flight.  The reference exponents m[] are
 // shared.  Tiles are handed to the P.V issuer strictly in order, through a
 // counter of committed tiles: a group may move m (and rescale the accumulators)
@@ -90,16 +97,19 @@ constexpr uint32_t kBoxBytes = 16384;       // 128 positions x 64 channels bf16,
 constexpr uint32_t kSlotBytes = 2 * kBoxBytes;   // a bf16 tile; an fp8 tile is one box
 constexpr uint32_t kA2Bytes = 2048;         // one 64 x 16 (bf16) or 64 x 32 (E4M3) constant tile
 constexpr float kGuard = 60.f;              // log2 units above m before a rescale
+constexpr uint32_t kGuardBits = (127u + 60u) << 7;     // 2^kGuard as bf16 bits
 constexpr float kGuard8 = 8.f;              // fp8 cache: probabilities stay below 2^8 (E4M3 ends at 448)
 constexpr float kHead8 = 3.f;               // fp8 cache: the largest score of a row in the split's first tile has probability 2^3
 constexpr float kMFloor = -1.0e30f;
 constexpr int kQBarrier = 1 + kSoftmaxGroups;   // named barrier over all softmax threads
+constexpr int kHand = 4;                   // barriers of each hand-over kind
 constexpr int kMaxRowsFp8 = 80;             // fp8 cache: 6 accumulator columns per padded row in 512
 
 struct TcConfig {
     int n_pad;   // MMA N: rows padded to a multiple of 16
     int ks, vs, pb;   // K slots, V slots, P buffers
-    int sb;           // S^T buffers in TMEM (2 or 3)
+    int sb;           // S^T buffers in TMEM (2 to 4)
+    int step;         // tiles handed over at a time (all groups on every tile: 2 where the buffers allow)
     int tmem_cols;
     int page_slots;   // paged cache: pool pages of this split's tiles, one entry per tile
     int slot_bytes;   // one K or V tile: 32 KB bf16, 16 KB fp8
@@ -107,7 +117,7 @@ struct TcConfig {
 
 // Byte offsets of the shared-memory regions (relative to a 1024-aligned base).
 struct SmemMap {
-    uint32_t k, v, q, p, a2, m, dl, tmx, vis, bars, misc, pages, total;
+    uint32_t k, v, q, p, a2, m, dl, tmx, bars, misc, pages, total;
 };
 __host__ __device__ inline SmemMap smem_map(const TcConfig &c)
 {
@@ -121,8 +131,7 @@ __host__ __device__ inline SmemMap smem_map(const TcConfig &c)
     s.m = o;    o += c.n_pad * 4;
     s.dl = o;   o += c.n_pad * 4;
     s.tmx = o;  o += 4 * c.n_pad * 4;
-    s.vis = o;  o += c.n_pad * 8;
-    s.bars = o; o += 8 * (2 * c.ks + 2 * c.vs + 4 * kSoftmaxGroups + 4);
+    s.bars = o; o += 8 * (2 * c.ks + 2 * c.vs + 4 * kHand + 4);
     s.misc = o; o += 16 + 4 * kSoftmaxWarps;     // TMEM address, abort flag, epoch of m, committed tiles, per-warp maxima of |q|
     s.pages = o; o += 4 * c.page_slots;
     s.total = o;
@@ -209,21 +218,32 @@ __device__ __forceinline__ void mma_ss(uint32_t d, uint64_t a, uint64_t b, uint3
     else mma_f16_ss(d, a, b, idesc, acc);
 }
 
-// Which draft slots a column's query sees: tail indices [lo, hi] (its own branch up to
-// itself); the context before the draft slots (tail index < 0) is visible to all.
-__device__ __forceinline__ bool column_sees(int2 lohi, int t)
+// The columns (query rows g * G + hg) that see a cache position: a range [lo, lo + n).  The
+// context before the draft slots (tail index t < 0) is visible to all; draft slot t to the
+// queries of its own branch from t on (the plain chain is one branch); a slot at or beyond
+// kv_len to none.
+struct Seen {
+    int lo;
+    uint32_t n;
+    __device__ __forceinline__ bool operator()(int col) const { return (uint32_t)(col - lo) < n; }
+};
+__device__ __forceinline__ Seen seen_by(int t, int G, int gamma, int branch_len)
 {
-    return t < 0 || (unsigned)(t - lohi.x) <= (unsigned)(lohi.y - lohi.x);
+    Seen s = {0, t < 0 ? 0xFFFFFFFFu : 0u};
+    if (t >= 0 && t < gamma) {
+        s.lo = t * G;
+        s.n = (uint32_t)((t / branch_len + 1) * branch_len * G - s.lo);
+    }
+    return s;
 }
 
-// exp2 of eight scaled scores of one position, packed to bf16; returns their maximum
-// kMask: 0 = every column sees the position; 1 = plain chain of draft tokens (query
-// col / G sees tail index t iff it is not below t); 2 = draft tree (table look-up)
-// kFp8: each probability goes out as two E4M3 values in neighbouring bytes, its leading
+// fp8 cache: exp2 of eight scaled scores of one position; returns the scores' maximum
+// kMask: the tile reaches into the draft slots, a column may not see the position
+// Each probability goes out as two E4M3 values in neighbouring bytes, its leading
 // four significant bits and the rest (see the head of this file).
-template <int kMask, bool kFp8>
+template <bool kMask>
 __device__ __forceinline__ float exp_chunk(const uint32_t (&r)[8], const float *m8, float scale,
-                                           const int2 *vis8, int col0, int G, int t, uint4 &dst)
+                                           Seen seen, int col0, uint4 &dst)
 {
     const float4 ma = *reinterpret_cast<const float4 *>(m8);
     const float4 mb = *reinterpret_cast<const float4 *>(m8 + 4);
@@ -231,35 +251,20 @@ __device__ __forceinline__ float exp_chunk(const uint32_t (&r)[8], const float *
     float x[8];
 #pragma unroll
     for (int k = 0; k < 8; ++k) x[k] = fmaf(__uint_as_float(r[k]), scale, -mm[k]);
-    if (kMask == 1) {
+    if (kMask) {
 #pragma unroll
-        for (int k = 0; k < 8; ++k) x[k] = ((col0 + k) / G >= t) ? x[k] : -INFINITY;
-    } else if (kMask == 2) {
-#pragma unroll
-        for (int k = 0; k < 8; ++k) x[k] = column_sees(vis8[k], t) ? x[k] : -INFINITY;
+        for (int k = 0; k < 8; ++k) x[k] = seen(col0 + k) ? x[k] : -INFINITY;
     }
     float mx = fmaxf(fmaxf(fmaxf(x[0], x[1]), fmaxf(x[2], x[3])),
                      fmaxf(fmaxf(x[4], x[5]), fmaxf(x[6], x[7])));
-    uint4 pk;
-    if (kFp8) {
-        uint32_t w[8];
+    uint32_t w[8];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const float pr = ex2(x[k]);
-            const float hd = e4m3_head(pr);
-            w[k] = pack_e4m3x2(hd, pr - hd);
-        }
-        pk.x = w[0] | (w[1] << 16);
-        pk.y = w[2] | (w[3] << 16);
-        pk.z = w[4] | (w[5] << 16);
-        pk.w = w[6] | (w[7] << 16);
-    } else {
-        pk.x = pack_bf16x2(ex2(x[0]), ex2(x[1]));
-        pk.y = pack_bf16x2(ex2(x[2]), ex2(x[3]));
-        pk.z = pack_bf16x2(ex2(x[4]), ex2(x[5]));
-        pk.w = pack_bf16x2(ex2(x[6]), ex2(x[7]));
+    for (int k = 0; k < 8; ++k) {
+        const float pr = ex2(x[k]);
+        const float hd = e4m3_head(pr);
+        w[k] = pack_e4m3x2(hd, pr - hd);
     }
-    dst = pk;
+    dst = make_uint4(w[0] | (w[1] << 16), w[2] | (w[3] << 16), w[4] | (w[5] << 16), w[6] | (w[7] << 16));
     return mx;
 }
 
@@ -269,9 +274,9 @@ __device__ __forceinline__ float exp_chunk(const uint32_t (&r)[8], const float *
 // draft slots, so columns are masked by what their query may see; the common tile carries
 // none of that.  The loop stays rolled: three groups run it at different places, and
 // the instruction cache holds the short form better.
-template <int kMask, bool kFp8>
+template <bool kMask>
 __device__ __forceinline__ float softmax_pass(uint32_t s_addr, int n8, const float *m_s, float scale,
-                                              const int2 *vis_s, int G, int t, uint8_t *prow, long long *tr,
+                                              Seen seen, uint8_t *prow, long long *tr,
                                               int tile)
 {
     float gmax = -INFINITY;
@@ -288,8 +293,7 @@ __device__ __forceinline__ float softmax_pass(uint32_t s_addr, int n8, const flo
         for (int u = 0; u < 4; ++u)
             if (cb + u < n8) {
                 uint4 pk;
-                gmax = fmaxf(gmax, exp_chunk<kMask, kFp8>(r[u], m_s + (cb + u) * 8, scale, vis_s + (cb + u) * 8,
-                                                          (cb + u) * 8, G, t, pk));
+                gmax = fmaxf(gmax, exp_chunk<kMask>(r[u], m_s + (cb + u) * 8, scale, seen, (cb + u) * 8, pk));
                 *reinterpret_cast<uint4 *>(prow + (cb + u) * 2048) = pk;
             }
         LVSPEC_TILE_TS(tr, 3, tile, (cb >> 2) * 3 + 2);     // their probabilities stored
@@ -300,50 +304,100 @@ __device__ __forceinline__ float softmax_pass(uint32_t s_addr, int n8, const flo
 // The same for a group that works on a share of the columns, chunks [c_lo, c_hi), of every
 // tile: exp2 of its chunks of S^T (up to
 // four TMEM loads in flight per wait), packed probabilities into pk, returns the
-// largest scaled score.  kMask != 0: the tile reaches into the draft slots, so
+// largest scaled score.  kMask: the tile reaches into the draft slots, so
 // columns are masked by what their query may see; the common tile carries none of that.
-template <int kMask, bool kFp8>
+template <bool kMask, int kC>
 __device__ __forceinline__ float softmax_pass_share(uint32_t s_addr, int c_lo, int c_hi, const float *m_s,
-                                              float scale, const int2 *vis_s, int G, int t,
-                                              uint4 (&pk)[kMaxChunks])
+                                              float scale, Seen seen, uint4 (&pk)[kC])
 {
     float gmax = -INFINITY;
 #pragma unroll
-    for (int h = 0; h < (kMaxChunks + 3) / 4; ++h) {
+    for (int h = 0; h < (kC + 3) / 4; ++h) {
         const int cb = c_lo + 4 * h;
         if (cb < c_hi) {
             uint32_t r[4][8];
 #pragma unroll
             for (int u = 0; u < 4; ++u)
-                if (4 * h + u < kMaxChunks && cb + u < c_hi) tmem_ld_x8(s_addr + (cb + u) * 8, r[u]);
+                if (4 * h + u < kC && cb + u < c_hi) tmem_ld_x8(s_addr + (cb + u) * 8, r[u]);
             tmem_wait_ld();
 #pragma unroll
             for (int u = 0; u < 4; ++u)
-                if (4 * h + u < kMaxChunks && cb + u < c_hi)
-                    gmax = fmaxf(gmax, exp_chunk<kMask, kFp8>(r[u], m_s + (cb + u) * 8, scale, vis_s + (cb + u) * 8,
-                                                              (cb + u) * 8, G, t, pk[4 * h + u]));
+                if (4 * h + u < kC && cb + u < c_hi)
+                    gmax = fmaxf(gmax, exp_chunk<kMask>(r[u], m_s + (cb + u) * 8, scale, seen, (cb + u) * 8,
+                                                              pk[4 * h + u]));
         }
     }
     return gmax;
 }
-// kTree: the draft slots hold several branches (the visibility table is only built
-// and read then; the plain chain keeps its arithmetic mask).  kPaged: K and V are page
-// pools and a tile's position in them comes from the sequence's block table.
+
+// bf16 exponentials of eight columns of one position, two columns per instruction where the
+// machine has a packed form; pmax takes the largest probabilities (bf16 pairs) for the guard.
+// y = m - score * scale, so that the packed multiply-add needs no negated operand.
+template <bool kMask>
+__device__ __forceinline__ uint4 exp_chunk_bf16(const uint32_t *r, const float *m8, uint64_t neg_scale2,
+                                                Seen seen, int col0, uint32_t &pmax)
+{
+    const ulonglong2 ma = *reinterpret_cast<const ulonglong2 *>(m8);
+    const ulonglong2 mb = *reinterpret_cast<const ulonglong2 *>(m8 + 4);
+    const uint64_t mm[4] = {ma.x, ma.y, mb.x, mb.y};
+    uint32_t w[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        float y0, y1;
+        unpack_f32x2(fma_f32x2(pack_f32x2(r[2 * k], r[2 * k + 1]), neg_scale2, mm[k]), y0, y1);
+        if (kMask) {
+            y0 = seen(col0 + 2 * k) ? y0 : INFINITY;
+            y1 = seen(col0 + 2 * k + 1) ? y1 : INFINITY;
+        }
+        w[k] = pack_bf16x2(ex2(-y0), ex2(-y1));
+        pmax = max_bf16x2(pmax, w[k]);
+    }
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// A group's share of the columns of one tile, chunks [c_lo, c_hi): exponentials of this
+// thread's position (up to four TMEM loads in flight per wait), stored as they come to its
+// place in the P^T buffer.
+template <bool kMask, int kC>
+__device__ __forceinline__ void softmax_share_bf16(uint32_t s_addr, int c_lo, int c_hi, const float *m_s,
+                                                   uint64_t neg_scale2, Seen seen,
+                                                   uint8_t *prow, uint32_t &pmax)
+{
+    constexpr int kB = kC < 4 ? kC : 4;      // chunks in flight
+#pragma unroll
+    for (int h = 0; h < (kC + kB - 1) / kB; ++h) {
+        const int cb = c_lo + kB * h;
+        if (cb < c_hi) {
+            uint32_t r[kB][8];
+#pragma unroll
+            for (int u = 0; u < kB; ++u)
+                if (kB * h + u < kC && cb + u < c_hi) tmem_ld_x8(s_addr + (cb + u) * 8, r[u]);
+            tmem_wait_ld();
+#pragma unroll
+            for (int u = 0; u < kB; ++u)
+                if (kB * h + u < kC && cb + u < c_hi)
+                    *reinterpret_cast<uint4 *>(prow + (cb + u) * 2048) =
+                        exp_chunk_bf16<kMask>(r[u], m_s + (cb + u) * 8, neg_scale2, seen, (cb + u) * 8, pmax);
+        }
+    }
+}
 // kFp8: E4M3 cache (tmap_q is not used: q is split into its two E4M3 tiles by the CTA).
-// kTurns: the softmax groups take the tiles in turn; otherwise all groups work on every
-// tile, each on a share of its columns (shorter per tile, and so at the two ends of a
-// CTA's stream, but the per-tile overheads are paid by all twelve warps: the form for few
-// query rows, where the stream is bound by HBM either way).
-template <bool kTree, bool kPaged, bool kFp8, bool kTurns>
+// kTurns: the softmax groups take the tiles in turn (fp8 cache only); otherwise all groups
+// work on every tile, each on a share of its columns, at most kC chunks of eight.
+// Draft trees and page pools are run-time cases (a mask range per position, a look-up per
+// tile): as template cases they gave nothing.
+template <bool kFp8, bool kTurns, int kC>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUtensorMap tmap_k,
                const __grid_constant__ CUtensorMap tmap_v, const __grid_constant__ CUtensorMap tmap_q)
 {
+    static_assert(kFp8 || !kTurns, "a bf16 cache does not go through in turns");
     // bytes of one K or V tile: two 64-channel boxes at head_dim 128 (bf16), one box at
     // head_dim 64 and for an fp8 tile of 128 channels
     const uint32_t kSlot = (uint32_t)P.cfg.slot_bytes;
     const bool two_boxes = kSlot == kSlotBytes;
     const int D = P.a.D;
+    const bool paged = P.a.page_size > 0;
     extern __shared__ uint8_t smem_raw[];
     const AttnParams &p = P.a;
     const TcConfig cfg = P.cfg;
@@ -405,7 +459,6 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
     float *m_s = reinterpret_cast<float *>(gbase + sm.m);
     float *dl_s = reinterpret_cast<float *>(gbase + sm.dl);
     float *tmx_s = reinterpret_cast<float *>(gbase + sm.tmx);
-    int2 *vis_s = reinterpret_cast<int2 *>(gbase + sm.vis);
     volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(gbase + sm.misc);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(gbase + sm.misc + 4);
     // how often the reference exponents m[] have been set or moved; tiles handed to the P.V issuer
@@ -423,12 +476,13 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
     // S^T and P^T buffers: a parity wait tells a phase from its neighbours only, so whoever
     // waits for a phase must know the phase before it to be over.  Each of these
     // barriers belongs to the tiles of one softmax group, which sees its phases in order.
-    auto s_full = [&](int i) { return bar1 + 8 * (i % kSoftmaxGroups); };
-    auto s_free = [&](int i) { return bar1 + 8 * (kSoftmaxGroups + i % kSoftmaxGroups); };
-    auto p_full = [&](int i) { return bar1 + 8 * (2 * kSoftmaxGroups + i % kSoftmaxGroups); };
-    auto p_free = [&](int i) { return bar1 + 8 * (3 * kSoftmaxGroups + i % kSoftmaxGroups); };
-    auto hand_parity = [](int i) { return (uint32_t)(i / kSoftmaxGroups) & 1u; };
-    const uint32_t drain_bar = bar1 + 8 * (4 * kSoftmaxGroups);
+    constexpr int kRound = kTurns ? kSoftmaxGroups : kHand;
+    auto s_full = [&](int i) { return bar1 + 8 * (i % kRound); };
+    auto s_free = [&](int i) { return bar1 + 8 * (kHand + i % kRound); };
+    auto p_full = [&](int i) { return bar1 + 8 * (2 * kHand + i % kRound); };
+    auto p_free = [&](int i) { return bar1 + 8 * (3 * kHand + i % kRound); };
+    auto hand_parity = [](int i) { return (uint32_t)(i / kRound) & 1u; };
+    const uint32_t drain_bar = bar1 + 8 * (4 * kHand);
     const uint32_t done_bar = drain_bar + 8;
     const uint32_t q_full = drain_bar + 16;
     const uint32_t pv_done = drain_bar + 24;
@@ -442,7 +496,7 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
     auto tile_at = [&](int i, int &pos0, int &map_row) {
         pos0 = (t_begin + i) * kTilePos;
         map_row = b;
-        if (kPaged) {
+        if (paged) {
             // a page holds a whole number of tiles; an entry outside the pool reads as zeros
             pos0 -= (pos0 / p.page_size) * p.page_size;
             map_row = page_s[i];
@@ -477,14 +531,14 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
         {
             // one barrier per lane, all at once (an mbarrier.init costs about a hundred
             // cycles): barriers sit in the order k_full, k_empty, v_full, v_empty,
-            // s_full[3], s_free[3], p_full[3], p_free[3], drain, done, q_full, pv_done
+            // s_full[4], s_free[4], p_full[4], p_free[4], drain, done, q_full, pv_done
             const int n_kv = 2 * cfg.ks + 2 * cfg.vs;
-            constexpr int n_sp = 4 * kSoftmaxGroups;
+            constexpr int n_sp = 4 * kHand;
             const int n_bars = n_kv + n_sp + 4;
             for (int i = lane; i < n_bars; i += 32) {
                 const int j = i - n_kv;          // index among the barriers after the rings
                 uint32_t count = 1;
-                if (j >= kSoftmaxGroups && j < 3 * kSoftmaxGroups) count = kTurns ? 4 : kSoftmaxWarps;   // s_free, p_full: the warps that work on a tile
+                if (j >= kHand && j < 3 * kHand) count = kTurns ? 4 : kSoftmaxWarps;   // s_free, p_full: the warps that work on a tile
                 else if (j == n_sp + 1) count = kSoftmaxWarps + 1;              // done
                 else if (kFp8 && j == n_sp + 2) count = kSoftmaxWarps;          // q_full: the warps that split q
                 mbar_init(bar0 + 8 * i, count);
@@ -498,7 +552,7 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
             fence_proxy_async_smem();
         }
         __syncwarp();
-        if (kPaged) {
+        if (paged) {
             // the block table too may come from the kernel before this one: the warp reads
             // this split's entries (one per tile) after the wait, then lane 0 goes on
             grid_dependency_wait();
@@ -537,17 +591,13 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
             *reinterpret_cast<uint4 *>(gbase + sm.q + h * (NP * 128) + r * 128 + cc * 16) =
                 make_uint4(0, 0, 0, 0);
         }
-        // P buffers start as zeros (columns beyond the last chunk stay zero)
-        for (uint32_t i = idx * 16; i < (uint32_t)(cfg.pb * NP * 256); i += kSoftmaxThreads * 16)
-            *reinterpret_cast<uint4 *>(gbase + sm.p + i) = make_uint4(0, 0, 0, 0);
+        // columns beyond the last chunk (at most one chunk, 2 KB, per P buffer) stay zero
+        if (n8 * 8 < NP)
+            for (int i = idx; i < cfg.pb * 128; i += kSoftmaxThreads)
+                *reinterpret_cast<uint4 *>(gbase + sm.p + (i >> 7) * (NP * 256) + n8 * 2048 + (i & 127) * 16) =
+                    make_uint4(0, 0, 0, 0);
         for (int n = idx; n < NP; n += kSoftmaxThreads) {
             m_s[n] = kFp8 ? kMFloor : 0.f;
-            if (kTree) {
-                // the draft slots column n's query sees: its branch's first slot .. its own slot
-                const int qi = n / G;
-                vis_s[n] = qi < gamma ? make_int2((qi / p.branch_len) * p.branch_len, qi)
-                                      : make_int2(1 << 30, (1 << 30) - 1);
-            }
         }
         // constant 64 x 16 tiles (K-major, no swizzle: the 8 positions of chunk c
         // at c * 1024, row r at (r / 8) * 128 + (r % 8) * 16).  Row 0 = ones (sums
@@ -722,7 +772,7 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
             for (int j = 0; j < 8; ++j)
                 qd[j] = make_smem_desc(base + sm.q + (j >> 2) * (NP * 128) + (j & 3) * 32, 16, 1024,
                                        kSwizzle128B);
-            Ring k_ring(cfg.ks), s_ring(cfg.sb), hand(kSoftmaxGroups), freed(kSoftmaxGroups);
+            Ring k_ring(cfg.ks), s_ring(cfg.sb), hand(kRound), freed(kRound);
             auto issue_qk = [&](int i) -> bool {
                 const int ks = k_ring.idx, sb = s_ring.idx;
                 LVSPEC_TILE_TS(tile_tr, 1, i, 0);     // starts waiting for the K tile
@@ -730,7 +780,7 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                 LVSPEC_TILE_TS(tile_tr, 1, i, 1);     // K tile there
                 // the tile that used this S^T buffer last (tile i - sb) has been read
                 if (i >= cfg.sb) {
-                    there = mbar_wait(bar1 + 8 * (kSoftmaxGroups + freed.idx), freed.parity, abort_flag) && there;
+                    there = mbar_wait(bar1 + 8 * (kHand + freed.idx), freed.parity, abort_flag) && there;
                     freed.next();
                 }
                 if (!__all_sync(0xffffffffu, there)) return false;
@@ -780,11 +830,14 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
             const uint64_t vd0 = make_smem_desc(base + sm.v, kBoxBytes, 1024, kSwizzle128B);
             const uint64_t pd0 = make_smem_desc(base + sm.p, 128, 2048, kSwizzleNone);
             const uint64_t a2d0 = make_smem_desc(base + sm.a2, 1024, 128, kSwizzleNone);
-            Ring v_ring(cfg.vs), p_ring(cfg.pb), hand(kSoftmaxGroups);
+            Ring v_ring(cfg.vs), p_ring(cfg.pb), hand(kRound);
             for (int i = 0; i < T; ++i, v_ring.next(), p_ring.next(), hand.next()) {
                 const int pb = p_ring.idx, vsl = v_ring.idx;
                 LVSPEC_TILE_TS(tile_tr, 2, i, 0);     // starts waiting for P^T
-                bool there = mbar_wait(bar1 + 8 * (2 * kSoftmaxGroups + hand.idx), hand.parity, abort_flag);   // p_full of tile i
+                // p_full of tile i (two tiles handed over together: on the first one's barrier)
+                bool there = true;
+                if (kTurns || cfg.step == 1 || !(i & 1))
+                    there = mbar_wait(bar1 + 8 * (2 * kHand + hand.idx), hand.parity, abort_flag);
                 LVSPEC_TILE_TS(tile_tr, 2, i, 1);     // P^T there
                 there = mbar_wait(v_full(vsl), v_ring.parity, abort_flag) && there;
                 if (!__all_sync(0xffffffffu, there)) break;
@@ -833,7 +886,7 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                 }
                 if (elect_one()) {
                     mma_commit(v_empty(vsl));
-                    mma_commit(bar1 + 8 * (3 * kSoftmaxGroups + hand.idx));     // p_free of tile i
+                    mma_commit(bar1 + 8 * (3 * kHand + hand.idx));     // p_free of tile i
                 }
                 __syncwarp();
                 LVSPEC_TILE_TS(tile_tr, 2, i, 3);     // sums and P.V issued
@@ -896,43 +949,13 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                 // when their turn comes.
                 bool my_turn = i == 0;
                 uint32_t e0 = 0;
-                if (i == 0) {
-                    if (!kFp8) {
-                        // reference exponent of each row: its score at the split's first position
-                        // (every warp reads the chunks c8 = its quarter, quarter + 4, ... from the TMEM
-                        // lanes it can reach; only the first quarter holds position 0)
-                        if (wq == 0) {
-#pragma unroll 1
-                            for (int cb = 0; cb < n8; cb += 2) {
-                                uint32_t r[2][8];
-#pragma unroll
-                                for (int u = 0; u < 2; ++u)
-                                    if (cb + u < n8) tmem_ld_x8(s_addr + (cb + u) * 8, r[u]);
-                                tmem_wait_ld();
-                                if (lane == 0) {
-#pragma unroll
-                                    for (int u = 0; u < 2; ++u)
-                                        if (cb + u < n8) {
-#pragma unroll
-                                            for (int k = 0; k < 8; ++k)
-                                                m_s[(cb + u) * 8 + k] = __uint_as_float(r[u][k]) * scale - kLift;
-                                        }
-                                }
-                            }
-                        }
-                        group_sync(bar_id);
-                        if (gtid == 0) {
-                            __threadfence_block();
-                            *epoch_s = 1;
-                        }
-                    }
-                } else {
+                if (i > 0) {
                     if (i < kSoftmaxGroups) wait_counter(epoch_s, 1);     // m comes from the first tile
                     e0 = *epoch_s;
                     __threadfence_block();
                 }
                 const bool tail = pos0 + kTilePos > L - gamma;
-                const int gmin = pos - L + gamma;           // tail index of `pos`: queries below it do not see it
+                const Seen seen = seen_by(tail ? pos - L + gamma : -1, G, gamma, p.branch_len);
                 // P^T goes straight to shared memory: the P.V product that read this buffer last is done
                 // (tile i - pb; this group saw tile i - 3 - pb's product done a turn ago)
                 if (i >= cfg.pb) mbar_wait(p_free(i - cfg.pb), hand_parity(i - cfg.pb), abort_flag);
@@ -946,9 +969,9 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                 for (int attempt = 0; attempt < 4; ++attempt) {
                     float gmax = -INFINITY;
                     if (!take_max)
-                        gmax = !tail ? softmax_pass<0, kFp8>(s_addr, n8, m_s, scale, vis_s, G, gmin, prow,
+                        gmax = !tail ? softmax_pass<false>(s_addr, n8, m_s, scale, seen, prow,
                                                              warp == kSoftmaxWarp0 ? tile_tr : nullptr, i)
-                                     : softmax_pass<kTree ? 2 : 1, kFp8>(s_addr, n8, m_s, scale, vis_s, G, gmin, prow, nullptr, i);
+                                     : softmax_pass<true>(s_addr, n8, m_s, scale, seen, prow, nullptr, i);
                     if (warp == kSoftmaxWarp0) LVSPEC_TILE_TS(tile_tr, 0, i, 3);     // exponentials done
                     if (!my_turn) {
                         wait_counter(committed_s, (uint32_t)i);
@@ -978,7 +1001,7 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                             for (int k = 0; k < 8; ++k) {
                                 s2[k] = __uint_as_float(r[k]) * scale;
                                 if constexpr (decltype(masked)::value) {
-                                    if (kTree ? !column_sees(vis_s[c8 * 8 + k], gmin) : (c8 * 8 + k) / G < gmin)
+                                    if (!seen(c8 * 8 + k))
                                         s2[k] = -INFINITY;
                                 }
                             }
@@ -1072,63 +1095,98 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                 advance(pb, cfg.pb);
             }
         } else {
-            // ring positions advance by counting, not by dividing
-            int pb = 0, vsl = 0;                 // P buffer and V slot of tile i
-            uint32_t pb_round = 0, vs_round = 0; // how often each ring has wrapped
-            for (int i = 0; i < T; ++i) {
-                const int pos0 = (t_begin + i) * kTilePos;
-                const int pos = pos0 + row;
-                const int sb = i & 1;
-                if (warp == kSoftmaxWarp0) LVSPEC_TILE_TS(tile_tr, 0, i, 0);     // starts waiting for S^T
-                mbar_wait(s_full(i), hand_parity(i), abort_flag);
-                if (warp == kSoftmaxWarp0) LVSPEC_TILE_TS(tile_tr, 0, i, 1);     // S^T there
-                tc_fence_after();
-                const uint32_t s_addr = tm_s0 + sb * NP + lane_addr;
-                if (!kFp8 && i == 0) {
-                    // reference exponent of each row: its score at the split's first position
-                    if (wq == 0) {
-                        for (int c8 = c_lo; c8 < c_hi; ++c8) {
-                            uint32_t r[8];
-                            tmem_ld_x8(s_addr + c8 * 8, r);
-                            tmem_wait_ld();
-                            if (lane == 0) {
-#pragma unroll
-                                for (int k = 0; k < 8; ++k) m_s[c8 * 8 + k] = __uint_as_float(r[k]) * scale - kLift;
-                            }
-                        }
-                    }
-                    group_sync(bar_id);
-                }
-                const bool tail = pos0 + kTilePos > L - gamma;
-                const int gmin = pos - L + gamma;           // tail index of `pos`: queries below it do not see it
-                uint8_t *prow = gbase + sm.p + pb * (NP * 256) + row * 16;
-                uint4 pk[kMaxChunks];   // this position's probabilities, 8 columns per entry
-
+            // Tiles go through in twos where the buffers allow (256 positions): one vote on the
+            // guard, one fence and one hand-over for both.
+            // Ring positions advance by counting, not by dividing.
+            int sbi = 0, pb = 0, vsl = 0;        // S^T buffer, P buffer and V slot of tile i
+            uint32_t vs_round = 0;               // how often the V ring has wrapped
+            const uint64_t neg_scale2 = pack_f32x2(__float_as_uint(-scale), __float_as_uint(-scale));
+            for (int i = 0; i < T; i += cfg.step) {
+                const int n_sub = min(cfg.step, T - i);
                 for (int attempt = 0; attempt < 3; ++attempt) {
                     // fp8 cache: E4M3 has 17 binades, so the reference exponent of a row starts
                     // from the largest score of the split's first tile (the path below), not
                     // from whatever score its first position happens to have
                     const bool first_max = kFp8 && i == 0 && attempt == 0;
-                    if (!first_max) {
-                        const float gmax =
-                            !tail ? softmax_pass_share<0, kFp8>(s_addr, c_lo, c_hi, m_s, scale, vis_s, G, gmin, pk)
-                                  : softmax_pass_share<kTree ? 2 : 1, kFp8>(s_addr, c_lo, c_hi, m_s, scale, vis_s, G, gmin, pk);
-                        if (warp == kSoftmaxWarp0) LVSPEC_TILE_TS(tile_tr, 0, i, 2);     // exponentials done
-                        if (!group_any(bar_id, gmax > kLimit)) break;
-                    }
-
-                    // ---- a score ran past the guard: move m up to the tile maximum ----
-                    for (int c8 = c_lo; c8 < c_hi; ++c8) {
-                        uint32_t r[8];
-                        tmem_ld_x8(s_addr + c8 * 8, r);
-                        tmem_wait_ld();
+                    float gmax = -INFINITY;
+                    uint32_t pmax = 0u;
+                    int sb_u = sbi, pb_u = pb;
+#pragma unroll 1
+                    for (int u = 0; u < n_sub; ++u) {
+                        const int iu = i + u;
+                        const int pos0 = (t_begin + iu) * kTilePos;
+                        if (attempt == 0 || iu == 1) {
+                            if (warp == kSoftmaxWarp0) LVSPEC_TILE_TS(tile_tr, 0, iu, 0);     // starts waiting for S^T
+                            mbar_wait(s_full(iu), hand_parity(iu), abort_flag);
+                            if (warp == kSoftmaxWarp0) LVSPEC_TILE_TS(tile_tr, 0, iu, 1);     // S^T there
+                            tc_fence_after();
+                        }
+                        const uint32_t s_addr = tm_s0 + sb_u * NP + lane_addr;
+                        if (!kFp8 && iu == 0 && attempt == 0) {
+                            // reference exponent of each row: its score at the split's first position
+                            if (wq == 0) {
+                                for (int c8 = c_lo; c8 < c_hi; ++c8) {
+                                    uint32_t r[8];
+                                    tmem_ld_x8(s_addr + c8 * 8, r);
+                                    tmem_wait_ld();
+                                    if (lane == 0) {
 #pragma unroll
-                        for (int k = 0; k < 8; ++k) {
-                            float s2 = __uint_as_float(r[k]) * scale;
-                            if (tail && (kTree ? !column_sees(vis_s[c8 * 8 + k], gmin) : (c8 * 8 + k) / G < gmin))
-                                s2 = -INFINITY;
-                            s2 = warp_max_f32(s2);
-                            if (lane == 0) tmx_s[wq * NP + c8 * 8 + k] = s2;
+                                        for (int k = 0; k < 8; ++k) m_s[c8 * 8 + k] = __uint_as_float(r[k]) * scale - kLift;
+                                    }
+                                }
+                            }
+                            group_sync(bar_id);
+                        }
+                        if (first_max) break;
+                        const bool tail = pos0 + kTilePos > L - gamma;
+                        const Seen seen = seen_by(tail ? pos0 + row - L + gamma : -1, G, gamma, p.branch_len);
+                        uint8_t *prow = gbase + sm.p + pb_u * (NP * 256) + row * 16;
+                        // P^T goes straight to shared memory, once the P.V product that read this buffer is done
+                        if (attempt == 0 && iu >= cfg.pb) mbar_wait(p_free(iu - cfg.pb), hand_parity(iu - cfg.pb), abort_flag);
+                        if (warp == kSoftmaxWarp0) LVSPEC_TILE_TS(tile_tr, 0, iu, 2);     // P buffer free
+                        if constexpr (kFp8) {
+                            uint4 pk[kC];   // this position's probabilities, 8 columns per entry
+                            gmax = fmaxf(gmax,
+                                !tail ? softmax_pass_share<false, kC>(s_addr, c_lo, c_hi, m_s, scale, seen, pk)
+                                      : softmax_pass_share<true, kC>(s_addr, c_lo, c_hi, m_s, scale, seen, pk));
+#pragma unroll
+                            for (int j = 0; j < kC; ++j)
+                                if (c_lo + j < c_hi) *reinterpret_cast<uint4 *>(prow + (c_lo + j) * 2048) = pk[j];
+                        } else if (!tail) {
+                            softmax_share_bf16<false, kC>(s_addr, c_lo, c_hi, m_s, neg_scale2, seen, prow, pmax);
+                        } else {
+                            softmax_share_bf16<true, kC>(s_addr, c_lo, c_hi, m_s, neg_scale2, seen, prow, pmax);
+                        }
+                        if (warp == kSoftmaxWarp0) LVSPEC_TILE_TS(tile_tr, 0, iu, 3);     // probabilities stored
+                        if (++sb_u == cfg.sb) sb_u = 0;
+                        if (++pb_u == cfg.pb) pb_u = 0;
+                    }
+                    const bool beyond = kFp8 ? gmax > kLimit : (pmax & 0xFFFFu) > kGuardBits || (pmax >> 16) > kGuardBits;
+                    if (!first_max && !group_any(bar_id, beyond)) break;
+
+                    // ---- a score ran past the guard: move m up to these tiles' maximum (fp8: first
+                    // to the first tile's) ----
+                    for (int u = 0; u < (first_max ? 1 : n_sub); ++u) {
+                        const int pos0 = (t_begin + i + u) * kTilePos;
+                        const bool tail = pos0 + kTilePos > L - gamma;
+                        const Seen seen = seen_by(tail ? pos0 + row - L + gamma : -1, G, gamma, p.branch_len);
+                        const int sbu = sbi + u < cfg.sb ? sbi + u : sbi + u - cfg.sb;
+                        const uint32_t s_addr = tm_s0 + sbu * NP + lane_addr;
+                        for (int c8 = c_lo; c8 < c_hi; ++c8) {
+                            uint32_t r[8];
+                            tmem_ld_x8(s_addr + c8 * 8, r);
+                            tmem_wait_ld();
+#pragma unroll
+                            for (int k = 0; k < 8; ++k) {
+                                float s2 = __uint_as_float(r[k]) * scale;
+                                if (tail && !seen(c8 * 8 + k))
+                                    s2 = -INFINITY;
+                                s2 = warp_max_f32(s2);
+                                if (lane == 0) {
+                                    float *dst = tmx_s + wq * NP + c8 * 8 + k;
+                                    *dst = u == 0 ? s2 : fmaxf(*dst, s2);
+                                }
+                            }
                         }
                     }
                     group_sync(bar_id);
@@ -1169,12 +1227,20 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                     }
                     group_sync(bar_id);
                 }
-                if (tail && grp == 0) {
+                if (warp == kSoftmaxWarp0) LVSPEC_TILE_TS(tile_tr, 0, i, 4);     // the group agrees: no rescale
+                if (grp == 0 && (t_begin + i + n_sub) * kTilePos > L) {
                     // slots at or beyond kv_len hold whatever the cache holds: zero their V
-                    // rows so that 0 * junk cannot poison the accumulators
-                    mbar_wait(v_full(vsl), vs_round & 1, abort_flag);
-                    if (pos >= L) {
-                        uint8_t *vrow = gbase + sm.v + vsl * kSlot + row * 128;
+                    // rows so that 0 * junk cannot poison the accumulators (they sit in the last tile)
+                    int vz = vsl;
+                    uint32_t vr = vs_round;
+                    if (n_sub == 2 && ++vz == cfg.vs) { vz = 0; ++vr; }
+                    // the slot's tile before is done with (a parity tells this phase from its
+                    // neighbours only, and the products may lag by the depth of the P^T ring)
+                    const int before = i + n_sub - 1 - cfg.vs;
+                    if (before >= 0) mbar_wait(p_free(before), hand_parity(before), abort_flag);
+                    mbar_wait(v_full(vz), vr & 1, abort_flag);
+                    if ((t_begin + i + n_sub - 1) * kTilePos + row >= L) {
+                        uint8_t *vrow = gbase + sm.v + vz * kSlot + row * 128;
 #pragma unroll
                         for (int c = 0; c < 8; ++c) {
                             *reinterpret_cast<uint4 *>(vrow + c * 16) = make_uint4(0, 0, 0, 0);
@@ -1182,25 +1248,22 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                         }
                     }
                 }
-                if (warp == kSoftmaxWarp0) LVSPEC_TILE_TS(tile_tr, 0, i, 3);     // the group agrees: no rescale
-                // P^T goes to shared memory once the P.V product that read this buffer is done
-                if (i >= cfg.pb) mbar_wait(p_free(i - cfg.pb), hand_parity(i - cfg.pb), abort_flag);
-                if (warp == kSoftmaxWarp0) LVSPEC_TILE_TS(tile_tr, 0, i, 4);     // P buffer free
-#pragma unroll
-                for (int j = 0; j < kMaxChunks; ++j)
-                    if (c_lo + j < c_hi) *reinterpret_cast<uint4 *>(prow + (c_lo + j) * 2048) = pk[j];
-                // one arrival per warp: S^T has been read (the next K.Q^T but one may overwrite
-                // it) and P^T, with any zeroed V rows, is in shared memory
+                // one arrival per warp: S^T has been read (later K.Q^T may overwrite it) and P^T,
+                // with any zeroed V rows, is in shared memory
                 tc_fence_before();
                 fence_proxy_async_smem();
                 __syncwarp();
                 if (lane == 0) {
-                    mbar_arrive(s_free(i));
                     mbar_arrive(p_full(i));
+                    mbar_arrive(s_free(i));
+                    if (n_sub == 2) mbar_arrive(s_free(i + 1));
                 }
                 if (warp == kSoftmaxWarp0) LVSPEC_TILE_TS(tile_tr, 0, i, 5);     // P^T stored and handed over
-                if (++pb == cfg.pb) { pb = 0; ++pb_round; }
-                if (++vsl == cfg.vs) { vsl = 0; ++vs_round; }
+                for (int u = 0; u < n_sub; ++u) {
+                    if (++sbi == cfg.sb) sbi = 0;
+                    if (++pb == cfg.pb) pb = 0;
+                    if (++vsl == cfg.vs) { vsl = 0; ++vs_round; }
+                }
             }
         }
 
@@ -1380,28 +1443,29 @@ TcConfig pick_config(int M, int page_slots, bool fp8, bool turns, int D)
     c.slot_bytes = small_tiles ? kBoxBytes : kSlotBytes;
     const int acc = fp8 ? 4 : 2;     // TMEM columns per padded row of O^T and the sums
     if (!turns) {
-        // All groups on every tile: S^T twice.  Six ring slots when they fit, also at the
-        // price of the second P buffer (with 40 rows the stream is bound by HBM: bytes in
-        // flight count, and the probabilities wait in registers for the buffer anyway).
-        c.sb = 2;
-        const int tries[6][3] = {{3, 3, 2}, {3, 3, 1}, {2, 3, 2}, {2, 2, 2}, {2, 3, 1}, {2, 2, 1}};
-        const int tries8[6][3] = {{5, 6, 2}, {5, 5, 2}, {4, 5, 2}, {4, 4, 2}, {4, 4, 1}, {3, 3, 1}};
-        for (int t = 0; t < 6; ++t) {
+        // All groups on every tile: as many S^T and P^T buffers as fit, up to two pairs, before
+        // more than two ring slots each.  64 KB of K/V in flight per CTA and die-wide 16 MB
+        // are enough for HBM, and more of them at the start of a launch only put later tiles
+        // ahead of the first one's (40 rows, 16 tiles per CTA: 26.9 us with 2 + 2 slots,
+        // 27.9 with 3 + 2 or 2 + 3).
+        c.sb = 512 / c.n_pad - acc;
+        if (c.sb > 4) c.sb = 4;
+        const int tries[5][3] = {{2, 2, 4}, {2, 2, 3}, {2, 2, 2}, {2, 3, 1}, {2, 2, 1}};
+        const int tries8[5][3] = {{4, 4, 4}, {4, 4, 3}, {4, 4, 2}, {4, 4, 1}, {3, 3, 1}};
+        for (int t = 0; t < 5; ++t) {
             const int *tr = small_tiles ? tries8[t] : tries[t];
             c.ks = tr[0]; c.vs = tr[1]; c.pb = tr[2];
             if (smem_map(c).total <= kMaxSmem) break;
         }
     } else {
-        // Tiles in turn: an S^T buffer per softmax group when TMEM has the columns, else
-        // two.  Shared memory: a P^T buffer per group before more ring slots (a group that
-        // shares its buffer waits for the product of an earlier tile before it can store
-        // anything); of the rings, V slots are held longer than K slots.  An fp8 tile is
-        // half the bytes: twice the slots for the same bytes in flight.
+        // Tiles in turn (fp8 cache): an S^T buffer per softmax group when TMEM has the columns,
+        // else two.  Three 16 KB slots each: a tile is half a bf16 tile's bytes, yet more
+        // slots delay the first tiles (40 rows, 64 layers of 32K: 25.4 us a layer with 5 + 5,
+        // 24.4 with 4 + 4, 23.9 with 3 + 3, 24.7 with 2 + 3).
         c.sb = (kSoftmaxGroups + acc) * c.n_pad <= 512 ? kSoftmaxGroups : 2;
-        const int tries[8][3] = {{3, 3, 3}, {2, 3, 3}, {3, 2, 3}, {2, 2, 3}, {2, 2, 2}, {2, 2, 1}, {1, 2, 1}, {1, 1, 1}};
-        const int tries8[8][3] = {{5, 6, 3}, {5, 5, 3}, {4, 5, 3}, {4, 4, 3}, {4, 4, 2}, {3, 3, 2}, {3, 3, 1}, {2, 2, 1}};
-        for (int t = 0; t < 8; ++t) {
-            const int *tr = small_tiles ? tries8[t] : tries[t];
+        const int tries[4][3] = {{3, 3, 3}, {3, 3, 2}, {3, 3, 1}, {2, 2, 1}};
+        for (int t = 0; t < 4; ++t) {
+            const int *tr = tries[t];
             c.ks = tr[0]; c.vs = tr[1]; c.pb = tr[2];
             if (smem_map(c).total <= kMaxSmem) break;
         }
@@ -1411,10 +1475,14 @@ TcConfig pick_config(int M, int page_slots, bool fp8, bool turns, int D)
     if (const char *e = std::getenv("LVSPEC_TC_RING")) {
         int ks, vs, pb, sb;
         if (std::sscanf(e, "%d,%d,%d,%d", &ks, &vs, &pb, &sb) == 4 && ks >= 1 && ks <= 8 && vs >= 1 && vs <= 8 &&
-            pb >= 1 && pb <= kSoftmaxGroups && sb >= 2 && sb <= kSoftmaxGroups && (turns || (sb == 2 && pb <= 2))) {
+            pb >= 1 && sb >= 2 && pb <= (turns ? kSoftmaxGroups : kHand) && sb <= (turns ? kSoftmaxGroups : kHand)) {
             c.ks = ks; c.vs = vs; c.pb = pb; c.sb = sb;
         }
     }
+    // Two tiles per hand-over need S^T and P^T buffers for the tiles after them too (with two
+    // S^T buffers the K.Q^T of the next pair waits for this one: 112 padded rows, 128-frame
+    // tree, 36.8 us a layer in pairs against 34.9 one by one), and a V ring that holds a pair.
+    c.step = !turns && c.sb >= 4 && c.pb >= 2 && c.vs >= 2 ? 2 : 1;
     int cols = 32;
     while (cols < (c.sb + acc) * c.n_pad) cols <<= 1;
     c.tmem_cols = cols;
@@ -1437,14 +1505,14 @@ cudaError_t launch_attn_tc(const AttnParams &p, const SeqInfo &seq, cudaStream_t
     // paged: one block-table entry per tile of the longest split, rounded up to 4
     const int tiles = (p.Lmax + kTilePos - 1) / kTilePos;
     const bool fp8 = p.fp8 != 0;
-    // Tiles in turn where a CTA streams long enough for the throughput of the softmax stage
-    // to outweigh its latency at the two ends of the stream (measured on the 40/8-head sweep:
-    // 5 to 10 % faster from about a hundred tiles per CTA, slower below 32), and with an fp8
-    // cache of up to 64 padded rows (half the bytes per tile for the same work; with more
-    // rows TMEM holds only two S^T buffers and the shared columns win).
-    // LVSPEC_TC_TURNS=0/1 overrides the choice (for measurements).
-    bool turns = (tiles + p.n_split - 1) / p.n_split >= 96 || (fp8 && p.M <= 64);
-    if (const char *e = std::getenv("LVSPEC_TC_TURNS"))
+    // Tiles in turn with an fp8 cache of up to 64 padded rows (half the bytes per tile for the
+    // same work: 24.2 us a layer at 40 rows of 32K against 29.0 with shared columns; with more
+    // rows TMEM holds only two S^T buffers and the shared columns win until the stream is
+    // long).  A bf16 cache goes through in pairs of tiles with shared columns, which beats
+    // turns at every length (long streams of 80 rows: 321 us against 331).
+    // LVSPEC_TC_TURNS=0/1 overrides the choice with an fp8 cache (for measurements).
+    bool turns = fp8 && (p.M <= 64 || (tiles + p.n_split - 1) / p.n_split >= 96);
+    if (const char *e = fp8 ? std::getenv("LVSPEC_TC_TURNS") : nullptr)
         if (e[0] == '0' || e[0] == '1') turns = e[0] == '1';
     P.cfg = pick_config(p.M, paged ? ((tiles + p.n_split - 1) / p.n_split + 4) & ~3 : 0, fp8, turns, p.D);
     if (smem_map(P.cfg).total > kMaxSmem || P.cfg.tmem_cols > 512) return cudaErrorInvalidConfiguration;
@@ -1459,13 +1527,10 @@ cudaError_t launch_attn_tc(const AttnParams &p, const SeqInfo &seq, cudaStream_t
     const size_t smem = smem_map(P.cfg).total + 1024;
     const bool tree = p.branch_len != p.gamma;
     if ((tree && paged) || (fp8 && (tree || paged))) return cudaErrorNotSupported;
-    auto kernel = fp8 ? (turns ? attn_tc_kernel<false, false, true, true> : attn_tc_kernel<false, false, true, false>)
-                  : turns ? (paged ? attn_tc_kernel<false, true, false, true>
-                                   : (tree ? attn_tc_kernel<true, false, false, true>
-                                           : attn_tc_kernel<false, false, false, true>))
-                          : (paged ? attn_tc_kernel<false, true, false, false>
-                                   : (tree ? attn_tc_kernel<true, false, false, false>
-                                           : attn_tc_kernel<false, false, false, false>));
+    const int share = ((p.M + 7) / 8 + kSoftmaxGroups - 1) / kSoftmaxGroups;    // column chunks of a softmax group
+    auto kernel = fp8 ? (turns ? attn_tc_kernel<true, true, 1> : attn_tc_kernel<true, false, 4>)
+                  : share <= 2 ? attn_tc_kernel<false, false, 2>
+                  : share <= 4 ? attn_tc_kernel<false, false, 4> : attn_tc_kernel<false, false, kMaxChunks>;
     cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
     cudaLaunchConfig_t cfg = {};
