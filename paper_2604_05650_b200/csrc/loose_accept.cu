@@ -8,11 +8,13 @@
 // partitioning.  The last CTA to finish for a sequence (an atomic ticket; no
 // CTA ever waits on another) merges the slices and evaluates the rule.
 #include "lvspec_internal.h"
+#include "sm100_ptx.cuh"
 
 namespace lvspec {
 namespace {
 
 constexpr int kThreads = 256;
+constexpr int kInFlight = 4;             // 16-byte loads a thread keeps in flight
 constexpr int kNoIndex = 0x7fffffff;
 
 struct Best {
@@ -49,6 +51,9 @@ __global__ void __launch_bounds__(kThreads) loose_accept_kernel(const AcceptPara
     const int per = (((V + p.n_vsplit - 1) / p.n_vsplit) + 3) & ~3;
     const int c0 = min(V, slice * per), c1 = min(V, c0 + per);
 
+    // the logits, masses and lengths may come from the kernel before this one
+    ptx::grid_launch_dependents();
+    ptx::grid_dependency_wait();
     Best best = {-INFINITY, kNoIndex};
     bool nan_seen = false;
     // elements up to the first 16-byte boundary, vector body, tail
@@ -59,13 +64,22 @@ __global__ void __launch_bounds__(kThreads) loose_accept_kernel(const AcceptPara
     const int body0 = c0 + head;
     const int n_vec = (c1 - body0) >> 2;
     const float4 *vec = reinterpret_cast<const float4 *>(row + body0);
-    for (int j = tid; j < n_vec; j += kThreads) {
-        const float4 x = __ldg(vec + j);
-        const int idx = body0 + 4 * j;
-        take(best, x.x, idx, nan_seen);
-        take(best, x.y, idx + 1, nan_seen);
-        take(best, x.z, idx + 2, nan_seen);
-        take(best, x.w, idx + 3, nan_seen);
+    // four loads in flight per thread: with eight rows of 152 K a thread has four or five
+    // in all, which then cost one trip to memory instead of one each
+    for (int j0 = tid; j0 < n_vec; j0 += kInFlight * kThreads) {
+        float4 x[kInFlight];
+#pragma unroll
+        for (int u = 0; u < kInFlight; ++u)
+            x[u] = j0 + u * kThreads < n_vec ? __ldg(vec + j0 + u * kThreads)
+                                             : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+#pragma unroll
+        for (int u = 0; u < kInFlight; ++u) {
+            const int idx = body0 + 4 * (j0 + u * kThreads);
+            take(best, x[u].x, idx, nan_seen);
+            take(best, x[u].y, idx + 1, nan_seen);
+            take(best, x[u].z, idx + 2, nan_seen);
+            take(best, x[u].w, idx + 3, nan_seen);
+        }
     }
     const int tail0 = body0 + 4 * n_vec;
     if (tail0 + tid < c1) take(best, row[tail0 + tid], tail0 + tid, nan_seen);
@@ -131,6 +145,7 @@ __global__ void __launch_bounds__(kThreads) loose_accept_kernel(const AcceptPara
         for (int h0 = 0; h0 < p.Hm; h0 += 32) {
             const float mine = h0 + lane < p.Hm ? mrow[h0 + lane] : 0.f;
             const int n = min(32, p.Hm - h0);
+#pragma unroll 8
             for (int h = 0; h < n; ++h) sc += (double)__shfl_sync(0xffffffffu, mine, h);
         }
         if (lane == 0) {
@@ -188,6 +203,8 @@ __global__ void __launch_bounds__(kThreads) loose_accept_kernel(const AcceptPara
 __global__ void select_branch_kernel(const int32_t *accept_len, int B, int R, int32_t *best_branch,
                                      int32_t *best_len)
 {
+    ptx::grid_launch_dependents();
+    ptx::grid_dependency_wait();
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= B) return;
     int best = 0, len = accept_len[(size_t)b * R];
@@ -202,19 +219,16 @@ __global__ void select_branch_kernel(const int32_t *accept_len, int B, int R, in
 }  // namespace
 
 cudaError_t launch_select_branch(const int32_t *accept_len, int B, int R, int32_t *best_branch,
-                                 int32_t *best_len, cudaStream_t stream, int *launches)
+                                 int32_t *best_len, bool pdl, cudaStream_t stream, int *launches)
 {
-    select_branch_kernel<<<(B + 127) / 128, 128, 0, stream>>>(accept_len, B, R, best_branch, best_len);
-    ++*launches;
-    return cudaGetLastError();
+    return launch_after(select_branch_kernel, dim3((B + 127) / 128), 128, 0, pdl, stream, launches, accept_len, B, R,
+                        best_branch, best_len);
 }
 
 cudaError_t launch_loose_accept(const AcceptParams &p, cudaStream_t stream, int *launches)
 {
     dim3 grid(p.n_vsplit, p.gamma, p.B);
-    loose_accept_kernel<<<grid, kThreads, 0, stream>>>(p);
-    ++*launches;
-    return cudaGetLastError();
+    return launch_after(loose_accept_kernel, grid, kThreads, 0, p.pdl != 0, stream, launches, p);
 }
 
 }  // namespace lvspec

@@ -377,6 +377,7 @@ lvspec_status_t run_accept(lvspec_ctx *ctx, int batch, int gamma, int vocab, int
     p.Hm = heads;
     p.n_loose = n_loose;
     p.window = window > gamma ? gamma : window;
+    p.pdl = ctx->pdl ? 1 : 0;
     const int rows = batch * gamma;
     const int vs = accept_vocab_slices(ctx, rows, vocab);
     p.n_vsplit = vs;
@@ -719,6 +720,7 @@ lvspec_status_t lvspec_verify_attention_spans(lvspec_ctx_t *ctx, const lvspec_at
         g.M = g.gamma * g.G;
         g.scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)g.D));
         g.n_gaps = (int)gaps[b].size() / 2;
+        g.pdl = ctx->pdl ? 1 : 0;
         int flat = 0;
         for (int i = 0; i < g.n_gaps; ++i) {
             g.gap_start[i] = gaps[b][2 * i];
@@ -843,7 +845,7 @@ lvspec_status_t lvspec_select_branch(lvspec_ctx_t *ctx, int32_t batch, int32_t n
     cudaError_t e = cudaSetDevice(ctx->device);
     if (e != cudaSuccess) return cuda_fail(ctx, "cudaSetDevice", e);
     int launches = 0;
-    e = launch_select_branch(accept_len, batch, n_branches, best_branch, best_len, ctx->stream, &launches);
+    e = launch_select_branch(accept_len, batch, n_branches, best_branch, best_len, ctx->pdl, ctx->stream, &launches);
     ctx->launches += launches;
     if (e != cudaSuccess) return cuda_fail(ctx, "branch selection kernel launch", e);
     return LVSPEC_OK;
@@ -875,7 +877,7 @@ lvspec_status_t lvspec_row_inv_norms(lvspec_ctx_t *ctx, int64_t rows, int32_t di
     cudaError_t e = cudaSetDevice(ctx->device);
     if (e != cudaSuccess) return cuda_fail(ctx, "cudaSetDevice", e);
     int launches = 0;
-    e = launch_row_inv_norms(static_cast<const uint16_t *>(x), rows, dim, inv_norm, ctx->stream, &launches);
+    e = launch_row_inv_norms(static_cast<const uint16_t *>(x), rows, dim, inv_norm, ctx->pdl, ctx->stream, &launches);
     ctx->launches += launches;
     if (e != cudaSuccess) return cuda_fail(ctx, "norm kernel launch", e);
     return LVSPEC_OK;

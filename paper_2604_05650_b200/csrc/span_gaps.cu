@@ -13,6 +13,7 @@
 // gap positions (few, long rounds: a round costs a trip to memory for the keys); a row's
 // sum over the lanes is a fixed butterfly, so the result does not depend on scheduling.
 #include "lvspec_internal.h"
+#include "sm100_ptx.cuh"
 
 namespace lvspec {
 namespace {
@@ -40,6 +41,8 @@ __global__ void __launch_bounds__(kGapThreads) gap_mass_kernel(const GapParams p
     const bool row_ok = r < M;
     const int g = row_ok ? r / G : 0, hg = row_ok ? r - g * G : 0;
     const size_t out_idx = ((size_t)b * p.gamma + g) * p.Hq + kvh * G + hg;
+    ptx::grid_launch_dependents();
+    ptx::grid_dependency_wait();
 
     for (int i = tid; i <= p.n_gaps; i += kGapThreads) {
         first_s[i] = p.gap_first[i];
@@ -128,9 +131,7 @@ __global__ void __launch_bounds__(kGapThreads) gap_mass_kernel(const GapParams p
 
 cudaError_t launch_gap_mass(const GapParams &p, cudaStream_t stream, int *launches)
 {
-    gap_mass_kernel<<<dim3(p.Hkv, (p.M + 7) / 8), kGapThreads, 0, stream>>>(p);
-    ++*launches;
-    return cudaGetLastError();
+    return launch_after(gap_mass_kernel, dim3(p.Hkv, (p.M + 7) / 8), kGapThreads, 0, p.pdl != 0, stream, launches, p);
 }
 
 }  // namespace lvspec

@@ -52,6 +52,8 @@ row_inv_norms_kernel(const uint16_t *x, long long rows, int dim, float *out)
 {
     const long long r = (long long)blockIdx.x * kNormWarps + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
+    grid_launch_dependents();
+    grid_dependency_wait();
     if (r >= rows) return;
     const uint4 *src = reinterpret_cast<const uint4 *>(x + r * dim);
     float acc = 0.f;
@@ -633,12 +635,11 @@ bool make_rows_map(CUtensorMap *map, const void *ptr, int d, int rows, int B, in
 }  // namespace
 
 cudaError_t launch_row_inv_norms(const uint16_t *x, long long rows, int dim, float *out,
-                                 cudaStream_t stream, int *launches)
+                                 bool pdl, cudaStream_t stream, int *launches)
 {
     const long long blocks = (rows + kNormWarps - 1) / kNormWarps;
-    row_inv_norms_kernel<<<(unsigned)blocks, 32 * kNormWarps, 0, stream>>>(x, rows, dim, out);
-    ++*launches;
-    return cudaGetLastError();
+    return launch_after(row_inv_norms_kernel, dim3((unsigned)blocks), 32 * kNormWarps, 0, pdl, stream, launches, x, rows,
+                        dim, out);
 }
 
 // Scratch behind p.cos_t: per (sequence, draft token) a row of lv_pad fp32 values (the
