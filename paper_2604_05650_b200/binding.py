@@ -9,6 +9,7 @@ for device memory and streams only) or as raw integer addresses.
 """
 from __future__ import annotations
 
+import array
 import ctypes
 import os
 from typing import Optional, Sequence
@@ -128,9 +129,7 @@ def load_library(path: Optional[str] = None) -> ctypes.CDLL:
 
 
 def _addr(x) -> Optional[int]:
-    if x is None:
-        return None
-    if isinstance(x, int):
+    if x is None or isinstance(x, int):
         return x
     if isinstance(x, np.ndarray):
         return x.ctypes.data
@@ -139,6 +138,21 @@ def _addr(x) -> Optional[int]:
 
 def _i32(a: Sequence[int]) -> np.ndarray:
     return np.ascontiguousarray(np.asarray(a, dtype=np.int32))
+
+
+def _host_i32(a, nested: bool = False):
+    """Host int32 array as (address, number of elements, what keeps it alive).  Lists of
+    plain integers (nested: of lists of them) take a short way: numpy's costs several
+    microseconds a call, which a decoding loop pays per layer."""
+    if type(a) is list:
+        try:
+            flat = array.array("i", [x for row in a for x in row] if nested else a)
+            if not nested or len(set(map(len, a))) <= 1:
+                return flat.buffer_info()[0], len(flat), flat
+        except TypeError:
+            pass
+    arr = _i32(a)
+    return arr.__array_interface__["data"][0], arr.size, arr
 
 
 class Context:
@@ -214,56 +228,56 @@ class Context:
         return int(fn(self._h, ctypes.byref(shape), int(max_kv_len)))
 
     # -- lvspec_verify_attention ------------------------------------------------
+    @staticmethod
+    def _lengths(shape, kv_len, visual_span):
+        """Addresses of the two host arrays, checked against the batch, and what keeps them."""
+        kv, n_kv, keep_kv = _host_i32(kv_len)
+        sp, n_sp, keep_sp = _host_i32(visual_span, True)
+        batch = shape.batch
+        if batch >= 1 and (n_kv != batch or n_sp != 2 * batch):
+            raise ValueError("kv_len needs B entries and visual_span B pairs")
+        return kv, sp, (keep_kv, keep_sp)
+
     def verify_attention(self, shape: AttnShape, q, k_cache, v_cache, kv_len, visual_span,
                          out, visual_mass) -> None:
-        kv_len, span = _i32(kv_len), _i32(visual_span)
-        if shape.batch >= 1 and (kv_len.size != shape.batch or span.size != 2 * shape.batch):
-            raise ValueError("kv_len needs B entries and visual_span B pairs")
+        kv_len, span, _keep = self._lengths(shape, kv_len, visual_span)
         self._check(self._lib.lvspec_verify_attention(
             self._h, ctypes.byref(shape), _addr(q), _addr(k_cache), _addr(v_cache),
-            kv_len.ctypes.data, span.ctypes.data, _addr(out), _addr(visual_mass)))
+            kv_len, span, _addr(out), _addr(visual_mass)))
 
     def verify_attention_strided(self, shape: AttnShape, k_strides, v_strides, q, k_cache, v_cache, kv_len,
                                  visual_span, out, visual_mass) -> None:
         """k_strides / v_strides: (batch, head, position) strides in elements."""
-        kv_len, span = _i32(kv_len), _i32(visual_span)
-        if shape.batch >= 1 and (kv_len.size != shape.batch or span.size != 2 * shape.batch):
-            raise ValueError("kv_len needs B entries and visual_span B pairs")
+        kv_len, span, _keep = self._lengths(shape, kv_len, visual_span)
         ks, vs = KvStrides(*[int(x) for x in k_strides]), KvStrides(*[int(x) for x in v_strides])
         self._check(self._lib.lvspec_verify_attention_strided(
             self._h, ctypes.byref(shape), ctypes.byref(ks), ctypes.byref(vs), _addr(q), _addr(k_cache),
-            _addr(v_cache), kv_len.ctypes.data, span.ctypes.data, _addr(out), _addr(visual_mass)))
+            _addr(v_cache), kv_len, span, _addr(out), _addr(visual_mass)))
 
     def verify_attention_fp8(self, shape: AttnShape, q, k_cache, v_cache, k_scale, v_scale, kv_len,
                              visual_span, out, visual_mass) -> None:
         """k_cache / v_cache: device uint8 E4M3 codes [B, Hkv, Lmax, D]; k_scale / v_scale:
         device fp32 [B, Hkv]."""
-        kv_len, span = _i32(kv_len), _i32(visual_span)
-        if shape.batch >= 1 and (kv_len.size != shape.batch or span.size != 2 * shape.batch):
-            raise ValueError("kv_len needs B entries and visual_span B pairs")
+        kv_len, span, _keep = self._lengths(shape, kv_len, visual_span)
         self._check(self._lib.lvspec_verify_attention_fp8(
             self._h, ctypes.byref(shape), _addr(q), _addr(k_cache), _addr(v_cache), _addr(k_scale),
-            _addr(v_scale), kv_len.ctypes.data, span.ctypes.data, _addr(out), _addr(visual_mass)))
+            _addr(v_scale), kv_len, span, _addr(out), _addr(visual_mass)))
 
     def verify_attention_tree(self, shape: AttnShape, n_branches, q, k_cache, v_cache, kv_len, visual_span,
                               out, visual_mass) -> None:
-        kv_len, span = _i32(kv_len), _i32(visual_span)
-        if shape.batch >= 1 and (kv_len.size != shape.batch or span.size != 2 * shape.batch):
-            raise ValueError("kv_len needs B entries and visual_span B pairs")
+        kv_len, span, _keep = self._lengths(shape, kv_len, visual_span)
         self._check(self._lib.lvspec_verify_attention_tree(
             self._h, ctypes.byref(shape), int(n_branches), _addr(q), _addr(k_cache), _addr(v_cache),
-            kv_len.ctypes.data, span.ctypes.data, _addr(out), _addr(visual_mass)))
+            kv_len, span, _addr(out), _addr(visual_mass)))
 
     def verify_attention_paged(self, shape: AttnShape, page_size, n_pages, q, k_pool, v_pool, block_table,
                                kv_len, visual_span, out, visual_mass) -> None:
         """k_pool / v_pool: device [n_pages, Hkv, page_size, D]; block_table: device int32
         [B, kv_capacity / page_size]; kv_len, visual_span: host."""
-        kv_len, span = _i32(kv_len), _i32(visual_span)
-        if shape.batch >= 1 and (kv_len.size != shape.batch or span.size != 2 * shape.batch):
-            raise ValueError("kv_len needs B entries and visual_span B pairs")
+        kv_len, span, _keep = self._lengths(shape, kv_len, visual_span)
         self._check(self._lib.lvspec_verify_attention_paged(
             self._h, ctypes.byref(shape), int(page_size), int(n_pages), _addr(q), _addr(k_pool),
-            _addr(v_pool), _addr(block_table), kv_len.ctypes.data, span.ctypes.data, _addr(out),
+            _addr(v_pool), _addr(block_table), kv_len, span, _addr(out),
             _addr(visual_mass)))
 
     def verify_attention_spans(self, shape: AttnShape, q, k_cache, v_cache, kv_len, visual_spans,
@@ -283,12 +297,10 @@ class Context:
 
     def verify_attention_host(self, shape: AttnShape, q, k_cache, v_cache, kv_len, visual_span,
                               out, visual_mass) -> None:
-        kv_len, span = _i32(kv_len), _i32(visual_span)
-        if shape.batch >= 1 and (kv_len.size != shape.batch or span.size != 2 * shape.batch):
-            raise ValueError("kv_len needs B entries and visual_span B pairs")
+        kv_len, span, _keep = self._lengths(shape, kv_len, visual_span)
         self._check(self._lib.lvspec_verify_attention_host(
             self._h, ctypes.byref(shape), _addr(q), _addr(k_cache), _addr(v_cache),
-            kv_len.ctypes.data, span.ctypes.data, _addr(out), _addr(visual_mass)))
+            kv_len, span, _addr(out), _addr(visual_mass)))
 
     # -- lvspec_loose_accept ----------------------------------------------------
     def loose_accept(self, batch, gamma, vocab, n_mass_heads, target_logits, draft_tokens,
