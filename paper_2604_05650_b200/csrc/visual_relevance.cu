@@ -46,6 +46,27 @@ __device__ __forceinline__ float sumsq_bf16x8(uint4 w, float acc)
     return acc;
 }
 
+// Sum of squares of one row of dim bf16 values (a multiple of 8) by one warp: kFlight 16-byte
+// loads in flight per lane, added in index order per lane, then over the lanes (a fixed order).
+template <int kFlight>
+__device__ __forceinline__ float row_sumsq(const uint16_t *row, int dim, int lane)
+{
+    const uint4 *src = reinterpret_cast<const uint4 *>(row);
+    float acc = 0.f;
+    const int n = dim / 8;
+    for (int i0 = lane; i0 < n; i0 += 32 * kFlight) {
+        uint4 w[kFlight];
+#pragma unroll
+        for (int u = 0; u < kFlight; ++u)
+            w[u] = i0 + 32 * u < n ? __ldg(src + i0 + 32 * u) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+        for (int u = 0; u < kFlight; ++u) acc = sumsq_bf16x8(w[u], acc);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    return acc;
+}
+
 // one warp per row; dim a multiple of 8
 __global__ void __launch_bounds__(32 * kNormWarps)
 row_inv_norms_kernel(const uint16_t *x, long long rows, int dim, float *out)
@@ -55,11 +76,7 @@ row_inv_norms_kernel(const uint16_t *x, long long rows, int dim, float *out)
     grid_launch_dependents();
     grid_dependency_wait();
     if (r >= rows) return;
-    const uint4 *src = reinterpret_cast<const uint4 *>(x + r * dim);
-    float acc = 0.f;
-    for (int i = lane; i < dim / 8; i += 32) acc = sumsq_bf16x8(__ldg(src + i), acc);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    const float acc = row_sumsq<8>(x + r * dim, dim, lane);
     if (lane == 0) out[r] = acc > 0.f ? 1.f / sqrtf(acc) : 0.f;
 }
 
@@ -79,7 +96,10 @@ struct CosParams {
     int NP;                 // K padded to a multiple of 16 (MMA N)
     int smem_bytes;         // dynamic shared memory of the launch (after 1024-byte alignment)
     int tmem_cols;
-    int tail_a, tail_b;     // row-group counts that have a one-box tensor map of their own (0 = none)
+    int cap;                // groups of 16 rows of the tallest chunk any CTA meets
+    int slabs;              // 64-channel slabs per stage
+    int stages;
+    int box_a, box_b;       // heights (groups) of the two lower boxes; the tallest is cap
     int n_grp;              // groups of 16 rows per batch element
     int total_groups;       // B * n_grp
     int chunk_groups;       // groups of 16 rows per chunk (<= kChunkGroups)
@@ -122,8 +142,7 @@ __device__ __forceinline__ bool wait_teardown(uint32_t bar, uint32_t parity)
 }
 
 __global__ void __launch_bounds__(kCosThreads, 1)
-cos_tc_kernel(const CosParams P, const __grid_constant__ CUtensorMap tmap_v,
-              const __grid_constant__ CUtensorMap tmap_v128, const __grid_constant__ CUtensorMap tmap_va,
+cos_tc_kernel(const CosParams P, const __grid_constant__ CUtensorMap tmap_v, const __grid_constant__ CUtensorMap tmap_va,
               const __grid_constant__ CUtensorMap tmap_vb, const __grid_constant__ CUtensorMap tmap_d)
 {
     extern __shared__ uint8_t smem_raw[];
@@ -141,18 +160,16 @@ cos_tc_kernel(const CosParams P, const __grid_constant__ CUtensorMap tmap_v,
         walk.n_grp = P.n_grp;
         walk.chunk_groups = P.chunk_groups;
     }
-    // A stage holds 64 channels of the tallest chunk this CTA can meet (row block 0,
-    // then row block 1, then the draft tile); the fewer rows, the more stages fit,
-    // and bytes in flight, not stages, are what covers the memory latency.
-    const int cap = max(1, min(P.chunk_groups, walk.end - walk.gg));
-    const uint32_t d_off = cap <= 8 ? (uint32_t)cap * kGroupBytes : kBlockBytes + (uint32_t)(cap - 8) * kGroupBytes;
-    const uint32_t stage_bytes = (d_off + (uint32_t)NP * 128u + 1023u) & ~1023u;
+    // A stage holds NS slabs of 64 channels of a chunk's rows, slab after slab as one TMA box
+    // delivers them ([slab][row][64 channels]), then the same slabs of the draft tile.
     // An MMA always reads whole row blocks of 128 rows (rows a chunk does not have are
-    // junk lanes nobody looks at), so from the last stage's start one or two full
-    // blocks must still lie inside the allocation.
-    const uint32_t read_extent = cap > 8 ? 2 * kBlockBytes : kBlockBytes;
-    const int S = min(kMaxStages,
-                      1 + (int)(((uint32_t)P.smem_bytes - kBarBytes - max(read_extent, stage_bytes)) / stage_bytes));
+    // junk lanes nobody looks at): the launch leaves room behind the last stage for that.
+    const int NS = P.slabs, S = P.stages, KS = (KC + NS - 1) / NS;
+    const uint32_t d_off = (uint32_t)(NS * P.cap) * kGroupBytes;
+    const uint32_t stage_bytes = d_off + (uint32_t)(NS * NP) * 128u;
+    // the box a chunk of n groups comes in: the lowest that holds it (rows beyond the chunk
+    // are read along where shares cross from one sequence to the next; beyond the last row: zeros)
+    const auto box_of = [&](int n) { return n <= P.box_a ? P.box_a : n <= P.box_b ? P.box_b : P.cap; };
 
     const uint32_t base0 = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t *gbase = smem_raw + (base0 - smem_u32(smem_raw));
@@ -171,9 +188,8 @@ cos_tc_kernel(const CosParams P, const __grid_constant__ CUtensorMap tmap_v,
     if (warp == 0) {
         if (lane == 0) prefetch_tensormap(&tmap_v);
         if (lane == 1) prefetch_tensormap(&tmap_d);
-        if (lane == 2) prefetch_tensormap(&tmap_v128);
-        if (lane == 3) prefetch_tensormap(&tmap_va);
-        if (lane == 4) prefetch_tensormap(&tmap_vb);
+        if (lane == 2) prefetch_tensormap(&tmap_va);
+        if (lane == 3) prefetch_tensormap(&tmap_vb);
         const int n_bars = 2 * S + 6;
         for (int j = lane; j < n_bars; j += 32) {
             uint32_t count = 1;
@@ -199,46 +215,29 @@ cos_tc_kernel(const CosParams P, const __grid_constant__ CUtensorMap tmap_v,
         // ------------------------------------------------------------ TMA producer
         if (lane == 0) {
             const uint64_t stream_policy = l2_evict_first_policy();
-            int n = 0;                       // stages filled so far
+            int n = 0, s = 0;                // stages filled so far, the next one's place in the ring
+            uint32_t round = 0;
             bool ok = true;
-            // Every CTA walks the channels from a different slab on (and around): at a row
+            // Every CTA walks the channels from a different stage on (and around): at a row
             // pitch like 10 KB the same slab of all rows shares its low address bits, and
             // with all CTAs on the same slab the requests crowd on few memory channels.
-            const int kc0 = (int)((blockIdx.x * 37u) % (unsigned)KC);
+            const int ks0 = (int)((blockIdx.x * 37u) % (unsigned)KS);
+            const uint32_t d_bytes = (uint32_t)(NS * NP) * 128u;
             while (ok && walk.next()) {
-                for (int kci = 0; kci < KC; ++kci, ++n) {
-                    const int kc = kci + kc0 < KC ? kci + kc0 : kci + kc0 - KC;
-                    const int s = n % S;
-                    if (n >= S && !mbar_wait(empty(s), ((n / S) - 1) & 1, abort_flag)) { ok = false; break; }
+                const int box = box_of(walk.n_groups);
+                const CUtensorMap *rows = box == P.box_a ? &tmap_va : box == P.box_b ? &tmap_vb : &tmap_v;
+                const uint32_t bytes = (uint32_t)(NS * box) * kGroupBytes + d_bytes;
+                for (int ksi = 0, ks = ks0; ksi < KS; ++ksi, ++n) {
+                    if (n >= S && !mbar_wait(empty(s), (round - 1u) & 1u, abort_flag)) { ok = false; break; }
                     const uint32_t dst = base + s * stage_bytes;
-                    mbar_arrive_expect_tx(full(s), (uint32_t)walk.n_groups * kGroupBytes + (uint32_t)NP * 128u);
-                    // a full row block in one box of 128 rows, the rest in boxes of 16
-                    int g = 0;
-                    if (walk.n_groups >= 8) {
-                        tma_load_3d_hint(dst, &tmap_v128, full(s), kc * 64, walk.row0, walk.b, stream_policy);
-                        g = 8;
-                    }
-                    if (walk.n_groups == 16) {
-                        tma_load_3d_hint(dst + kBlockBytes, &tmap_v128, full(s), kc * 64, walk.row0 + 128,
-                                         walk.b, stream_policy);
-                        g = 16;
-                    }
-                    // what is left of the chunk: in one box when its height is one of the
-                    // two the launch made maps for (issuing a TMA costs the producer
-                    // more than a hundred cycles), else in boxes of 16 rows
-                    const int left = walk.n_groups - g;
-                    if (left > 0 && left == P.tail_a) {
-                        tma_load_3d_hint(dst + g * kGroupBytes, &tmap_va, full(s), kc * 64,
-                                         walk.row0 + g * 16, walk.b, stream_policy);
-                    } else if (left > 0 && left == P.tail_b) {
-                        tma_load_3d_hint(dst + g * kGroupBytes, &tmap_vb, full(s), kc * 64,
-                                         walk.row0 + g * 16, walk.b, stream_policy);
-                    } else {
-                        for (; g < walk.n_groups; ++g)
-                            tma_load_3d_hint(dst + g * kGroupBytes, &tmap_v, full(s), kc * 64,
-                                             walk.row0 + g * 16, walk.b, stream_policy);
-                    }
-                    tma_load_3d(dst + d_off, &tmap_d, full(s), kc * 64, 0, walk.b);
+                    // two requests a stage, however many rows and slabs it holds: each costs the
+                    // producer a hundred cycles and more, which bounded the stream when every slab
+                    // took two or three (slabs beyond the last read as zeros)
+                    mbar_arrive_expect_tx(full(s), bytes);
+                    tma_load_4d_hint(dst, rows, full(s), 0, walk.row0, ks * NS, walk.b, stream_policy);
+                    tma_load_4d(dst + d_off, &tmap_d, full(s), 0, 0, ks * NS, walk.b);
+                    if (++ks == KS) ks = 0;
+                    if (++s == S) { s = 0; ++round; }
                 }
             }
             if (*abort_flag) {
@@ -248,42 +247,60 @@ cos_tc_kernel(const CosParams P, const __grid_constant__ CUtensorMap tmap_v,
         }
     } else if (warp == 1) {
         // -------------------------------------------------------------- MMA issuer
-        if (lane == 0) {
+        // The whole warp runs the loop and one elected lane issues: the descriptors are then the same
+        // in every lane and stay where the instruction takes its operands from.
+        {
             const uint32_t idesc = make_idesc_bf16(128, NP, 0, 0);
             int s = 0, chunk = 0;
             uint32_t round = 0;
             bool ok = true;
+            const int ks0 = (int)((blockIdx.x * 37u) % (unsigned)KS);    // as the producer
             while (ok && walk.next()) {
                 const int buf = chunk & 1;
-                if (chunk >= 2 && !mbar_wait(acc_free(buf), ((chunk >> 1) - 1) & 1, abort_flag)) break;
+                if (chunk >= 2 && !__all_sync(0xffffffffu, mbar_wait(acc_free(buf), ((chunk >> 1) - 1) & 1, abort_flag))) break;
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + buf * 2 * NP;
                 const bool two_blocks = walk.n_groups > 8;
-                for (int kc = 0; kc < KC; ++kc) {
-                    if (!mbar_wait(full(s), round & 1, abort_flag)) { ok = false; break; }
+                const uint32_t slab_step = (uint32_t)box_of(walk.n_groups) * (kGroupBytes >> 4);    // descriptor units
+                const uint32_t d_step = (uint32_t)NP * 8u;
+                uint32_t acc = 0u;
+                for (int ksi = 0, ks = ks0; ksi < KS; ++ksi) {
+                    if (!__all_sync(0xffffffffu, mbar_wait(full(s), round & 1, abort_flag))) { ok = false; break; }
                     tc_fence_after();
                     const uint32_t a0 = base + s * stage_bytes;
-                    const uint64_t da = make_smem_desc(a0, 16, 1024, kSwizzle128B);
-                    const uint64_t db = make_smem_desc(a0 + d_off, 16, 1024, kSwizzle128B);
+                    uint64_t da = make_smem_desc(a0, 16, 1024, kSwizzle128B);
+                    uint64_t db = make_smem_desc(a0 + d_off, 16, 1024, kSwizzle128B);
+                    const int n_slabs = min(NS, KC - ks * NS);
+                    if (elect_one()) {
+                        for (int c = 0; c < n_slabs; ++c, da += slab_step, db += d_step) {
 #pragma unroll
-                    for (int kk = 0; kk < 4; ++kk)
-                        mma_f16_ss(d_tmem, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2), idesc,
-                                   (kc | kk) != 0 ? 1u : 0u);
-                    if (two_blocks) {
+                            for (int kk = 0; kk < 4; ++kk) {
+                                mma_f16_ss(d_tmem, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2), idesc, kk || c ? 1u : acc);
+                            }
+                            if (two_blocks) {
 #pragma unroll
-                        for (int kk = 0; kk < 4; ++kk)
-                            mma_f16_ss(d_tmem + NP, da + (uint64_t)((kBlockBytes >> 4) + kk * 2),
-                                       db + (uint64_t)(kk * 2), idesc, (kc | kk) != 0 ? 1u : 0u);
+                                for (int kk = 0; kk < 4; ++kk)
+                                    mma_f16_ss(d_tmem + NP, da + (uint64_t)((kBlockBytes >> 4) + kk * 2),
+                                               db + (uint64_t)(kk * 2), idesc, kk || c ? 1u : acc);
+                            }
+                        }
+                        mma_commit(empty(s));
                     }
-                    mma_commit(empty(s));
+                    __syncwarp();
+                    acc = 1u;
+                    if (++ks == KS) ks = 0;
                     if (++s == S) { s = 0; ++round; }
                 }
                 if (!ok) break;
-                mma_commit(acc_full(buf));
+                if (elect_one()) mma_commit(acc_full(buf));
+                __syncwarp();
                 ++chunk;
             }
-            mma_commit(drain_bar);         // this thread's MMAs have drained
-            wait_teardown(drain_bar, 0);
+            if (elect_one()) {
+                mma_commit(drain_bar);         // the elected lane's MMAs have drained
+                wait_teardown(drain_bar, 0);
+            }
+            __syncwarp();
         }
     } else {
         // ---------------------------------------------------------- epilogue warps
@@ -301,13 +318,8 @@ cos_tc_kernel(const CosParams P, const __grid_constant__ CUtensorMap tmap_v,
                 if (cur_b >= 0) asm volatile("bar.sync 1, 128;" ::: "memory");   // the old ones are no longer read
                 cur_b = walk.b;
                 for (int k = wq; k < NP; k += 4) {
-                    float acc = 0.f;
-                    if (k < p.K) {
-                        const uint4 *src = reinterpret_cast<const uint4 *>(p.h_draft + ((size_t)cur_b * p.K + k) * p.d);
-                        for (int i = lane; i < p.d / 8; i += 32) acc = sumsq_bf16x8(__ldg(src + i), acc);
-#pragma unroll
-                        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-                    }
+                    const float acc =
+                        k < p.K ? row_sumsq<8>(p.h_draft + ((size_t)cur_b * p.K + k) * p.d, p.d, lane) : 0.f;
                     if (lane == 0) dinv_s[k] = acc > 0.f ? 1.f / sqrtf(acc) : 0.f;
                 }
                 asm volatile("bar.sync 1, 128;" ::: "memory");
@@ -618,16 +630,17 @@ EncodeTiledFn encode_fn()
     return fn;
 }
 
-// [B][rows][d] bf16 as a 3-D tensor; boxes of 64 channels x box_rows rows, 128-byte swizzle
-bool make_rows_map(CUtensorMap *map, const void *ptr, int d, int rows, int B, int box_rows)
+// [B][rows][d] bf16 as a 4-D tensor (64 channels, rows, slabs of 64 channels, sequences);
+// boxes of box_rows rows x box_slabs slabs land slab by slab, 128-byte swizzle
+bool make_rows_map(CUtensorMap *map, const void *ptr, int d, int rows, int B, int box_rows, int box_slabs)
 {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return false;
-    const cuuint64_t dims[3] = {(cuuint64_t)d, (cuuint64_t)rows, (cuuint64_t)B};
-    const cuuint64_t strides[2] = {(cuuint64_t)d * 2, (cuuint64_t)rows * d * 2};
-    const cuuint32_t box[3] = {64, (cuuint32_t)box_rows, 1};
-    const cuuint32_t estr[3] = {1, 1, 1};
-    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(ptr), dims, strides, box,
+    const cuuint64_t dims[4] = {64, (cuuint64_t)rows, (cuuint64_t)(d / 64), (cuuint64_t)B};
+    const cuuint64_t strides[3] = {(cuuint64_t)d * 2, 128, (cuuint64_t)rows * d * 2};
+    const cuuint32_t box[4] = {64, (cuuint32_t)box_rows, (cuuint32_t)box_slabs, 1};
+    const cuuint32_t estr[4] = {1, 1, 1, 1};
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(ptr), dims, strides, box,
               estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
@@ -667,29 +680,35 @@ cudaError_t launch_visual_relevance(const RelevanceParams &p, cudaStream_t strea
     P.tmem_cols = cols;
     P.n_grp = (p.lv + 15) / 16;
     P.total_groups = p.B * P.n_grp;
-    // The shares are `per` or `per + 1` groups; what a share leaves after its full chunks
-    // and its full row block is the tail that gets a map of its own.  (Chunks as tall as
-    // possible: every stage of a chunk costs the producer the same two or three TMA
-    // requests whatever its height; shares cut into three chunks of 64 rows, so that
-    // epilogues could run beside the stream, took twice the time.)
+    // The shares are `per` or `per + 1` groups, walked in chunks of up to 16 (as tall as
+    // possible: a chunk's stages cost the same whatever their height); the two tails a share can
+    // leave have boxes of their own height.
     const int n_cta = P.total_groups < p.n_sm ? P.total_groups : p.n_sm;
     P.chunk_groups = kChunkGroups;
-    auto tail_of = [](int groups) {
-        const int t = groups % kChunkGroups;
-        return t > 8 ? t - 8 : t;       // 0..8 groups
-    };
-    P.tail_a = tail_of(P.total_groups / n_cta);
-    P.tail_b = tail_of(P.total_groups / n_cta + 1);
-    if (P.tail_a * 16 > p.lv) P.tail_a = 0;
-    if (P.tail_b * 16 > p.lv) P.tail_b = 0;
-    CUtensorMap mv, mv128, mva, mvb, md;
-    if (!make_rows_map(&mv, p.h_visual, p.d, p.lv, p.B, 16) ||
-        // (fewer than 128 rows never make a full row block: the wide map is then not used)
-        !make_rows_map(&mv128, p.h_visual, p.d, p.lv, p.B, p.lv >= 128 ? 128 : 16) ||
-        !make_rows_map(&mva, p.h_visual, p.d, p.lv, p.B, P.tail_a > 0 ? P.tail_a * 16 : 16) ||
-        !make_rows_map(&mvb, p.h_visual, p.d, p.lv, p.B, P.tail_b > 0 ? P.tail_b * 16 : 16) ||
+    const int per = P.total_groups / n_cta, most = per + (P.total_groups % n_cta != 0 ? 1 : 0);
+    P.cap = most < kChunkGroups ? most : kChunkGroups;
+    const int tail_a = per % kChunkGroups, tail_b = most % kChunkGroups;
+    P.box_a = tail_a > 0 ? tail_a : P.cap;
+    P.box_b = tail_b > 0 ? tail_b : P.cap;
+    if (P.box_a > P.box_b) { const int t = P.box_a; P.box_a = P.box_b; P.box_b = t; }
+    // Slabs per stage: about 48 KB a stage, so that four are in flight; a row's piece of a stage is then
+    // up to 1 KB in one place (measured: see the file's head).
+    const int slab_bytes = P.cap * (int)kGroupBytes + NP * 128;
+    P.slabs = 49152 / slab_bytes;
+    if (P.slabs > 16) P.slabs = 16;
+    if (P.slabs > p.d / 64) P.slabs = p.d / 64;
+    if (P.slabs < 1) P.slabs = 1;
+    // behind the last stage: what an MMA may read of row blocks beyond the last slab's rows
+    const int extent = P.cap > 8 ? 2 * (int)kBlockBytes : (int)kBlockBytes;
+    const int behind = extent - P.cap * (int)kGroupBytes - P.slabs * NP * 128;
+    P.stages = (P.smem_bytes - (int)kBarBytes - (behind > 0 ? behind : 0)) / (P.slabs * slab_bytes);
+    if (P.stages > kMaxStages) P.stages = kMaxStages;
+    CUtensorMap mv, mva, mvb, md;
+    if (!make_rows_map(&mv, p.h_visual, p.d, p.lv, p.B, P.cap * 16, P.slabs) ||
+        !make_rows_map(&mva, p.h_visual, p.d, p.lv, p.B, P.box_a * 16, P.slabs) ||
+        !make_rows_map(&mvb, p.h_visual, p.d, p.lv, p.B, P.box_b * 16, P.slabs) ||
         // the draft rows as they are: the box is NP rows high, the rows beyond K read as zeros
-        !make_rows_map(&md, p.h_draft, p.d, p.K, p.B, NP))
+        !make_rows_map(&md, p.h_draft, p.d, p.K, p.B, NP, P.slabs))
         return cudaErrorInvalidValue;
     const size_t smem = (size_t)P.smem_bytes + 1024;
     cudaError_t err = cudaFuncSetAttribute(cos_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -701,7 +720,7 @@ cudaError_t launch_visual_relevance(const RelevanceParams &p, cudaStream_t strea
     cfg.stream = stream;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    err = cudaLaunchKernelEx(&cfg, cos_tc_kernel, P, mv, mv128, mva, mvb, md);
+    err = cudaLaunchKernelEx(&cfg, cos_tc_kernel, P, mv, mva, mvb, md);
     ++*launches;
     if (err != cudaSuccess) return err;
 
