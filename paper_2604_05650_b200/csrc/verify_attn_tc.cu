@@ -523,6 +523,9 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                              stream_policy);
     };
 
+    float scale_cta = p.scale_log2;     // softmax scale of this CTA (fp8 cache: with the K scale and q's shift)
+    float v_scale = 1.f;
+
     // ------------------------------------------------------------------ prologue
     // The producer thread sets the barriers up and starts the first loads at
     // once; the other warps prepare shared memory and TMEM meanwhile.
@@ -540,7 +543,6 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                 uint32_t count = 1;
                 if (j >= kHand && j < 3 * kHand) count = kTurns ? 4 : kSoftmaxWarps;   // s_free, p_full: the warps that work on a tile
                 else if (j == n_sp + 1) count = kSoftmaxWarps + 1;              // done
-                else if (kFp8 && j == n_sp + 2) count = kSoftmaxWarps;          // q_full: the warps that split q
                 mbar_init(bar0 + 8 * i, count);
             }
             if (lane == 0) {
@@ -599,37 +601,71 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
         for (int n = idx; n < NP; n += kSoftmaxThreads) {
             m_s[n] = kFp8 ? kMFloor : 0.f;
         }
-        // constant 64 x 16 tiles (K-major, no swizzle: the 8 positions of chunk c
-        // at c * 1024, row r at (r / 8) * 128 + (r % 8) * 16).  Row 0 = ones (sums
-        // l), row 1 = 1 inside the visual span (sums l_vis), rows 2.. = 0.
-        // tile 0: block inside the span, 1: outside, 2: the 16-block holding the
-        // span start, 3: the 16-block holding the span end
-        // (fp8 cache: the tiles are 64 x 32 E4M3, 16 positions per 16-byte chunk, and the
-        // boundary tiles cover the 32-block holding the span's start / end)
-        for (uint32_t i = idx * 16; i < 4 * kA2Bytes; i += kSoftmaxThreads * 16) {
-            const int tile = i / kA2Bytes, off = i % kA2Bytes;
-            const int c = off / 1024, rr = (off % 1024) / 16;   // rr = row index 0..63
-            uint4 val = make_uint4(0, 0, 0, 0);
-            if (rr < 2) {
-                constexpr int kPer = kFp8 ? 16 : 8;             // positions per 16-byte chunk
-                uint32_t w[4] = {0, 0, 0, 0};
+        if (kFp8) {
+            // (q may come from the kernel before this one)
+            grid_dependency_wait();
+            // ---- q as two E4M3 operand tiles (128-byte swizzle, one 128-byte row per query row)
+            // chunk = 8 channels of one row (16 bytes of bf16 in, 8 + 8 bytes out)
+            const int idx = tid - 32 * kSoftmaxWarp0;
+            const int n_chunks = NP * 16;
+            constexpr int kMine = (kMaxRowsFp8 * 16 + kSoftmaxThreads - 1) / kSoftmaxThreads;
+            uint4 qv[kMine];
+            float amax = 0.f;
 #pragma unroll
-                for (int k = 0; k < kPer; ++k) {
-                    int ind = 1;
-                    if (rr == 1) {
-                        if (tile == 0) ind = 1;
-                        else if (tile == 1) ind = 0;
-                        else {
-                            const int pos = ((tile == 2 ? vs : ve) & ~(2 * kPer - 1)) + c * kPer + k;
-                            ind = (pos >= vs && pos < ve) ? 1 : 0;
-                        }
+            for (int u = 0; u < kMine; ++u) {
+                const int ch = idx + u * kSoftmaxThreads;
+                qv[u] = make_uint4(0, 0, 0, 0);
+                if (ch < n_chunks) {
+                    const int n = ch >> 4, c = ch & 15;
+                    if (n < M) {
+                        const int g = n / G, hg = n - g * G;
+                        qv[u] = __ldg(reinterpret_cast<const uint4 *>(
+                            p.q + (((size_t)b * gamma + g) * p.Hq + kvh * G + hg) * 128 + c * 8));
                     }
-                    if (kFp8) w[k >> 2] |= (ind ? 0x38u : 0u) << (8 * (k & 3));       // E4M3 1.0
-                    else w[k >> 1] |= (ind ? 0x3F80u : 0u) << (16 * (k & 1));         // bf16 1.0
+                    const uint32_t w[4] = {qv[u].x, qv[u].y, qv[u].z, qv[u].w};
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        amax = fmaxf(amax, fabsf(__uint_as_float(w[k] << 16)));
+                        amax = fmaxf(amax, fabsf(__uint_as_float(w[k] & 0xFFFF0000u)));
+                    }
                 }
-                val = make_uint4(w[0], w[1], w[2], w[3]);
             }
-            *reinterpret_cast<uint4 *>(gbase + sm.a2 + i) = val;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+            volatile float *wmax = reinterpret_cast<volatile float *>(gbase + sm.misc + 16);
+            if (lane == 0) wmax[warp - kSoftmaxWarp0] = amax;
+            asm volatile("bar.sync %0, %1;" ::"r"(kQBarrier), "r"(kSoftmaxThreads) : "memory");
+            amax = 0.f;
+#pragma unroll
+            for (int u = 0; u < kSoftmaxWarps; ++u) amax = fmaxf(amax, wmax[u]);
+            // power of two that brings the largest magnitude into [128, 256) (NaN or Inf in q:
+            // no shift; the result is then NaN as it would be with any cache)
+            int shift = 0;
+            if (amax > 0.f && amax < INFINITY) shift = 7 - ((int)((__float_as_uint(amax) >> 23) & 0xFF) - 127);
+            shift = max(-100, min(100, shift));
+            const float up = __uint_as_float((uint32_t)(127 + shift) << 23);
+#pragma unroll
+            for (int u = 0; u < kMine; ++u) {
+                const int ch = idx + u * kSoftmaxThreads;
+                if (ch < n_chunks) {
+                    const int n = ch >> 4, c = ch & 15;
+                    const uint32_t w[4] = {qv[u].x, qv[u].y, qv[u].z, qv[u].w};
+                    uint32_t hd[4], rs[4];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const float x0 = __uint_as_float(w[k] << 16) * up, x1 = __uint_as_float(w[k] & 0xFFFF0000u) * up;
+                        const float h0 = e4m3_head(x0), h1 = e4m3_head(x1);
+                        hd[k] = pack_e4m3x2(h0, h1);
+                        rs[k] = pack_e4m3x2(x0 - h0, x1 - h1);
+                    }
+                    const uint32_t off = n * 128 + (((c >> 1) ^ (n & 7)) << 4) + ((c & 1) << 3);
+                    *reinterpret_cast<uint2 *>(gbase + sm.q + off) = make_uint2(hd[0] | (hd[1] << 16), hd[2] | (hd[3] << 16));
+                    *reinterpret_cast<uint2 *>(gbase + sm.q + NP * 128 + off) =
+                        make_uint2(rs[0] | (rs[1] << 16), rs[2] | (rs[3] << 16));
+                }
+            }
+            scale_cta = p.scale_log2 * __ldg(p.k_scale + bh) * __uint_as_float((uint32_t)(127 - shift) << 23);
+            v_scale = __ldg(p.v_scale + bh);
         }
         fence_proxy_async_smem();
     }
@@ -645,76 +681,6 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
     // accumulator columns: the S^T buffers, then O^T and the sums (fp8 cache: two columns per row)
     constexpr int kAccCols = kFp8 ? 2 : 1;
     const uint32_t tm_s0 = tmem_base, tm_o = tmem_base + cfg.sb * NP, tm_l = tm_o + kAccCols * NP;
-    float scale_cta = p.scale_log2;     // softmax scale of this CTA (fp8 cache: with the K scale and q's shift)
-    float v_scale = 1.f;
-    if (kFp8 && warp >= kSoftmaxWarp0 && warp < kPvWarp) {
-        // ---- q as two E4M3 operand tiles (128-byte swizzle, one 128-byte row per query row)
-        // chunk = 8 channels of one row (16 bytes of bf16 in, 8 + 8 bytes out)
-        const int idx = tid - 32 * kSoftmaxWarp0;
-        const int n_chunks = NP * 16;
-        constexpr int kMine = (kMaxRowsFp8 * 16 + kSoftmaxThreads - 1) / kSoftmaxThreads;
-        uint4 qv[kMine];
-        float amax = 0.f;
-#pragma unroll
-        for (int u = 0; u < kMine; ++u) {
-            const int ch = idx + u * kSoftmaxThreads;
-            qv[u] = make_uint4(0, 0, 0, 0);
-            if (ch < n_chunks) {
-                const int n = ch >> 4, c = ch & 15;
-                if (n < M) {
-                    const int g = n / G, hg = n - g * G;
-                    qv[u] = __ldg(reinterpret_cast<const uint4 *>(
-                        p.q + (((size_t)b * gamma + g) * p.Hq + kvh * G + hg) * 128 + c * 8));
-                }
-                const uint32_t w[4] = {qv[u].x, qv[u].y, qv[u].z, qv[u].w};
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    amax = fmaxf(amax, fabsf(__uint_as_float(w[k] << 16)));
-                    amax = fmaxf(amax, fabsf(__uint_as_float(w[k] & 0xFFFF0000u)));
-                }
-            }
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-        volatile float *wmax = reinterpret_cast<volatile float *>(gbase + sm.misc + 16);
-        if (lane == 0) wmax[warp - kSoftmaxWarp0] = amax;
-        asm volatile("bar.sync %0, %1;" ::"r"(kQBarrier), "r"(kSoftmaxThreads) : "memory");
-        amax = 0.f;
-#pragma unroll
-        for (int u = 0; u < kSoftmaxWarps; ++u) amax = fmaxf(amax, wmax[u]);
-        // power of two that brings the largest magnitude into [128, 256) (NaN or Inf in q:
-        // no shift; the result is then NaN as it would be with any cache)
-        int shift = 0;
-        if (amax > 0.f && amax < INFINITY) shift = 7 - ((int)((__float_as_uint(amax) >> 23) & 0xFF) - 127);
-        shift = max(-100, min(100, shift));
-        const float up = __uint_as_float((uint32_t)(127 + shift) << 23);
-#pragma unroll
-        for (int u = 0; u < kMine; ++u) {
-            const int ch = idx + u * kSoftmaxThreads;
-            if (ch < n_chunks) {
-                const int n = ch >> 4, c = ch & 15;
-                const uint32_t w[4] = {qv[u].x, qv[u].y, qv[u].z, qv[u].w};
-                uint32_t hd[4], rs[4];
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const float x0 = __uint_as_float(w[k] << 16) * up, x1 = __uint_as_float(w[k] & 0xFFFF0000u) * up;
-                    const float h0 = e4m3_head(x0), h1 = e4m3_head(x1);
-                    hd[k] = pack_e4m3x2(h0, h1);
-                    rs[k] = pack_e4m3x2(x0 - h0, x1 - h1);
-                }
-                const uint32_t off = n * 128 + (((c >> 1) ^ (n & 7)) << 4) + ((c & 1) << 3);
-                *reinterpret_cast<uint2 *>(gbase + sm.q + off) = make_uint2(hd[0] | (hd[1] << 16), hd[2] | (hd[3] << 16));
-                *reinterpret_cast<uint2 *>(gbase + sm.q + NP * 128 + off) =
-                    make_uint2(rs[0] | (rs[1] << 16), rs[2] | (rs[3] << 16));
-            }
-        }
-        fence_proxy_async_smem();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(q_full);
-        scale_cta = p.scale_log2 * __ldg(p.k_scale + bh) * __uint_as_float((uint32_t)(127 - shift) << 23);
-        v_scale = __ldg(p.v_scale + bh);
-    }
-
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer
         if (lane == 0) {
@@ -750,7 +716,7 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
             }
             if (*abort_flag) {
                 // wait (bounded) for the copies still in flight before the CTA leaves
-                wait_unconditional(q_full, 0);
+                if (!kFp8) wait_unconditional(q_full, 0);
                 for (int j = max(0, nk - cfg.ks); j < nk; ++j)
                     wait_unconditional(k_full(j % cfg.ks), (j / cfg.ks) & 1);
                 for (int j = max(0, nv - cfg.vs); j < nv; ++j)
@@ -809,7 +775,8 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                 hand.next();
                 return true;
             };
-            bool ok = __all_sync(0xffffffffu, mbar_wait(q_full, 0, abort_flag));
+            // (fp8 cache: the CTA has split q itself, ahead of the barrier above)
+            bool ok = kFp8 || __all_sync(0xffffffffu, mbar_wait(q_full, 0, abort_flag));
             for (int i = 0; ok && i < T; ++i) ok = issue_qk(i);
             // every MMA issued by the elected lane has finished before TMEM is released
             if (elect_one()) {
@@ -822,6 +789,36 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
         // ------------------------------------------------- P.V and sum MMA issuer
         // (whole warp in the loop, one elected lane issues: see the K.Q^T issuer)
         {
+            // This warp is idle until the first P^T: it makes its constant tiles, 64 x 16 bf16 (K-major,
+            // no swizzle: the 8 positions of chunk c at c * 1024, row r at (r / 8) * 128 +
+            // (r % 8) * 16).  Row 0 = ones (sums l), row 1 = 1 inside the visual span (sums
+            // l_vis), rows 2.. = 0.  Tile 0: block inside the span, 1: outside, 2: the 16-block
+            // holding the span start, 3: the 16-block holding the span end.
+            // (fp8 cache: the tiles are 64 x 32 E4M3, 16 positions per 16-byte chunk, and the
+            // boundary tiles cover the 32-block holding the span's start / end)
+#pragma unroll 1
+            for (uint32_t i = lane * 16; i < 4 * kA2Bytes; i += 512)
+                *reinterpret_cast<uint4 *>(gbase + sm.a2 + i) = make_uint4(0, 0, 0, 0);
+            __syncwarp();
+            if (lane < 16) {
+                constexpr int kPer = kFp8 ? 16 : 8;             // positions per 16-byte chunk
+                const int tile = lane >> 2, c = (lane >> 1) & 1, rr = lane & 1;
+                const int p0 = ((tile == 2 ? vs : ve) & ~(2 * kPer - 1)) + c * kPer;
+                // the chunk's positions [lo, hi) count
+                const int lo = rr == 1 && tile >= 2 ? vs - p0 : 0;
+                const int hi = rr == 0 || tile == 0 ? kPer : tile == 1 ? 0 : ve - p0;
+                uint32_t w[4] = {0, 0, 0, 0};
+#pragma unroll
+                for (int k = 0; k < kPer; ++k) {
+                    const bool one = k >= lo && k < hi;
+                    if (kFp8) w[k >> 2] |= (one ? 0x38u : 0u) << (8 * (k & 3));       // E4M3 1.0
+                    else w[k >> 1] |= (one ? 0x3F80u : 0u) << (16 * (k & 1));         // bf16 1.0
+                }
+                *reinterpret_cast<uint4 *>(gbase + sm.a2 + tile * kA2Bytes + c * 1024 + rr * 16) =
+                    make_uint4(w[0], w[1], w[2], w[3]);
+            }
+            fence_proxy_async_smem();
+            __syncwarp();
             const uint32_t idesc_pv = kFp8 ? make_idesc_e4m3(128, 2 * NP, 1, 1) : make_idesc_bf16(128, NP, 1, 1);
             const uint32_t idesc_sum = kFp8 ? make_idesc_e4m3(64, 2 * NP, 0, 1) : make_idesc_bf16(64, NP, 0, 1);
             // one MMA covers 16 positions of a bf16 tile, 32 of an fp8 tile
@@ -936,6 +933,35 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                 idx += kSoftmaxGroups;
                 while (idx >= n) idx -= n;
             };
+            // E4M3 has 17 binades, so the reference exponent of a row starts from the largest score
+            // of the split's first tile, not from whatever score its first position happens to
+            // have: all groups take a share of the columns (the last barrier keeps a group that is
+            // late from meeting the hand-over barrier of tile 0 two phases on)
+            {
+                mbar_wait(s_full(0), 0, abort_flag);
+                tc_fence_after();
+                const int pos = t_begin * kTilePos + row;
+                const Seen seen = seen_by(t_begin * kTilePos + kTilePos > L - gamma ? pos - L + gamma : -1, G, gamma, p.branch_len);
+#pragma unroll 1
+                for (int c8 = grp; c8 < n8; c8 += kSoftmaxGroups) {
+                    uint32_t r[8];
+                    tmem_ld_x8(tm_s0 + lane_addr + c8 * 8, r);
+                    tmem_wait_ld();
+                    float s2[8];
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) s2[k] = warp_max_f32(seen(c8 * 8 + k) ? __uint_as_float(r[k]) * scale : -INFINITY);
+                    if (lane == 0) {
+                        float *dst = tmx_s + wq * NP + c8 * 8;
+                        *reinterpret_cast<float4 *>(dst) = make_float4(s2[0], s2[1], s2[2], s2[3]);
+                        *reinterpret_cast<float4 *>(dst + 4) = make_float4(s2[4], s2[5], s2[6], s2[7]);
+                    }
+                }
+                asm volatile("bar.sync %0, %1;" ::"r"(kQBarrier), "r"(kSoftmaxThreads) : "memory");
+                for (int n = tid - 32 * kSoftmaxWarp0; n < n8 * 8; n += kSoftmaxThreads)
+                    m_s[n] = fmaxf(kMFloor, fmaxf(fmaxf(tmx_s[n], tmx_s[NP + n]),
+                                                  fmaxf(tmx_s[2 * NP + n], tmx_s[3 * NP + n])) - kLift);
+                asm volatile("bar.sync %0, %1;" ::"r"(kQBarrier), "r"(kSoftmaxThreads) : "memory");
+            }
             for (int i = grp; i < T; i += kSoftmaxGroups) {
                 const int pos0 = (t_begin + i) * kTilePos;
                 const int pos = pos0 + row;
@@ -945,12 +971,11 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                 tc_fence_after();
                 const uint32_t s_addr = tm_s0 + sbi * NP + lane_addr;
                 // The oldest uncommitted tile is the one whose group may move m.  Tile 0 is that
-                // from the start and sets m up; the others read m under an epoch and check it
-                // when their turn comes.
+                // from the start; the others read m under an epoch and check it when their turn
+                // comes.
                 bool my_turn = i == 0;
                 uint32_t e0 = 0;
                 if (i > 0) {
-                    if (i < kSoftmaxGroups) wait_counter(epoch_s, 1);     // m comes from the first tile
                     e0 = *epoch_s;
                     __threadfence_block();
                 }
@@ -962,14 +987,8 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                 if (warp == kSoftmaxWarp0) LVSPEC_TILE_TS(tile_tr, 0, i, 2);     // P buffer free
                 uint8_t *prow = gbase + sm.p + pb * (NP * 256) + row * 16;
 
-                // fp8 cache: E4M3 has 17 binades, so the reference exponent of a row starts
-                // from the largest score of the split's first tile (the path below), not
-                // from whatever score its first position happens to have
-                bool take_max = kFp8 && i == 0;
-                for (int attempt = 0; attempt < 4; ++attempt) {
-                    float gmax = -INFINITY;
-                    if (!take_max)
-                        gmax = !tail ? softmax_pass<false>(s_addr, n8, m_s, scale, seen, prow,
+                for (int attempt = 0; attempt < 3; ++attempt) {
+                    const float gmax = !tail ? softmax_pass<false>(s_addr, n8, m_s, scale, seen, prow,
                                                              warp == kSoftmaxWarp0 ? tile_tr : nullptr, i)
                                      : softmax_pass<true>(s_addr, n8, m_s, scale, seen, prow, nullptr, i);
                     if (warp == kSoftmaxWarp0) LVSPEC_TILE_TS(tile_tr, 0, i, 3);     // exponentials done
@@ -982,10 +1001,9 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                         if (!group_any(bar_id, stale || gmax > kLimit)) break;
                         // m moved while some thread computed under the old one: once more
                         if (group_any(bar_id, stale)) continue;
-                    } else if (!take_max && !group_any(bar_id, gmax > kLimit)) {
+                    } else if (!group_any(bar_id, gmax > kLimit)) {
                         break;
                     }
-                    take_max = false;
 
                     // ---- a score ran past the guard: move m up to the tile maximum ----
                     // (the masked form, with its divisions, only where the tile reaches the draft slots)
