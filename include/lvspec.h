@@ -129,7 +129,8 @@ const char *lvspec_status_string(lvspec_status_t status);
 uint64_t lvspec_launch_count(const lvspec_ctx_t *ctx);
 
 /* KV splits the library would use for `shape` with the longest sequence
- * `max_kv_len` (what n_split = 0 resolves to); 0 on invalid input. */
+ * `max_kv_len` (what n_split = 0 resolves to when all sequences are that long; a batch of
+ * different lengths may get up to two CTAs per SM); 0 on invalid input. */
 int32_t lvspec_attention_splits(const lvspec_ctx_t *ctx, const lvspec_attn_shape_t *shape,
                                 int32_t max_kv_len);
 /* The same for lvspec_verify_attention_fp8 (half the bytes per tile: it takes more splits). */

@@ -1,6 +1,7 @@
 // Host side of liblvspec.so: context, argument validation, scratch memory and
 // the launch sequence of each call.  Every step of the verify path itself runs
 // in the kernels; nothing here computes on the CPU.
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -109,10 +110,10 @@ int resolve_kernel(const lvspec_attn_shape_t *s)
 
 // KV splits per (sequence, KV head) when the caller leaves the choice to the library.
 // The tensor-core kernel runs one CTA per SM.  One CTA works through a tile in a time
-// that grows with the query rows it carries (measured: about 2.1 k cycles at 48 padded
-// rows, 2.7 k at 80), so with 40 rows about three quarters of the SMs already stream at
-// the HBM bandwidth, with 80 rows nearly all are needed, and with an fp8 cache (half the
-// bytes per tile for the same work) the device never gets there.  Splits are whole
+// that grows with the query rows it carries (about 2.1 k cycles at 48 padded rows, 2.7 k
+// at 80), so with 40 rows about four fifths of the SMs already stream at
+// the HBM bandwidth, with 80 rows all are needed, and with half the bytes per tile (fp8
+// cache, head_dim 64) the device never gets there.  Splits are whole
 // 128-position tiles, so a split count that does not divide the tile count leaves a last
 // round in which only the CTAs with one tile more are at work, far below the device's
 // bandwidth: with 40 rows, 16 splits of 16 tiles beat 18 splits of 14 or 15 on eight
@@ -121,41 +122,95 @@ int resolve_kernel(const lvspec_attn_shape_t *s)
 // their CTA count reaches, the uneven last round at the bandwidth of its few CTAs, and a
 // charge per CTA for writing its partial and merging it.  A pure function of the shape:
 // results stay reproducible from run to run.
+struct SplitModel {
+    int units, tiles, most;     // (sequence, KV head) pairs; tiles of the longest sequence; splits of one wave
+    double saturating;          // CTAs that reach the HBM bandwidth
+    double rate(double ctas) const { return ctas >= saturating ? 1.0 : ctas / saturating; }
+};
+
+SplitModel split_model(const lvspec_ctx *ctx, const lvspec_attn_shape_t *s, int max_kv_len, bool fp8)
+{
+    SplitModel m;
+    m.tiles = (max_kv_len + 127) / 128;           // splits never go below 128 positions
+    m.units = s->batch * s->n_kv_heads;
+    m.most = ctx->n_sm / m.units;                 // one CTA per SM, one wave
+    if (m.most < 1) m.most = 1;
+    if (m.most > m.tiles) m.most = m.tiles;
+    if (m.most > 256) m.most = 256;
+    const int n_pad = (s->gamma * (s->n_q_heads / s->n_kv_heads) + 15) & ~15;
+    double share = 0.8 * (1100.0 + 20.0 * n_pad) / (1100.0 + 20.0 * 48);
+    // (few rows: the hand-over of a tile takes what it takes)
+    if (fp8 || s->head_dim == 64) share *= 2.1;
+    else if (share < 0.8) share = 0.8;
+    m.saturating = share * ctx->n_sm;
+    return m;
+}
+
 int choose_splits(const lvspec_ctx *ctx, const lvspec_attn_shape_t *s, int max_kv_len, bool fp8 = false)
 {
-    const int tiles = (max_kv_len + 127) / 128;           // splits never go below 128 positions
-    const int units = s->batch * s->n_kv_heads;
+    const SplitModel m = split_model(ctx, s, max_kv_len, fp8);
     if (resolve_kernel(s) != LVSPEC_KERNEL_TCGEN05) {
-        int want = (2 * ctx->n_sm + units - 1) / units;    // about two CTAs per SM
+        int want = (2 * ctx->n_sm + m.units - 1) / m.units;    // about two CTAs per SM
         if (want < 1) want = 1;
-        if (want > tiles) want = tiles;
+        if (want > m.tiles) want = m.tiles;
         if (want > 256) want = 256;
         return want;
     }
-    int most = ctx->n_sm / units;                          // one CTA per SM, one wave
-    if (most < 1) most = 1;
-    if (most > tiles) most = tiles;
-    if (most > 256) most = 256;
-    // CTAs that reach the HBM bandwidth
-    const int n_pad = (s->gamma * (s->n_q_heads / s->n_kv_heads) + 15) & ~15;
-    double share = 0.73 * (1100.0 + 20.0 * n_pad) / (1100.0 + 20.0 * 48);
-    if (share < 0.6) share = 0.6;
-    if (fp8) share *= 2.3;
-    const double saturating = share * ctx->n_sm;
-    auto rate = [&](double ctas) { return ctas >= saturating ? 1.0 : ctas / saturating; };
-    int best = most;
+    int best = m.most;
     double best_cost = 0.0;
-    for (int ns = most; ns >= 1; --ns) {
-        const double ctas = (double)ns * units;
-        const int t_lo = tiles / ns, rem = tiles - t_lo * ns;
-        double cost = t_lo * ctas / rate(ctas) + 0.7 * ctas;
-        if (rem > 0) cost += (double)rem * units / rate((double)rem * units);
-        if (ns == most || cost < best_cost) {
+    for (int ns = m.most; ns >= 1; --ns) {
+        const double ctas = (double)ns * m.units;
+        const int t_lo = m.tiles / ns, rem = m.tiles - t_lo * ns;
+        double cost = t_lo * ctas / m.rate(ctas) + 0.7 * ctas;
+        if (rem > 0) cost += (double)rem * m.units / m.rate((double)rem * m.units);
+        if (ns == m.most || cost < best_cost) {
             best = ns;
             best_cost = cost;
         }
     }
     return best;
+}
+
+// Splits of two waves of CTAs (tensor-core kernel).
+int two_wave_splits(const lvspec_ctx *ctx, const SplitModel &m)
+{
+    int ns = 2 * ctx->n_sm / m.units;
+    if (ns > m.tiles) ns = m.tiles;
+    return ns > 256 ? 256 : ns;
+}
+
+// The same for a batch whose sequences differ in length.  Every sequence is cut into the
+// same number of splits, so in one wave the CTAs of the short ones leave their SMs idle while
+// those of the longest go on; in two waves the second fills in, at the price of a CTA's fixed
+// cost (prologue, first tile, tail) once more.  One wave is modelled as a fluid: CTAs share
+// the bandwidth, no CTA is faster than it is where all of them saturate it.  Measured, one wave
+// -> two: 16 sequences of 8 to 16 K (40 rows) 148 -> 132 us a layer, 8 of 65 to 130 K
+// 552 -> 484, 8 of 20 to 39 K at 72 rows 191 -> 166, 4 of 12 to 20 K 52.2 -> 50.6.
+int choose_splits_for(const lvspec_ctx *ctx, const lvspec_attn_shape_t *s, const SeqInfo &seq, int max_kv_len, bool fp8)
+{
+    const int one = choose_splits(ctx, s, max_kv_len, fp8);
+    if (s->batch < 2 || resolve_kernel(s) != LVSPEC_KERNEL_TCGEN05) return one;
+    int tiles[LVSPEC_MAX_BATCH];
+    long long total = 0;
+    for (int b = 0; b < s->batch; ++b) {
+        tiles[b] = (seq.kv_len[b] + 127) / 128;
+        total += tiles[b];
+    }
+    const SplitModel m = split_model(ctx, s, max_kv_len, fp8);
+    const int two = two_wave_splits(ctx, m);
+    if (total == (long long)m.tiles * s->batch || two <= one) return one;
+    std::sort(tiles, tiles + s->batch);
+    const double per_seq = (double)s->n_kv_heads * one;     // CTAs of a sequence
+    double cost_one = 0.7 * one * m.units, prev = 0.0;
+    for (int b = 0; b < s->batch; ++b) {
+        const double len = (double)tiles[b] / one, active = (s->batch - b) * per_seq;
+        cost_one += (len - prev) * (active > m.saturating ? active : m.saturating);
+        prev = len;
+    }
+    const int n_pad = (s->gamma * (s->n_q_heads / s->n_kv_heads) + 15) & ~15;
+    const double cost_two = (double)total * s->n_kv_heads / m.rate(ctx->n_sm) + 0.7 * two * m.units +
+                            (2.0 + n_pad / 32.0) * (fp8 || s->head_dim == 64 ? 2.0 : 1.0) * ctx->n_sm;
+    return cost_two < cost_one ? two : one;
 }
 
 // Vocabulary slices of the acceptance kernel: enough CTAs for two per SM, at least 4096
@@ -259,7 +314,7 @@ lvspec_status_t run_attention(lvspec_ctx *ctx, const lvspec_attn_shape_t *s, con
     p.Lmax = s->kv_capacity;
     p.G = p.Hq / p.Hkv;
     p.M = p.gamma * p.G;
-    p.n_split = s->n_split > 0 ? s->n_split : choose_splits(ctx, s, max_len, fp8 != nullptr);
+    p.n_split = s->n_split > 0 ? s->n_split : choose_splits_for(ctx, s, seq, max_len, fp8 != nullptr);
     p.scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)p.D));
     p.pdl = ctx->pdl ? 1 : 0;
     p.branch_len = branch_len > 0 ? branch_len : p.gamma;
@@ -556,6 +611,11 @@ size_t lvspec_attention_workspace_bytes(const lvspec_ctx_t *ctx, const lvspec_at
         n_split = choose_splits(ctx, shape, max_kv_len);
         const int n8 = choose_splits(ctx, shape, max_kv_len, true);
         if (n8 > n_split) n_split = n8;
+        // and a batch of different lengths may go in two waves
+        if (shape->batch > 1) {
+            const int two = two_wave_splits(ctx, split_model(ctx, shape, max_kv_len, false));
+            if (two > n_split) n_split = two;
+        }
     }
     // the call with several spans never runs the tensor-core kernel on a single split
     const int n_eff = n_split < 2 ? 2 : n_split;
