@@ -355,29 +355,27 @@ __device__ __forceinline__ uint4 exp_chunk_bf16(const uint32_t *r, const float *
     return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-// A group's share of the columns of one tile, chunks [c_lo, c_hi): exponentials of this
-// thread's position (up to four TMEM loads in flight per wait), stored as they come to its
-// place in the P^T buffer.
+// A group's share of the columns of one tile, n_c chunks from column col0 on: exponentials of
+// this thread's position (up to four TMEM loads in flight per wait), stored as they come to
+// its place in the P^T buffer.  The addresses are those of the share's first chunk.
 template <bool kMask, int kC>
-__device__ __forceinline__ void softmax_share_bf16(uint32_t s_addr, int c_lo, int c_hi, const float *m_s,
-                                                   uint64_t neg_scale2, Seen seen,
-                                                   uint8_t *prow, uint32_t &pmax)
+__device__ __forceinline__ void softmax_share_bf16(uint32_t s_addr, int n_c, const float *m_s, uint64_t neg_scale2,
+                                                   Seen seen, int col0, uint8_t *prow, uint32_t &pmax)
 {
     constexpr int kB = kC < 4 ? kC : 4;      // chunks in flight
 #pragma unroll
     for (int h = 0; h < (kC + kB - 1) / kB; ++h) {
-        const int cb = c_lo + kB * h;
-        if (cb < c_hi) {
+        if (kB * h < n_c) {
             uint32_t r[kB][8];
 #pragma unroll
             for (int u = 0; u < kB; ++u)
-                if (kB * h + u < kC && cb + u < c_hi) tmem_ld_x8(s_addr + (cb + u) * 8, r[u]);
+                if (kB * h + u < kC && kB * h + u < n_c) tmem_ld_x8(s_addr + (kB * h + u) * 8, r[u]);
             tmem_wait_ld();
 #pragma unroll
             for (int u = 0; u < kB; ++u)
-                if (kB * h + u < kC && cb + u < c_hi)
-                    *reinterpret_cast<uint4 *>(prow + (cb + u) * 2048) =
-                        exp_chunk_bf16<kMask>(r[u], m_s + (cb + u) * 8, neg_scale2, seen, (cb + u) * 8, pmax);
+                if (kB * h + u < kC && kB * h + u < n_c)
+                    *reinterpret_cast<uint4 *>(prow + (kB * h + u) * 2048) =
+                        exp_chunk_bf16<kMask>(r[u], m_s + (kB * h + u) * 8, neg_scale2, seen, col0 + (kB * h + u) * 8, pmax);
         }
     }
 }
@@ -1116,11 +1114,28 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
             // Tiles go through in twos where the buffers allow (256 positions): one vote on the
             // guard, one fence and one hand-over for both.
             // Ring positions advance by counting, not by dividing.
-            int sbi = 0, pb = 0, vsl = 0;        // S^T buffer, P buffer and V slot of tile i
-            uint32_t vs_round = 0;               // how often the V ring has wrapped
+            int sbi = 0, pb = 0;                 // S^T buffer and P buffer of tile i
             const uint64_t neg_scale2 = pack_f32x2(__float_as_uint(-scale), __float_as_uint(-scale));
+            if (!kFp8) {
+                // reference exponent of each row: its score at the split's first position
+                mbar_wait(s_full(0), 0, abort_flag);
+                tc_fence_after();
+                if (wq == 0) {
+                    for (int c8 = c_lo; c8 < c_hi; ++c8) {
+                        uint32_t r[8];
+                        tmem_ld_x8(tm_s0 + lane_addr + c8 * 8, r);
+                        tmem_wait_ld();
+                        if (lane == 0) {
+#pragma unroll
+                            for (int k = 0; k < 8; ++k) m_s[c8 * 8 + k] = __uint_as_float(r[k]) * scale - kLift;
+                        }
+                    }
+                }
+                group_sync(bar_id);
+            }
             for (int i = 0; i < T; i += cfg.step) {
                 const int n_sub = min(cfg.step, T - i);
+                int sb_u, pb_u;
                 for (int attempt = 0; attempt < 3; ++attempt) {
                     // fp8 cache: E4M3 has 17 binades, so the reference exponent of a row starts
                     // from the largest score of the split's first tile (the path below), not
@@ -1128,36 +1143,23 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                     const bool first_max = kFp8 && i == 0 && attempt == 0;
                     float gmax = -INFINITY;
                     uint32_t pmax = 0u;
-                    int sb_u = sbi, pb_u = pb;
+                    sb_u = sbi;
+                    pb_u = pb;
 #pragma unroll 1
                     for (int u = 0; u < n_sub; ++u) {
                         const int iu = i + u;
                         const int pos0 = (t_begin + iu) * kTilePos;
-                        if (attempt == 0 || iu == 1) {
+                        if (!kFp8 || attempt == 0 || iu == 1) {     // (a phase that is over is over at once)
                             if (warp == kSoftmaxWarp0) LVSPEC_TILE_TS(tile_tr, 0, iu, 0);     // starts waiting for S^T
                             mbar_wait(s_full(iu), hand_parity(iu), abort_flag);
                             if (warp == kSoftmaxWarp0) LVSPEC_TILE_TS(tile_tr, 0, iu, 1);     // S^T there
                             tc_fence_after();
                         }
                         const uint32_t s_addr = tm_s0 + sb_u * NP + lane_addr;
-                        if (!kFp8 && iu == 0 && attempt == 0) {
-                            // reference exponent of each row: its score at the split's first position
-                            if (wq == 0) {
-                                for (int c8 = c_lo; c8 < c_hi; ++c8) {
-                                    uint32_t r[8];
-                                    tmem_ld_x8(s_addr + c8 * 8, r);
-                                    tmem_wait_ld();
-                                    if (lane == 0) {
-#pragma unroll
-                                        for (int k = 0; k < 8; ++k) m_s[c8 * 8 + k] = __uint_as_float(r[k]) * scale - kLift;
-                                    }
-                                }
-                            }
-                            group_sync(bar_id);
-                        }
                         if (first_max) break;
                         const bool tail = pos0 + kTilePos > L - gamma;
-                        const Seen seen = seen_by(tail ? pos0 + row - L + gamma : -1, G, gamma, p.branch_len);
+                        Seen seen = {0, 0xFFFFFFFFu};
+                        if (tail) seen = seen_by(pos0 + row - L + gamma, G, gamma, p.branch_len);
                         uint8_t *prow = gbase + sm.p + pb_u * (NP * 256) + row * 16;
                         // P^T goes straight to shared memory, once the P.V product that read this buffer is done
                         if (attempt == 0 && iu >= cfg.pb) mbar_wait(p_free(iu - cfg.pb), hand_parity(iu - cfg.pb), abort_flag);
@@ -1171,9 +1173,11 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                             for (int j = 0; j < kC; ++j)
                                 if (c_lo + j < c_hi) *reinterpret_cast<uint4 *>(prow + (c_lo + j) * 2048) = pk[j];
                         } else if (!tail) {
-                            softmax_share_bf16<false, kC>(s_addr, c_lo, c_hi, m_s, neg_scale2, seen, prow, pmax);
+                            softmax_share_bf16<false, kC>(s_addr + c_lo * 8, c_hi - c_lo, m_s + c_lo * 8, neg_scale2, seen, c_lo * 8,
+                                                          prow + c_lo * 2048, pmax);
                         } else {
-                            softmax_share_bf16<true, kC>(s_addr, c_lo, c_hi, m_s, neg_scale2, seen, prow, pmax);
+                            softmax_share_bf16<true, kC>(s_addr + c_lo * 8, c_hi - c_lo, m_s + c_lo * 8, neg_scale2, seen, c_lo * 8,
+                                                         prow + c_lo * 2048, pmax);
                         }
                         if (warp == kSoftmaxWarp0) LVSPEC_TILE_TS(tile_tr, 0, iu, 3);     // probabilities stored
                         if (++sb_u == cfg.sb) sb_u = 0;
@@ -1249,9 +1253,7 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                 if (grp == 0 && (t_begin + i + n_sub) * kTilePos > L) {
                     // slots at or beyond kv_len hold whatever the cache holds: zero their V
                     // rows so that 0 * junk cannot poison the accumulators (they sit in the last tile)
-                    int vz = vsl;
-                    uint32_t vr = vs_round;
-                    if (n_sub == 2 && ++vz == cfg.vs) { vz = 0; ++vr; }
+                    const int vz = (i + n_sub - 1) % cfg.vs, vr = (i + n_sub - 1) / cfg.vs;
                     // the slot's tile before is done with (a parity tells this phase from its
                     // neighbours only, and the products may lag by the depth of the P^T ring)
                     const int before = i + n_sub - 1 - cfg.vs;
@@ -1272,16 +1274,15 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                 fence_proxy_async_smem();
                 __syncwarp();
                 if (lane == 0) {
-                    mbar_arrive(p_full(i));
+                    // (with one K slot the next K.Q^T goes first: the slot's load hangs on it)
+                    if (cfg.ks > 1) mbar_arrive(p_full(i));
                     mbar_arrive(s_free(i));
                     if (n_sub == 2) mbar_arrive(s_free(i + 1));
+                    if (cfg.ks == 1) mbar_arrive(p_full(i));
                 }
                 if (warp == kSoftmaxWarp0) LVSPEC_TILE_TS(tile_tr, 0, i, 5);     // P^T stored and handed over
-                for (int u = 0; u < n_sub; ++u) {
-                    if (++sbi == cfg.sb) sbi = 0;
-                    if (++pb == cfg.pb) pb = 0;
-                    if (++vsl == cfg.vs) { vsl = 0; ++vs_round; }
-                }
+                sbi = sb_u;
+                pb = pb_u;
             }
         }
 
@@ -1465,10 +1466,11 @@ TcConfig pick_config(int M, int page_slots, bool fp8, bool turns, int D)
         // more than two ring slots each.  64 KB of K/V in flight per CTA and die-wide 16 MB
         // are enough for HBM, and more of them at the start of a launch only put later tiles
         // ahead of the first one's (40 rows, 16 tiles per CTA: 26.9 us with 2 + 2 slots,
-        // 27.9 with 3 + 2 or 2 + 3).
+        // 27.9 with 3 + 2 or 2 + 3).  At 128 rows a second P^T buffer before a second K slot: 38.3 us
+        // a layer of 32K against 47.1.
         c.sb = 512 / c.n_pad - acc;
         if (c.sb > 4) c.sb = 4;
-        const int tries[5][3] = {{2, 2, 4}, {2, 2, 3}, {2, 2, 2}, {2, 3, 1}, {2, 2, 1}};
+        const int tries[5][3] = {{2, 2, 4}, {2, 2, 3}, {2, 2, 2}, {1, 2, 2}, {2, 2, 1}};
         const int tries8[5][3] = {{4, 4, 4}, {4, 4, 3}, {4, 4, 2}, {4, 4, 1}, {3, 3, 1}};
         for (int t = 0; t < 5; ++t) {
             const int *tr = small_tiles ? tries8[t] : tries[t];
