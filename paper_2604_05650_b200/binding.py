@@ -142,15 +142,18 @@ def _i32(a: Sequence[int]) -> np.ndarray:
 
 def _host_i32(a, nested: bool = False):
     """Host int32 array as (address, number of elements, what keeps it alive).  Lists of
-    plain integers (nested: of lists of them) take a short way: numpy's costs several
-    microseconds a call, which a decoding loop pays per layer."""
-    if type(a) is list:
-        try:
-            flat = array.array("i", [x for row in a for x in row] if nested else a)
-            if not nested or len(set(map(len, a))) <= 1:
-                return flat.buffer_info()[0], len(flat), flat
-        except TypeError:
-            pass
+    plain integers (nested: of lists or tuples of them, all as long) take a short way: numpy's
+    costs several microseconds a call, which a decoding loop pays per layer.  All else is
+    numpy's to convert or to refuse."""
+    if type(a) is list and a:
+        if nested:
+            flat = [x for row in a for x in row] if {list, tuple}.issuperset(map(type, a)) else ()
+            plain = len(set(map(len, a))) == 1 if flat else False
+        else:
+            flat, plain = a, True
+        if plain and set(map(type, flat)) == {int}:
+            arr = array.array("i", flat)
+            return arr.buffer_info()[0], len(arr), arr
     arr = _i32(a)
     return arr.__array_interface__["data"][0], arr.size, arr
 

@@ -25,6 +25,28 @@ def test_same_as_numpy(value, nested):
     assert n == want.size and _read(addr, n) == want.tolist()
 
 
+class _Index:
+    """An integer to array.array, nothing to numpy."""
+    def __index__(self):
+        return 3
+
+    def __int__(self):
+        raise TypeError("no")
+
+
+@pytest.mark.parametrize("value,nested", [
+    ([{0, 3}], True), ([{0: 1, 3: 2}], True), ([b"ab"], True), ([frozenset([4, 9]), [0, 3]], True),
+    ([_Index(), 2], False), ([[_Index(), 2]], True), ([iter([0, 3])], True),
+])
+def test_what_numpy_refuses_stays_refused(value, nested):
+    """Rows that are not sequences, and elements that only look like integers, do not slip
+    through the short way (a set's order is not the caller's)."""
+    with pytest.raises((OverflowError, ValueError, TypeError)) as want:
+        np.asarray(value, dtype=np.int32)
+    with pytest.raises(want.type):
+        binding._host_i32(value, nested)
+
+
 @pytest.mark.parametrize("value,nested", [([2**31], False), ([[0, 2**40]], True), (["x"], False), ([[0, 1], [2]], True),
                                           ([None], False)])
 def test_refused_as_before(value, nested):
