@@ -145,13 +145,19 @@ def _host_i32(a, nested: bool = False):
     plain integers (nested: of lists or tuples of them, all as long) take a short way: numpy's
     costs several microseconds a call, which a decoding loop pays per layer.  All else is
     numpy's to convert or to refuse."""
-    if type(a) is list and a:
+    if type(a) is list:
+        flat = a
         if nested:
-            flat = [x for row in a for x in row] if {list, tuple}.issuperset(map(type, a)) else ()
-            plain = len(set(map(len, a))) == 1 if flat else False
+            flat = []
+            for row in a:
+                if type(row) is not list and type(row) is not tuple or len(row) != len(a[0]):
+                    flat = None
+                    break
+                flat += row
+        for x in flat or (None,):
+            if type(x) is not int:
+                break
         else:
-            flat, plain = a, True
-        if plain and set(map(type, flat)) == {int}:
             arr = array.array("i", flat)
             return arr.buffer_info()[0], len(arr), arr
     arr = _i32(a)
