@@ -146,8 +146,9 @@ int32_t lvspec_attention_splits_fp8(const lvspec_ctx_t *ctx, const lvspec_attn_s
  * buffer first:
  *
  *   lvspec_*_workspace_bytes  bytes of scratch the call of that shape needs
- *       (attention: any of the lvspec_verify_attention* forms with `shape`, the
- *       longest sequence `max_kv_len` and the split choice `shape->n_split`;
+ *       (attention: any of the lvspec_verify_attention* forms with `shape`,
+ *       sequences of up to `max_kv_len` positions, alike or not, and the split
+ *       choice `shape->n_split`;
  *       accept: any of the lvspec_loose_accept* forms that take a context;
  *       relevance: lvspec_visual_relevance).  0 on invalid input.
  *   lvspec_reserve            grows the buffer to at least `workspace_bytes`

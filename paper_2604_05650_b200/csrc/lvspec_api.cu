@@ -179,7 +179,19 @@ int two_wave_splits(const lvspec_ctx *ctx, const SplitModel &m)
     return ns > 256 ? 256 : ns;
 }
 
-// The same for a batch whose sequences differ in length.  Every sequence is cut into the
+// The most splits any call of this shape with sequences of up to max_kv_len positions takes
+// by itself, whatever the cache format and the lengths: what scratch is sized for.  Unlike
+// the choice itself (even cuts are preferred: 10 splits of 19 tiles, 18 of 18), it never falls
+// as max_kv_len grows.
+int most_splits(const lvspec_ctx *ctx, const lvspec_attn_shape_t *s, int max_kv_len)
+{
+    if (resolve_kernel(s) != LVSPEC_KERNEL_TCGEN05) return choose_splits(ctx, s, max_kv_len);
+    const SplitModel m = split_model(ctx, s, max_kv_len, false);
+    const int two = s->batch > 1 ? two_wave_splits(ctx, m) : 0;
+    return two > m.most ? two : m.most;
+}
+
+// The choice for a batch whose sequences differ in length.  Every sequence is cut into the
 // same number of splits, so in one wave the CTAs of the short ones leave their SMs idle while
 // those of the longest go on; in two waves the second fills in, at the price of a CTA's fixed
 // cost (prologue, first tile, tail) once more.  One wave is modelled as a fluid: CTAs share
@@ -605,18 +617,7 @@ size_t lvspec_attention_workspace_bytes(const lvspec_ctx_t *ctx, const lvspec_at
     if (!ctx || !shape || shape->batch < 1 || shape->n_kv_heads < 1 || shape->gamma < 1 ||
         shape->n_q_heads < shape->n_kv_heads || shape->head_dim < 1 || max_kv_len < 1 || shape->n_split < 0)
         return 0;
-    // the library's own choice differs between the bf16 and the fp8 cache: the larger of the two
-    int n_split = shape->n_split;
-    if (n_split == 0) {
-        n_split = choose_splits(ctx, shape, max_kv_len);
-        const int n8 = choose_splits(ctx, shape, max_kv_len, true);
-        if (n8 > n_split) n_split = n8;
-        // and a batch of different lengths may go in two waves
-        if (shape->batch > 1) {
-            const int two = two_wave_splits(ctx, split_model(ctx, shape, max_kv_len, false));
-            if (two > n_split) n_split = two;
-        }
-    }
+    const int n_split = shape->n_split > 0 ? shape->n_split : most_splits(ctx, shape, max_kv_len);
     // the call with several spans never runs the tensor-core kernel on a single split
     const int n_eff = n_split < 2 ? 2 : n_split;
     const int M = shape->gamma * (shape->n_q_heads / shape->n_kv_heads);

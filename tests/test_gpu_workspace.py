@@ -135,6 +135,25 @@ def test_workspace_queries_cover_what_the_calls_take():
         ctx.close()
 
 
+@pytest.mark.parametrize("heads", [(64, 8, 14), (16, 4, 16), (40, 8, 8), (64, 8, 10), (8, 2, 4)])
+@pytest.mark.parametrize("batch", [1, 3])
+def test_the_figure_for_a_length_covers_all_shorter_ones(heads, batch):
+    """The library's split count is not monotone in the length (18 tiles: 18 splits, 19 tiles: 10);
+    the figure for the longest sequence has to cover the count of every shorter one."""
+    from paper_2604_05650_b200 import binding
+    ctx = _fresh_ctx()
+    try:
+        hq, hkv, gamma = heads
+        M = gamma * hq // hkv
+        most = 0
+        for tiles in range(1, 300):
+            shape = binding.attn_shape(batch, gamma, hq, hkv, 128, 128 * tiles)
+            most = max(most, ctx.attention_splits(shape, 128 * tiles), ctx.attention_splits(shape, 128 * tiles, fp8=True))
+            assert ctx.attention_workspace_bytes(shape, 128 * tiles) >= batch * hkv * most * M * (128 + 4) * 4, tiles
+    finally:
+        ctx.close()
+
+
 @pytest.mark.parametrize("kernel", [1, 2])
 def test_splits_without_tiles_after_the_scratch_held_nan(oracle_mod, kernel):
     """A ragged batch leaves the shorter sequences with splits that own no tile; such a
