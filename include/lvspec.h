@@ -155,9 +155,12 @@ int32_t lvspec_attention_splits_fp8(const lvspec_ctx_t *ctx, const lvspec_attn_s
  *       (the largest of the figures above); never shrinks it.
  *   lvspec_workspace_capacity bytes the context holds now.
  *
- * While the context's stream is being captured, a call that would have to grow
- * the buffer returns LVSPEC_ERR_WORKSPACE instead, launches nothing and leaves
- * the capture valid; lvspec_reserve does the same.  The *_host forms also own
+ * An attention call that leaves the split count to the library sizes the buffer by
+ * the same figure, so a step run once can be captured with any lengths up to its
+ * longest.  While the context's stream is being captured, a call that would have to
+ * grow the buffer returns LVSPEC_ERR_WORKSPACE instead, launches nothing and leaves
+ * the capture valid (a batch of different lengths first makes do with the splits of
+ * one CTA per SM); lvspec_reserve does the same.  The *_host forms also own
  * device staging memory for their copies; they synchronise anyway and are not
  * meant for capture. */
 size_t lvspec_attention_workspace_bytes(const lvspec_ctx_t *ctx, const lvspec_attn_shape_t *shape,

@@ -23,6 +23,7 @@ struct lvspec_ctx {
     uint32_t *rel_counters = nullptr; // [LVSPEC_MAX_BATCH * LVSPEC_MAX_GAMMA] candidate counts of the relevance score
     void *scratch = nullptr;          // split partials / argmax partials
     size_t scratch_bytes = 0;
+    bool scratch_in_graph = false;    // a call was captured although two waves would not fit: see run_attention
     void *staging = nullptr;          // device copies for the *_host calls
     size_t staging_bytes = 0;
     uint64_t launches = 0;
@@ -350,11 +351,25 @@ lvspec_status_t run_attention(lvspec_ctx *ctx, const lvspec_attn_shape_t *s, con
     if (k_strides) { p.k_sb = k_strides->batch; p.k_sh = k_strides->head; p.k_sp = k_strides->position; }
     if (v_strides) { p.v_sb = v_strides->batch; p.v_sh = v_strides->head; p.v_sp = v_strides->position; }
 
+    // Scratch is sized for the most splits these lengths could get, alike or not: the first call of
+    // a shape, not the first one whose lengths differ, pays for the growth, and a step run once
+    // can be captured with any lengths.  A capture cannot grow it: two waves then become one where
+    // only one fits, and stay one in later calls (growing would free what the graph uses).
+    auto scratch_for = [&](int n_split) {
+        return attention_scratch_bytes(p.B, p.Hkv, n_split, p.M, p.D, p.gamma, p.Hq, lse2 != nullptr);
+    };
+    size_t want = scratch_for(s->n_split > 0 ? p.n_split : most_splits(ctx, s, max_len));
+    if (want > ctx->scratch_bytes && s->n_split == 0 && (ctx->scratch_in_graph || stream_is_capturing(ctx))) {
+        ctx->scratch_in_graph = true;
+        if (scratch_for(p.n_split) > ctx->scratch_bytes) p.n_split = choose_splits(ctx, s, max_len, fp8 != nullptr);
+        want = scratch_for(p.n_split);
+    }
     const size_t o_bytes = part_o_elems(p) * sizeof(float);
     const size_t st_bytes = part_stat_elems(p) * sizeof(float);
-    lvspec_status_t st = ensure(ctx, &ctx->scratch, &ctx->scratch_bytes,
-                                attention_scratch_bytes(p.B, p.Hkv, p.n_split, p.M, p.D, p.gamma, p.Hq,
-                                                        lse2 != nullptr), false);
+    lvspec_status_t st = ensure(ctx, &ctx->scratch, &ctx->scratch_bytes, want, false);
+    // (no memory for the most: what this call needs may still be had)
+    if (st == LVSPEC_ERR_WORKSPACE && want > scratch_for(p.n_split))
+        st = ensure(ctx, &ctx->scratch, &ctx->scratch_bytes, scratch_for(p.n_split), false);
     if (st != LVSPEC_OK) return st;
     p.part_o = static_cast<float *>(ctx->scratch);
     p.part_stat = reinterpret_cast<float *>(static_cast<char *>(ctx->scratch) + o_bytes);

@@ -154,6 +154,55 @@ def test_the_figure_for_a_length_covers_all_shorter_ones(heads, batch):
         ctx.close()
 
 
+@pytest.mark.parametrize("first", ["equal lengths", "nothing"])
+def test_a_ragged_batch_can_be_captured(oracle_mod, first):
+    """Different lengths may get two waves of CTAs, more partials than a fresh context holds here
+    (9.3 MiB).  Captured after a step of equal lengths they get them; captured first of all, they
+    make do with one wave, and later calls leave the buffer the graph uses alone."""
+    import torch
+    from paper_2604_05650_b200 import binding
+    from gpu_util import dev_bf16, bf16_to_f64, assert_attention_close, run_attention
+    import test_gpu_attention as A
+    ctx = _fresh_ctx()
+    try:
+        B, gamma, Hq, Hkv, L = 16, 8, 72, 8, 4000
+        kv_len = [L] + [300] * 15
+        case = A._case(91, B, gamma, Hq, Hkv, 128, L, kv_len, [[10, n - 20] for n in kv_len])
+        q, k, v, kl, sp = case
+        ref_out, ref_mass = oracle_mod.verify_attention(*case)
+        shape = binding.attn_shape(B, gamma, Hq, Hkv, 128, L)
+        cap = ctx.workspace_capacity()
+        assert ctx.attention_workspace_bytes(shape, L) > cap
+        two = {n: run_attention(ctx, *case, n_split=n)[0] for n in (1, 2)} if first != "nothing" else None
+        dq, dk, dv = dev_bf16(q), dev_bf16(k), dev_bf16(v)
+        out = torch.full(q.shape, float("nan"), dtype=torch.bfloat16, device="cuda")
+        mass = torch.full(q.shape[:3], float("nan"), dtype=torch.float32, device="cuda")
+        if first != "nothing":
+            ctx.close()
+            ctx = _fresh_ctx()
+            ctx.set_stream(torch.cuda.current_stream().cuda_stream)
+            ctx.verify_attention(shape, dq, dk, dv, [L] * B, [[0, 10]] * B, out, mass)
+            torch.cuda.synchronize()
+            cap = ctx.workspace_capacity()
+            assert cap >= ctx.attention_workspace_bytes(shape, L)
+        stream, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            ctx.set_stream(torch.cuda.current_stream().cuda_stream)
+            ctx.verify_attention(shape, dq, dk, dv, kv_len, sp, out, mass)
+        ctx.set_stream(torch.cuda.current_stream().cuda_stream)
+        for _ in range(2):
+            out.fill_(float("nan"))
+            graph.replay()
+            torch.cuda.synchronize()
+            got = bf16_to_f64(out)
+            assert_attention_close(got, mass.cpu().numpy().astype(np.float64), ref_out, ref_mass)
+            assert two is None or ((got == two[2]).all() and (got != two[1]).any())
+            run_attention(ctx, *case)
+            assert ctx.workspace_capacity() == cap and ctx.device_status() == 0
+    finally:
+        ctx.close()
+
+
 @pytest.mark.parametrize("kernel", [1, 2])
 def test_splits_without_tiles_after_the_scratch_held_nan(oracle_mod, kernel):
     """A ragged batch leaves the shorter sequences with splits that own no tile; such a
