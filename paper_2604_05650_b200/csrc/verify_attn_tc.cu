@@ -1253,13 +1253,16 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                 if (grp == 0 && (t_begin + i + n_sub) * kTilePos > L) {
                     // slots at or beyond kv_len hold whatever the cache holds: zero their V
                     // rows so that 0 * junk cannot poison the accumulators (they sit in the last tile)
-                    const int vz = (i + n_sub - 1) % cfg.vs, vr = (i + n_sub - 1) / cfg.vs;
-                    // the slot's tile before is done with (a parity tells this phase from its
-                    // neighbours only, and the products may lag by the depth of the P^T ring)
-                    const int before = i + n_sub - 1 - cfg.vs;
-                    if (before >= 0) mbar_wait(p_free(before), hand_parity(before), abort_flag);
+                    const int last = i + n_sub - 1, vz = last % cfg.vs, vr = last / cfg.vs;
+                    // The slot's tile before is done with.  This group has waited for the products of
+                    // all tiles up to last - pb before it wrote to their P^T buffers; only a V ring shorter
+                    // than the P^T ring may hold a later one.  (A parity tells a phase from its neighbours
+                    // only: the barrier of an older tile may be two phases on, and a wait there would
+                    // not end.)
+                    const int before = last - cfg.vs;
+                    if (cfg.vs < cfg.pb && before >= 0) mbar_wait(p_free(before), hand_parity(before), abort_flag);
                     mbar_wait(v_full(vz), vr & 1, abort_flag);
-                    if ((t_begin + i + n_sub - 1) * kTilePos + row >= L) {
+                    if ((t_begin + last) * kTilePos + row >= L) {
                         uint8_t *vrow = gbase + sm.v + vz * kSlot + row * 128;
 #pragma unroll
                         for (int c = 0; c < 8; ++c) {

@@ -55,6 +55,17 @@ def test_buffer_counts(ctx, oracle_mod, monkeypatch, ring):
         A._check(ctx, oracle_mod, case, n_split=1, kernel=2)
 
 
+@pytest.mark.parametrize("ring", ["2,5,1,2", "2,8,1,2", "2,8,2,4", "3,5,4,4", "2,6,4,4", "2,7,3,3", "4,4,4,4"])
+def test_v_rings_longer_than_the_hand_over_ring(ctx, oracle_mod, monkeypatch, ring):
+    """More V slots than hand-over barriers (they fit at head_dim 64): the slot of the last tile, whose
+    rows beyond kv_len are zeroed, was used by a tile whose barrier may be two phases on."""
+    monkeypatch.setenv("LVSPEC_TC_RING", ring)
+    kv_len = [128 * n + 63 for n in (37, 30, 9, 12)]
+    case = _junk_beyond(A._case(78, 4, 8, 10, 2, 64, 128 * 38, kv_len, [[130, 1100]] * 4), kv_len)
+    A._check(ctx, oracle_mod, case, n_split=1, kernel=2)
+    A._check(ctx, oracle_mod, case, n_split=2, kernel=2)
+
+
 @pytest.mark.parametrize("branch", [(1, 3), (2, 5), (5, 2), (13, 1)])
 def test_draft_ranges(ctx, oracle_mod, branch):
     """Which draft slots a column sees, as a range of columns per slot: trees of several
