@@ -24,12 +24,12 @@
 // pipe, bounded the loop), warps 2-13 = three softmax groups of four warps.
 // The softmax stage has two organisations.  With a bf16 cache all three groups work on
 // every tile, each on a third of the columns (a thread is one cache position, TMEM lane
-// quarter = warp % 4), and tiles go through in pairs: one vote on the guard, one fence and
-// one hand-over to the P.V issuer for 256 positions, while the products of the pair before
-// and the K.Q^T of the next run beside.  (Handed over one by one, a tile costs about 2.1 k
-// cycles of which the exponentials are 0.4 k; in pairs the stream is bound by HBM at 80 rows
-// too: 72B-shaped layer of 32K positions 29.5 us against 30.0, 128K positions x 4 at 80
-// rows 321 us against 331 in turns.)
+// quarter = warp % 4).  Up to 80 rows tiles go through in pairs where the stream is long: one
+// vote on the guard, one fence and one hand-over to the P.V issuer for 256 positions, while the
+// products of the pair before and the K.Q^T of the next run beside.  (Handed over one by one, a
+// tile costs about 2.1 k cycles of which the exponentials are 0.4 k; in pairs a long stream is
+// bound by HBM at 80 rows too: 128K positions x 4, 331 us a layer against 347.  Where the
+// line lies, and the other side of it: pick_config.)
 // With an fp8 cache of up to 64 rows the groups take the tiles in turn (tile i belongs to
 // group i % 3, a thread works through all N columns of its tile), so the latencies of one
 // tile hide behind the exponentials of the two tiles the other groups are
@@ -110,6 +110,7 @@ struct TcConfig {
     int ks, vs, pb;   // K slots, V slots, P buffers
     int sb;           // S^T buffers in TMEM (2 to 4)
     int step;         // tiles handed over at a time (all groups on every tile: 2 where the buffers allow)
+    int pair_from;    // ... in a CTA of at least so many tiles; else one by one
     int tmem_cols;
     int page_slots;   // paged cache: pool pages of this split's tiles, one entry per tile
     int slot_bytes;   // one K or V tile: 32 KB bf16, 16 KB fp8
@@ -436,6 +437,10 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
     const int t_base = n_tiles / p.n_split, t_rem = n_tiles - t_base * p.n_split;
     const int t_begin = split * t_base + min(split, t_rem);
     const int T = t_base + (split < t_rem ? 1 : 0);
+
+    // tiles per hand-over (no test of T where it is 1 anyway: with the widest shares the extra
+    // register costs 1.5 % at 100 rows)
+    const int step = kC == kMaxChunks || T >= cfg.pair_from ? cfg.step : 1;
 
     const size_t unit = ((size_t)b * p.Hkv + kvh) * p.n_split + split;
     float *part_o = p.part_o + unit * (size_t)M * P.a.D;
@@ -831,7 +836,7 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                 LVSPEC_TILE_TS(tile_tr, 2, i, 0);     // starts waiting for P^T
                 // p_full of tile i (two tiles handed over together: on the first one's barrier)
                 bool there = true;
-                if (kTurns || cfg.step == 1 || !(i & 1))
+                if (kTurns || step == 1 || !(i & 1))
                     there = mbar_wait(bar1 + 8 * (2 * kHand + hand.idx), hand.parity, abort_flag);
                 LVSPEC_TILE_TS(tile_tr, 2, i, 1);     // P^T there
                 there = mbar_wait(v_full(vsl), v_ring.parity, abort_flag) && there;
@@ -1111,8 +1116,8 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                 advance(pb, cfg.pb);
             }
         } else {
-            // Tiles go through in twos where the buffers allow (256 positions): one vote on the
-            // guard, one fence and one hand-over for both.
+            // Tiles go through in twos where the buffers allow and the stream is long (256
+            // positions): one vote on the guard, one fence and one hand-over for both.
             // Ring positions advance by counting, not by dividing.
             int sbi = 0, pb = 0;                 // S^T buffer and P buffer of tile i
             const uint64_t neg_scale2 = pack_f32x2(__float_as_uint(-scale), __float_as_uint(-scale));
@@ -1133,8 +1138,8 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                 }
                 group_sync(bar_id);
             }
-            for (int i = 0; i < T; i += cfg.step) {
-                const int n_sub = min(cfg.step, T - i);
+            for (int i = 0; i < T; i += step) {
+                const int n_sub = min(step, T - i);
                 int sb_u, pb_u;
                 for (int attempt = 0; attempt < 3; ++attempt) {
                     // fp8 cache: E4M3 has 17 binades, so the reference exponent of a row starts
@@ -1505,7 +1510,13 @@ TcConfig pick_config(int M, int page_slots, bool fp8, bool turns, int D)
     // Two tiles per hand-over need S^T and P^T buffers for the tiles after them too (with two
     // S^T buffers the K.Q^T of the next pair waits for this one: 112 padded rows, 128-frame
     // tree, 36.8 us a layer in pairs against 34.9 one by one), and a V ring that holds a pair.
+    // In a short stream the first tile's product waits for the second tile to arrive, and
+    // the last pair's products run when nothing else does: us a layer one by one / in pairs,
+    // 40 rows: 2 tiles 10.3 / 10.7, 8 (batch 16) 18.6 / 19.2, 12 22.7 / 23.0, 16 26.7 / 27.3; 56 rows:
+    // 2 tiles 11.1 / 11.3, 7 or 8 19.4 / 19.7; 80 rows: 2 tiles 12.3 / 12.7, 7 or 8 20.2 / 20.0,
+    // several hundred 347 / 331.  Half-size tiles (32 rows): 2 11.9 / 12.0, 4 14.1 / 13.7, 7 18.1 / 17.4.
     c.step = !turns && c.sb >= 4 && c.pb >= 2 && c.vs >= 2 ? 2 : 1;
+    c.pair_from = small_tiles ? 3 : c.n_pad > 64 ? 5 : 17;
     int cols = 32;
     while (cols < (c.sb + acc) * c.n_pad) cols <<= 1;
     c.tmem_cols = cols;

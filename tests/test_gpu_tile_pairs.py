@@ -1,8 +1,9 @@
-"""bf16 cache: tiles go through the softmax stage in pairs where the buffers allow, one by
-one elsewhere.  The sizes at which that can go wrong: odd and even tile counts per CTA, a
-last tile that holds one position, draft slots across a tile boundary, every number of
-column chunks per softmax group, streams long enough for the softmax stage to run ahead of
-the P.V products by all its buffers, junk beyond kv_len."""
+"""bf16 cache: tiles go through the softmax stage in pairs where the buffers allow and a CTA
+has many (from 17 tiles on up to 64 padded rows, from 5 on above, from 3 on at head_dim 64),
+one by one elsewhere.  The sizes at which that can go wrong: odd and even tile counts per CTA
+on both sides, a last tile that holds one position, draft slots across a tile boundary, every
+number of column chunks per softmax group, streams long enough for the softmax stage to run
+ahead of the P.V products by all its buffers, junk beyond kv_len."""
 import numpy as np
 import pytest
 
@@ -31,8 +32,8 @@ def _junk_beyond(case, kv_len):
 
 @pytest.mark.parametrize("rows", [(2, 8, 1), (8, 40, 8), (8, 28, 4), (10, 64, 8), (12, 64, 8), (13, 64, 8), (16, 64, 8)],
                          ids=["16", "40", "56", "80", "96", "104", "128"])
-@pytest.mark.parametrize("tiles", [1, 2, 3, 4, 5, 9])
-def test_tiles_per_cta(ctx, oracle_mod, rows, tiles):
+@pytest.mark.parametrize("tiles", [1, 2, 3, 4, 5, 8, 9, 16, 17])
+def test_tiles_per_cta(ctx, oracle_mod, rows, tiles, head_dim=128):
     gamma, hq, hkv = rows
     hq, hkv = hq // hkv, 1                               # one KV head: the same rows
     lmax = 128 * tiles * 2
@@ -40,9 +41,15 @@ def test_tiles_per_cta(ctx, oracle_mod, rows, tiles):
     kv_len = [128 * (tiles - 1) + 1 + gamma // 2 if tiles > 1 else 128, lmax - 127]
     kv_len = [max(n, gamma) for n in kv_len]
     span = [[0, n - gamma] for n in kv_len]
-    case = _junk_beyond(A._case(900 + tiles, 2, gamma, hq, hkv, 128, lmax, kv_len, span), kv_len)
+    case = _junk_beyond(A._case(900 + tiles, 2, gamma, hq, hkv, head_dim, lmax, kv_len, span), kv_len)
     A._check(ctx, oracle_mod, case, n_split=1, kernel=2)
     A._check(ctx, oracle_mod, case, n_split=2, kernel=2)
+
+
+@pytest.mark.parametrize("rows", [(8, 8, 2), (9, 64, 8)], ids=["32", "72"])
+@pytest.mark.parametrize("tiles", [1, 2, 3, 5])
+def test_tiles_per_cta_at_head_dim_64(ctx, oracle_mod, rows, tiles):
+    test_tiles_per_cta(ctx, oracle_mod, rows, tiles, head_dim=64)
 
 
 @pytest.mark.parametrize("ring", ["2,2,4,4", "2,2,2,4", "2,2,3,3", "2,2,2,2", "2,3,1,2", "1,1,1,2"])
