@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(kThreads) loose_accept_kernel(const AcceptPara
         float4 x[kInFlight];
 #pragma unroll
         for (int u = 0; u < kInFlight; ++u)
-            x[u] = j0 + u * kThreads < n_vec ? __ldg(vec + j0 + u * kThreads)
+            x[u] = j0 + u * kThreads < n_vec ? vec[j0 + u * kThreads]
                                              : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
 #pragma unroll
         for (int u = 0; u < kInFlight; ++u) {

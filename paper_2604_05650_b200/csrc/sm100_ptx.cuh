@@ -162,7 +162,9 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const void *tmap, uint
 
 // ---- programmatic dependent launch -------------------------------------------
 // Blocks until the grids this launch depends on have completed and their
-// writes are visible (returns at once for an ordinary launch).
+// writes are visible (returns at once for an ordinary launch).  What they wrote is read by
+// plain loads: it changes while this grid is resident, which the non-coherent path (__ldg)
+// does not allow.
 __device__ __forceinline__ void grid_dependency_wait()
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");

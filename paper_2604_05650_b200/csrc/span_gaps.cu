@@ -84,8 +84,8 @@ __global__ void __launch_bounds__(kGapThreads) gap_mass_kernel(const GapParams p
                 const int j = j0 + 8 * u;
                 const int pos = j < kGapTile ? pos_s[j] : -1;
                 const uint32_t *src = reinterpret_cast<const uint32_t *>(k_head + (size_t)(pos >= 0 ? pos : 0) * p.D);
-                lo[u] = pos >= 0 ? __ldg(src + lane) : 0u;
-                hi[u] = (pos >= 0 && words > 32) ? __ldg(src + 32 + lane) : 0u;
+                lo[u] = pos >= 0 ? src[lane] : 0u;
+                hi[u] = (pos >= 0 && words > 32) ? src[32 + lane] : 0u;
             }
 #pragma unroll
             for (int u = 0; u < 8; ++u) {

@@ -562,7 +562,7 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
             // this split's entries (one per tile) after the wait, then lane 0 goes on
             grid_dependency_wait();
             const int32_t *row = p.block_table + (size_t)b * p.pages_per_seq;
-            for (int i = lane; i < T; i += 32) page_s[i] = __ldg(row + ((t_begin + i) * kTilePos) / p.page_size);
+            for (int i = lane; i < T; i += 32) page_s[i] = row[((t_begin + i) * kTilePos) / p.page_size];
             __syncwarp();
         }
         if (lane == 0) {
@@ -622,8 +622,8 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                     const int n = ch >> 4, c = ch & 15;
                     if (n < M) {
                         const int g = n / G, hg = n - g * G;
-                        qv[u] = __ldg(reinterpret_cast<const uint4 *>(
-                            p.q + (((size_t)b * gamma + g) * p.Hq + kvh * G + hg) * 128 + c * 8));
+                        qv[u] = *reinterpret_cast<const uint4 *>(
+                            p.q + (((size_t)b * gamma + g) * p.Hq + kvh * G + hg) * 128 + c * 8);
                     }
                     const uint32_t w[4] = {qv[u].x, qv[u].y, qv[u].z, qv[u].w};
 #pragma unroll
@@ -667,8 +667,8 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                         make_uint2(rs[0] | (rs[1] << 16), rs[2] | (rs[3] << 16));
                 }
             }
-            scale_cta = p.scale_log2 * __ldg(p.k_scale + bh) * __uint_as_float((uint32_t)(127 - shift) << 23);
-            v_scale = __ldg(p.v_scale + bh);
+            scale_cta = p.scale_log2 * p.k_scale[bh] * __uint_as_float((uint32_t)(127 - shift) << 23);
+            v_scale = p.v_scale[bh];
         }
         fence_proxy_async_smem();
     }
