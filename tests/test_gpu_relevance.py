@@ -52,7 +52,7 @@ def _rand(seed, B, K, lv, d):
     # B, K, lv, d, top_n
     (1, 4, 300, 256, 10),
     (2, 10, 1000, 512, 10),        # ragged: 1000 = 62 groups of 16 + 8 rows
-    (3, 8, 777, 128, 5),           # chunks cross batch elements
+    (3, 8, 777, 128, 5),           # three batch elements, one group of 16 rows per CTA
     (1, 16, 2100, 64, 1),          # N = 1: the maximum; one stage per chunk
     (1, 17, 500, 192, 100),        # K padded to 32; N = 100
     (2, 1, 5, 64, 10),             # fewer visual tokens than N: plain mean
@@ -62,6 +62,39 @@ def _rand(seed, B, K, lv, d):
 def test_small_shapes(ctx, oracle_mod, shape):
     B, K, lv, d, n = shape
     hd, hv = _rand(31, B, K, lv, d)
+    ref = oracle_mod.visual_relevance(hd, hv, n)
+    got, inv = _run(ctx, hd, hv, n)
+    assert np.isfinite(got).all()
+    assert np.abs(got - ref).max() <= TOL, np.abs(got - ref).max()
+    norms = np.linalg.norm(W.bf16_bits_to_f32(hv).astype(np.float64), axis=-1)
+    assert np.abs(inv * norms - 1.0).max() <= 1e-5
+
+
+@pytest.mark.parametrize("shape", [
+    # B, K, lv, d, top_n
+    (2, 10, 5499, 256, 10),        # 4 or 5 groups per CTA; one CTA has the end of one sequence and the start of the next
+    (3, 17, 5499, 320, 100),       # two seams, K padded to 32, a last stage that is not full
+    (2, 4, 20001, 128, 10),        # 16 or 17 groups: chunks of 16 and of 1 in one CTA, in boxes of different height
+    (5, 8, 10007, 64, 33),         # 21 or 22 groups: chunks of 16 and 5 or 6, cut again at the seams
+    (2, 33, 18950, 192, 7),        # 16 groups for all but a few CTAs, K padded to 48
+])
+def test_shares_across_sequences_and_chunks_of_different_height(ctx, oracle_mod, shape):
+    """A CTA's share of the visual rows may cross from one sequence to the next, and its chunks
+    come in boxes that may be taller than the chunk (the rows read along belong to another
+    CTA, or lie beyond the last row): none of them may reach a score."""
+    import torch
+    B, K, lv, d, n = shape
+    groups = (lv + 15) // 16
+    n_cta = min(torch.cuda.get_device_properties(0).multi_processor_count, B * groups)
+    per, rem = divmod(B * groups, n_cta)
+    starts = {c * per + min(c, rem) for c in range(n_cta)}
+    assert per > 1 and not {b * groups for b in range(1, B)} & starts        # a share crosses every seam
+    hd, hv = _rand(37, B, K, lv, d)
+    # the rows at the seams are the drafts' own: what a draft row must see, and the other
+    # sequence's must not
+    for b in range(B):
+        hv[b, :min(K, 8)] = hd[b, :min(K, 8)]
+        hv[b, lv - min(K, 8):] = hd[(b + 1) % B, :min(K, 8)]
     ref = oracle_mod.visual_relevance(hd, hv, n)
     got, inv = _run(ctx, hd, hv, n)
     assert np.isfinite(got).all()

@@ -1,9 +1,10 @@
 """The tensor-core attention kernel has two organisations of its softmax stage: all
-warp groups on every tile, each on a share of the columns, and the groups taking the
-tiles in turn (chosen by the library from the stream length per CTA and the cache
-format; LVSPEC_TC_TURNS=0/1, read at every launch, forces one).  Both must pass the same
-parity bar, above all where the reference exponents move while other groups are at work
-on later tiles: scores that climb along the cache, tile after tile."""
+warp groups on every tile, each on a share of the columns (a bf16 cache always), and the
+groups taking the tiles in turn (an fp8 cache up to 64 rows, or with a long stream per CTA;
+LVSPEC_TC_TURNS=0/1, read at every launch, forces one with an fp8 cache and means nothing
+with a bf16 one).  All must pass the same parity bar, above all where the reference exponents
+move while other groups are at work on later tiles: scores that climb along the cache, tile
+after tile."""
 import numpy as np
 import pytest
 
@@ -43,7 +44,7 @@ def organisation(request, monkeypatch):
     (1, 16, 16, 2, 900, [897], [[0, 881]], 1),              # 128 rows: two S^T buffers, one P^T buffer
     (3, 4, 8, 2, 640, [640, 130, 385], [[10, 600], [0, 126], [5, 381]], 4),   # splits without tiles
 ])
-def test_shapes(ctx, oracle_mod, organisation, shape):
+def test_shapes(ctx, oracle_mod, shape):
     B, gamma, Hq, Hkv, Lmax, kv_len, span, n_split = shape
     A._check(ctx, oracle_mod, A._case(31, B, gamma, Hq, Hkv, 128, Lmax, kv_len, span), n_split=n_split, kernel=2)
 
@@ -52,13 +53,13 @@ def test_shapes(ctx, oracle_mod, organisation, shape):
     (1, 4, 8, 2, 1024, [1024], [[64, 832]], 0),             # the tiny config's shape
     (2, 8, 16, 4, 2048, [2000, 300], [[100, 1500], [0, 290]], 1),
 ])
-def test_head_dim_64(ctx, oracle_mod, organisation, shape):
+def test_head_dim_64(ctx, oracle_mod, shape):
     B, gamma, Hq, Hkv, Lmax, kv_len, span, n_split = shape
     A._check(ctx, oracle_mod, A._case(36, B, gamma, Hq, Hkv, 64, Lmax, kv_len, span), n_split=n_split, kernel=2)
 
 
 @pytest.mark.parametrize("n_split", [1, 3])
-def test_scores_climbing_tile_after_tile(ctx, oracle_mod, organisation, n_split):
+def test_scores_climbing_tile_after_tile(ctx, oracle_mod, n_split):
     """The score of every row grows by about 80 binades per 128-position tile (more than
     the guard of 60), so every tile moves the reference exponents, while the groups that
     hold the next tiles have already read the old ones; twice the climb pauses for a few
@@ -74,7 +75,7 @@ def test_scores_climbing_tile_after_tile(ctx, oracle_mod, organisation, n_split)
     A._check(ctx, oracle_mod, (q, W.f32_to_bf16_bits(kf), v, kv_len, span), n_split=n_split, kernel=2)
 
 
-def test_junk_beyond_kv_len(ctx, oracle_mod, organisation):
+def test_junk_beyond_kv_len(ctx, oracle_mod):
     case = list(A._case(33, 2, 4, 8, 2, 128, 1024, [900, 385], [[10, 800], [0, 381]]))
     for t in (1, 2):
         case[t][0, :, 900:] = 0x7FC0            # NaN
@@ -82,7 +83,7 @@ def test_junk_beyond_kv_len(ctx, oracle_mod, organisation):
     A._check(ctx, oracle_mod, tuple(case), n_split=1, kernel=2)
 
 
-def test_reproducible_and_split_invariant(ctx, oracle_mod, organisation):
+def test_reproducible_and_split_invariant(ctx, oracle_mod):
     case = A._case(34, 1, 8, 16, 2, 128, 3000, [2990], [[40, 2500]])
     a = A._check(ctx, oracle_mod, case, n_split=1, kernel=2)
     b = A._check(ctx, oracle_mod, case, n_split=1, kernel=2)
@@ -95,12 +96,12 @@ def test_reproducible_and_split_invariant(ctx, oracle_mod, organisation):
     (1, 2, 10, 10, 2, 128, [3000], [[300, 2500]], 1),        # two branches of ten, one CTA per head
     (2, 2, 4, 8, 2, 128, [700, 391], [[10, 500], [0, 380]], 3),
 ])
-def test_tree(ctx, oracle_mod, organisation, shape):
+def test_tree(ctx, oracle_mod, shape):
     TR.test_tree_attention(ctx, oracle_mod, shape, 2)
 
 
 @pytest.mark.parametrize("case", [PG.CASES[1], PG.CASES[3]], ids=["ragged", "one-cta-per-head"])
-def test_paged(ctx, oracle_mod, organisation, case):
+def test_paged(ctx, oracle_mod, case):
     PG.test_paged_matches_oracle_and_contiguous(ctx, oracle_mod, case)
 
 
@@ -114,7 +115,7 @@ def test_fp8_scores_climbing(ctx, oracle_mod, organisation):
     F8.test_scores_climbing_far_above_the_first_tile(ctx, oracle_mod, 1)
 
 
-def test_random_shapes_with_moving_references(ctx, oracle_mod, organisation):
+def test_random_shapes_with_moving_references(ctx, oracle_mod):
     """Seeded random shapes, split counts and lengths; the keys are scaled up so that scores
     spread over a hundred binades and the reference exponents move at unpredictable tiles.
     A few positions then carry a row's whole mass, where nothing averages the rounding of
@@ -146,14 +147,15 @@ def test_random_shapes_with_moving_references(ctx, oracle_mod, organisation):
         assert np.abs(mass - ref_mass).max() <= 2.0 ** -9, (case_id, np.abs(mass - ref_mass).max())
 
 
-@pytest.mark.parametrize("ring", ["2,2,1,2", "2,2,2,2", "3,2,2,3", "1,1,1,2", "2,3,3,3"])
-def test_turns_with_fewer_buffers(ctx, oracle_mod, monkeypatch, ring):
+RINGS = ["2,2,1,2", "2,2,2,2", "3,2,2,3", "1,1,1,2", "2,3,3,3"]
+
+
+@pytest.mark.parametrize("ring", RINGS)
+def test_fewer_buffers(ctx, oracle_mod, monkeypatch, ring):
     """LVSPEC_TC_RING="K slots,V slots,P buffers,S buffers" (read at every launch) forces the
-    buffer counts that large row counts make the library fall back to: groups that share
-    P^T and S^T buffers wait for tiles other groups hold, and the hand-over barriers, indexed
-    by tile, must still tell every phase apart.  One CTA streams 32 tiles, with moving
+    buffer counts that large row counts make the library fall back to: the hand-over barriers,
+    indexed by tile, must still tell every phase apart.  One CTA streams 32 tiles, with moving
     reference exponents in the second case."""
-    monkeypatch.setenv("LVSPEC_TC_TURNS", "1")
     monkeypatch.setenv("LVSPEC_TC_RING", ring)
     A._check(ctx, oracle_mod, A._case(37, 1, 8, 40, 8, 128, 4096, [4001], [[256, 3000]]), n_split=1, kernel=2)
     q, k, v, kv_len, span = A._case(38, 2, 4, 8, 2, 128, 2304, [2304, 700], [[100, 2000], [0, 650]])
@@ -163,3 +165,90 @@ def test_turns_with_fewer_buffers(ctx, oracle_mod, monkeypatch, ring):
     out, mass = run_attention(ctx, q, k, v, kv_len, span, n_split=2, kernel=2)
     assert (np.abs(out - ref_out) <= 1e-2 + 1e-2 * np.abs(ref_out)).all()
     assert np.abs(mass - ref_mass).max() <= 2.0 ** -9
+
+
+# ------------------------------------------------------------------ fp8 cache, both organisations
+def _mass_bound(q, k8, ks, kv_len):
+    """[B, gamma, Hq]: how far the visual mass may be off with an fp8 cache.  A probability is kept
+    as two E4M3 numbers, 2^-9 relative, whose smallest step is 2^-9 where the largest score of the
+    row has at least 2^3: half of that, 2^-13 of the largest probability, may be missing from
+    each position."""
+    import torch
+    B, gamma, Hq, D = q.shape
+    G = Hq // k8.shape[1]
+    kf = torch.from_numpy(k8).view(torch.float8_e4m3fn).to(torch.float64).numpy() * ks[:, :, None, None].astype(np.float64)
+    qf = W.bf16_bits_to_f32(q).astype(np.float64)
+    bound = np.zeros((B, gamma, Hq))
+    for b in range(B):
+        for h in range(Hq):
+            s = qf[b, :, h] @ kf[b, h // G, :kv_len[b]].T / np.sqrt(D)
+            t = np.arange(kv_len[b])[None, :] - (kv_len[b] - gamma)
+            s = np.where(t <= np.arange(gamma)[:, None], s, -np.inf)
+            p = np.exp(s - s.max(1, keepdims=True))
+            bound[b, :, h] = 2.0 ** -9 + np.minimum(p, 2.0 ** -13).sum(1) / p.sum(1)
+    return bound
+
+
+def _check_fp8_moving(ctx, oracle_mod, case, n_split):
+    q, k8, v8, ks, vs, kv_len, span = case
+    ref_out, ref_mass = oracle_mod.verify_attention_fp8(*case)
+    out, mass = F8.run_fp8(ctx, *case, n_split=n_split)
+    assert np.isfinite(out).all() and np.isfinite(mass).all()
+    assert (np.abs(out - ref_out) <= 1e-2 + 1e-2 * np.abs(ref_out)).all()
+    assert (np.abs(mass - ref_mass) <= _mass_bound(q, k8, ks, kv_len)).all()
+
+
+@pytest.mark.parametrize("shape", [
+    # B, gamma, Hq, Hkv, Lmax, kv_len, span, n_split
+    (1, 8, 40, 8, 4096, [4000], [[256, 3000]], 1),          # 32 tiles in one CTA
+    (2, 10, 16, 2, 3072, [3072, 1111], [[100, 2500], [0, 1000]], 2),          # 80 rows: two S^T buffers
+    (1, 16, 12, 3, 1536, [1500], [[64, 1400]], 3),          # 64 rows
+    (3, 4, 8, 2, 640, [640, 130, 385], [[10, 600], [0, 126], [5, 381]], 4),   # splits without tiles
+    (2, 3, 6, 3, 900, [900, 3], [[7, 800], [0, 0]], 1),     # kv_len == gamma
+])
+def test_fp8_shapes(ctx, oracle_mod, organisation, shape):
+    B, gamma, Hq, Hkv, Lmax, kv_len, span, n_split = shape
+    F8._check(ctx, oracle_mod, F8._case(45, B, gamma, Hq, Hkv, Lmax, kv_len, span), n_split=n_split)
+
+
+def test_fp8_junk_beyond_kv_len(ctx, oracle_mod, organisation):
+    case = list(F8._case(33, 2, 4, 8, 2, 1024, [900, 385], [[10, 800], [0, 381]]))
+    for t in (1, 2):
+        case[t][0, :, 900:] = 0x7F            # NaN
+        case[t][1, :, 385:] = 0xFE            # the largest negative value
+    F8._check(ctx, oracle_mod, tuple(case), n_split=1)
+
+
+def test_fp8_reproducible(ctx, oracle_mod, organisation):
+    case = F8._case(34, 1, 8, 16, 2, 3000, [2990], [[40, 2500]])
+    a, b = F8.run_fp8(ctx, *case, n_split=1), F8.run_fp8(ctx, *case, n_split=1)
+    assert (a[0] == b[0]).all() and (a[1] == b[1]).all()
+
+
+def test_fp8_random_shapes_with_moving_references(ctx, oracle_mod, organisation):
+    """As for bf16 above: keys scaled up, so that the reference exponents move while other groups
+    hold later tiles computed under the old ones."""
+    rng = np.random.default_rng(2605)
+    for case_id in range(16):
+        Hkv = int(rng.choice([1, 2, 4]))
+        G = int(rng.choice([1, 2, 5, 8]))
+        gamma = int(rng.integers(1, min(16, 80 // G) + 1))
+        B = int(rng.choice([1, 1, 2, 3]))
+        Lmax = int(rng.integers(3, 30)) * 128 + int(rng.integers(0, 128))
+        kv_len = [int(rng.integers(max(gamma, 130), Lmax + 1)) for _ in range(B)]
+        span = []
+        for L in kv_len:
+            a = int(rng.integers(0, L - gamma + 1))
+            span.append([a, int(rng.integers(a, L - gamma + 1))])
+        n_split, gain = int(rng.choice([0, 1, 1, 2, 3, 7])), float(rng.choice([1.0, 3.0, 8.0]))
+        case = F8._case(1000 + case_id, B, gamma, G * Hkv, Hkv, Lmax, kv_len, span, k_gain=gain)
+        _check_fp8_moving(ctx, oracle_mod, case, n_split)
+
+
+@pytest.mark.parametrize("ring", RINGS)
+def test_fp8_turns_with_fewer_buffers(ctx, oracle_mod, monkeypatch, ring):
+    """Groups that share P^T and S^T buffers wait for tiles other groups hold."""
+    monkeypatch.setenv("LVSPEC_TC_TURNS", "1")
+    monkeypatch.setenv("LVSPEC_TC_RING", ring)
+    F8._check(ctx, oracle_mod, F8._case(37, 1, 8, 40, 8, 4096, [4001], [[256, 3000]]), n_split=1)
+    _check_fp8_moving(ctx, oracle_mod, F8._case(38, 2, 4, 8, 2, 2304, [2304, 700], [[100, 2000], [0, 650]], k_gain=6.0), 2)

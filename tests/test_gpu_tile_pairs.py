@@ -86,26 +86,3 @@ def test_draft_ranges(ctx, oracle_mod, branch):
     for n_split in (1, 3):
         out, mass, _ = TR._run_tree(ctx, case, n_branches, 2, n_split)
         assert_attention_close(out, mass, ref_out, ref_mass)
-
-
-def test_two_waves_of_a_ragged_batch(oracle_mod):
-    """Lengths that differ: the library may cut the sequences for two waves of CTAs; the figure
-    the workspace query returns covers that too."""
-    import torch
-    from gpu_util import run_attention, assert_attention_close
-    from paper_2604_05650_b200 import binding
-    c = binding.Context(0)
-    try:
-        batch, kv_len = 12, [3000 - 230 * b for b in range(12)]
-        case = A._case(61, batch, 2, 8, 8, 128, 3000, kv_len, [[10, n - 50] for n in kv_len])
-        shape = binding.attn_shape(batch, 2, 8, 8, 128, 3000)
-        c.reserve(c.attention_workspace_bytes(shape, 3000))
-        cap = c.workspace_capacity()
-        ref_out, ref_mass = oracle_mod.verify_attention(*case)
-        out, mass = run_attention(c, *case)
-        assert_attention_close(out, mass, ref_out, ref_mass)
-        again, _ = run_attention(c, *case)
-        assert (again == out).all() and c.workspace_capacity() == cap
-        torch.cuda.synchronize()
-    finally:
-        c.close()
