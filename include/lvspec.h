@@ -97,10 +97,13 @@ typedef struct {
  * kernels need (a few MiB, grown on demand by later calls) and zeroes it.
  * Errors: INVALID_ARG (null out pointer, bad ordinal), CUDA (no device or
  * driver), WORKSPACE.
- * The attention kernels of a context are launched "programmatically dependent"
- * on the kernel before them in the stream (their set-up overlaps that kernel's
- * tail; they still wait for it to finish before they read any input).  The
- * environment variable LVSPEC_NO_PDL=1, read here, makes them plain launches. */
+ * The tensor-core attention, its merge, the gap masses of several spans, the
+ * acceptance pass, the branch choice and the row norms are launched
+ * "programmatically dependent" on the kernel before them in the stream (their
+ * set-up overlaps that kernel's tail; they still wait for it to finish before they
+ * read any input).  The environment variable LVSPEC_NO_PDL=1, read here, makes
+ * them plain launches.  The relevance score's kernels are always launched so; the
+ * plain attention kernel and lvspec_loose_accept_static never. */
 lvspec_status_t lvspec_create(lvspec_ctx_t **ctx, int device);
 
 /* Synchronises the context's stream, frees its scratch memory and the context. */

@@ -8,8 +8,9 @@
 //                       rows = two row blocks with one accumulator each;
 //                       S[row, k] = H_V[row, :] . H_D[k, :] on the tensor core
 //                       (tcgen05, MMA M = 128 rows, N = K padded to 16 by the TMA
-//                       unit's zero fill, the hidden dimension in TMA stages of 64
-//                       channels); its otherwise idle epilogue warps take H_D's
+//                       unit's zero fill, the hidden dimension in stages of up to 16
+//                       slabs of 64 channels, one TMA box of H_V and one of H_D a
+//                       stage); its otherwise idle epilogue warps take H_D's
 //                       reciprocal norms meanwhile; then
 //                       cosine = S * inv_norm_v[row] * inv_norm_d[k].
 //                       N <= 32: every warp keeps, per draft token, only the N largest
@@ -700,8 +701,9 @@ cudaError_t launch_visual_relevance(const RelevanceParams &p, cudaStream_t strea
     P.box_a = tail_a > 0 ? tail_a : P.cap;
     P.box_b = tail_b > 0 ? tail_b : P.cap;
     if (P.box_a > P.box_b) { const int t = P.box_a; P.box_a = P.box_b; P.box_b = t; }
-    // Slabs per stage: about 48 KB a stage, so that four are in flight; a row's piece of a stage is then
-    // up to 1 KB in one place (measured: see the file's head).
+    // Slabs per stage: about 48 KB a stage, so that four are in flight; a row's piece of a stage is
+    // then up to 2 KB in one place (25088 rows of 5120: 61.2 us a pass with 48 KB, 64.5 with
+    // 25 KB, 62.5 with 74 KB, 63.3 with 98 KB).
     const int slab_bytes = P.cap * (int)kGroupBytes + NP * 128;
     P.slabs = 49152 / slab_bytes;
     if (P.slabs > 16) P.slabs = 16;

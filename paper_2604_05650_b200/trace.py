@@ -133,9 +133,9 @@ def main() -> None:
         print("tile | K.Q^T issuer: waits for K, K there, S^T free, issued | first softmax warp: see below | P.V issuer: waits"
               " for P^T, there, V there, issued | softmax pass of that warp, per four chunks of columns (tiles in turn"
               " only): asks for S^T, has it, probabilities stored")
-        print("first softmax warp, all groups on every tile (short streams per CTA, bf16 cache): waits for S^T, there,"
-              " exponentials done, group agreed on the guard, P buffer free, P^T handed over")
-        print("first softmax warp, groups take the tiles in turn (it has every third tile; long streams, fp8 cache): waits"
+        print("first softmax warp, all groups on every tile (bf16 cache): waits for S^T, there, P buffer free, probabilities"
+              " stored, group agreed on the guard, P^T handed over (the last two once per hand-over, in the first tile's line)")
+        print("first softmax warp, groups take the tiles in turn (it has every third tile; fp8 cache): waits"
               " for S^T, there, P buffer free, exponentials done, its turn came and m stood, P^T handed over")
         rel = lambda a: " ".join(f"{int(x) - c0:6d}" if x else "     -" for x in a)
         for i in range(32):
