@@ -149,6 +149,13 @@ __device__ __forceinline__ void tma_load_4d_hint(uint32_t dst, const void *tmap,
           "l"(policy)
         : "memory");
 }
+// Asks for a tile to be brought into L2.
+__device__ __forceinline__ void tma_prefetch_4d(const void *tmap, int c0, int c1, int c2, int c3)
+{
+    asm volatile("cp.async.bulk.prefetch.tensor.4d.L2.global.tile [%0, {%1, %2, %3, %4}];"
+                 ::"l"(reinterpret_cast<uint64_t>(tmap)), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
+                 : "memory");
+}
 // 4-D tile load (innermost coordinate first).
 __device__ __forceinline__ void tma_load_4d(uint32_t dst, const void *tmap, uint32_t bar, int c0,
                                             int c1, int c2, int c3)

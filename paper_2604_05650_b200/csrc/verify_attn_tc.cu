@@ -526,6 +526,19 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                              stream_policy);
     };
 
+    // With one K slot (113 rows and more) a K tile can be loaded only when the one before has been
+    // used: it is brought into L2 meanwhile, behind the loads that are needed sooner.  (120 rows of
+    // 32K 39.4 -> 36.7 us a layer, 128 rows 38.9 -> 37.3; V tiles too: 41.2 and 40.1.)
+    auto prefetch_k = [&](int i) {
+        if constexpr (kC == kMaxChunks) {
+            if (cfg.ks > 1 || i >= T) return;
+            int pos0, map_row;
+            tile_at(i, pos0, map_row);
+            tma_prefetch_4d(&tmap_k, 0, pos0, kvh, map_row);
+            if (two_boxes) tma_prefetch_4d(&tmap_k, 64, pos0, kvh, map_row);
+        }
+    };
+
     float scale_cta = p.scale_log2;     // softmax scale of this CTA (fp8 cache: with the K scale and q's shift)
     float v_scale = 1.f;
 
@@ -582,6 +595,7 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                 load_v(i);
             }
             for (int i = max(first_v, 1); i < first_k; ++i) load_k(i);    // a K ring deeper than the V ring
+            prefetch_k(first_k);
         }
         __syncwarp();
     } else if (warp == 1) {
@@ -696,6 +710,7 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                 if (nk < T && mbar_test_wait(k_empty(nk % cfg.ks), ((nk / cfg.ks) - 1) & 1)) {
                     load_k(nk);
                     ++nk;
+                    prefetch_k(nk);
                     progress = true;
                 }
                 if (nv < T && mbar_test_wait(v_empty(nv % cfg.vs), ((nv / cfg.vs) - 1) & 1)) {

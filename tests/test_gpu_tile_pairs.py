@@ -30,8 +30,8 @@ def _junk_beyond(case, kv_len):
     return q, k, v, lens, span
 
 
-@pytest.mark.parametrize("rows", [(2, 8, 1), (8, 40, 8), (8, 28, 4), (10, 64, 8), (12, 64, 8), (13, 64, 8), (16, 64, 8)],
-                         ids=["16", "40", "56", "80", "96", "104", "128"])
+@pytest.mark.parametrize("rows", [(2, 8, 1), (8, 40, 8), (8, 28, 4), (10, 64, 8), (12, 64, 8), (13, 64, 8), (15, 64, 8), (16, 64, 8)],
+                         ids=["16", "40", "56", "80", "96", "104", "120", "128"])
 @pytest.mark.parametrize("tiles", [1, 2, 3, 4, 5, 8, 9, 16, 17])
 def test_tiles_per_cta(ctx, oracle_mod, rows, tiles, head_dim=128):
     gamma, hq, hkv = rows
@@ -46,7 +46,7 @@ def test_tiles_per_cta(ctx, oracle_mod, rows, tiles, head_dim=128):
     A._check(ctx, oracle_mod, case, n_split=2, kernel=2)
 
 
-@pytest.mark.parametrize("rows", [(8, 8, 2), (9, 64, 8)], ids=["32", "72"])
+@pytest.mark.parametrize("rows", [(8, 8, 2), (9, 64, 8), (15, 64, 8), (16, 64, 8)], ids=["32", "72", "120", "128"])
 @pytest.mark.parametrize("tiles", [1, 2, 3, 5])
 def test_tiles_per_cta_at_head_dim_64(ctx, oracle_mod, rows, tiles):
     test_tiles_per_cta(ctx, oracle_mod, rows, tiles, head_dim=64)
