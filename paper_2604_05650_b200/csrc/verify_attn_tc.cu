@@ -475,10 +475,14 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
     auto v_full = [&](int s) { return bar0 + 8 * (2 * cfg.ks + s); };
     auto v_empty = [&](int s) { return bar0 + 8 * (2 * cfg.ks + cfg.vs + s); };
     const uint32_t bar1 = bar0 + 8 * (2 * cfg.ks + 2 * cfg.vs);
-    // The hand-over barriers of tile i are those of index i % 3, whatever the number of
+    // The hand-over barriers of tile i are those of index i % kRound, whatever the number of
     // S^T and P^T buffers: a parity wait tells a phase from its neighbours only, so whoever
-    // waits for a phase must know the phase before it to be over.  Each of these
-    // barriers belongs to the tiles of one softmax group, which sees its phases in order.
+    // waits for a phase must know the phase before it to be over, and the one after it not to
+    // be.  In turns (three barriers) each of them belongs to the tiles of one softmax group,
+    // which sees its phases in order.  With shared columns (four) every group waits for the
+    // product of tile i - pb before it writes tile i, and no product of a tile that is not yet
+    // handed over can end: with pb <= 4 no tile's phase is further than one from what a group
+    // may wait for.
     constexpr int kRound = kTurns ? kSoftmaxGroups : kHand;
     auto s_full = [&](int i) { return bar1 + 8 * (i % kRound); };
     auto s_free = [&](int i) { return bar1 + 8 * (kHand + i % kRound); };
@@ -1024,7 +1028,7 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                     }
 
                     // ---- a score ran past the guard: move m up to the tile maximum ----
-                    // (the masked form, with its divisions, only where the tile reaches the draft slots)
+                    // (the masked form only where the tile reaches the draft slots)
                     auto tile_max = [&](auto masked) {
 #pragma unroll 1
                         for (int c8 = 0; c8 < n8; ++c8) {
@@ -1486,8 +1490,8 @@ TcConfig pick_config(int M, int page_slots, bool fp8, bool turns, int D)
     const int acc = fp8 ? 4 : 2;     // TMEM columns per padded row of O^T and the sums
     if (!turns) {
         // All groups on every tile: as many S^T and P^T buffers as fit, up to two pairs, before
-        // more than two ring slots each.  64 KB of K/V in flight per CTA and die-wide 16 MB
-        // are enough for HBM, and more of them at the start of a launch only put later tiles
+        // more than two ring slots each.  128 KB of K/V in flight per CTA, 16 to 19 MB on the
+        // device, are enough for HBM, and more of them at the start of a launch only put later tiles
         // ahead of the first one's (40 rows, 16 tiles per CTA: 26.9 us with 2 + 2 slots,
         // 27.9 with 3 + 2 or 2 + 3).  At 128 rows a second P^T buffer before a second K slot: 38.3 us
         // a layer of 32K against 47.1.
@@ -1527,7 +1531,7 @@ TcConfig pick_config(int M, int page_slots, bool fp8, bool turns, int D)
     // tree, 36.8 us a layer in pairs against 34.9 one by one), and a V ring that holds a pair.
     // In a short stream the first tile's product waits for the second tile to arrive, and
     // the last pair's products run when nothing else does: us a layer one by one / in pairs,
-    // 40 rows: 2 tiles 10.3 / 10.7, 8 (batch 16) 18.6 / 19.2, 12 22.7 / 23.0, 16 26.7 / 27.3; 56 rows:
+    // 20 rows: 8 tiles (batch 16) 18.6 / 19.2; 40 rows: 2 10.3 / 10.7, 12 22.7 / 23.0, 16 26.7 / 27.3; 56 rows:
     // 2 tiles 11.1 / 11.3, 7 or 8 19.4 / 19.7; 80 rows: 2 tiles 12.3 / 12.7, 7 or 8 20.2 / 20.0,
     // several hundred 347 / 331.  Half-size tiles (32 rows): 2 11.9 / 12.0, 4 14.1 / 13.7, 7 18.1 / 17.4.
     c.step = !turns && c.sb >= 4 && c.pb >= 2 && c.vs >= 2 ? 2 : 1;
