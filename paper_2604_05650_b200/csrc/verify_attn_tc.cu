@@ -1493,12 +1493,13 @@ TcConfig pick_config(int M, int page_slots, bool fp8, bool turns, int D)
         // more than two ring slots each.  128 KB of K/V in flight per CTA, 16 to 19 MB on the
         // device, are enough for HBM, and more of them at the start of a launch only put later tiles
         // ahead of the first one's (40 rows, 16 tiles per CTA: 26.9 us with 2 + 2 slots,
-        // 27.9 with 3 + 2 or 2 + 3).  At 128 rows a second P^T buffer before a second K slot: 38.3 us
+        // 27.9 with 3 + 2 or 2 + 3).  Half-size tiles: 3 + 4 slots and two P^T buffers rather than
+        // 4 + 4 and one (120 rows of 32K at head_dim 64: 33.9 us a layer).  At 128 rows a second P^T buffer before a second K slot: 38.3 us
         // a layer of 32K against 47.1.
         c.sb = 512 / c.n_pad - acc;
         if (c.sb > 4) c.sb = 4;
         const int tries[5][3] = {{2, 2, 4}, {2, 2, 3}, {2, 2, 2}, {1, 2, 2}, {2, 2, 1}};
-        const int tries8[5][3] = {{4, 4, 4}, {4, 4, 3}, {4, 4, 2}, {4, 4, 1}, {3, 3, 1}};
+        const int tries8[5][3] = {{4, 4, 4}, {4, 4, 3}, {4, 4, 2}, {3, 4, 2}, {3, 3, 1}};
         for (int t = 0; t < 5; ++t) {
             const int *tr = small_tiles ? tries8[t] : tries[t];
             c.ks = tr[0]; c.vs = tr[1]; c.pb = tr[2];
