@@ -121,11 +121,15 @@ int resolve_kernel(const lvspec_attn_shape_t *s)
 // heads of 256 tiles.  The count is therefore chosen by a small model of the stream, in
 // units of the time the whole device takes for one tile: the even rounds at the bandwidth
 // their CTA count reaches, the uneven last round at the bandwidth of its few CTAs, and a
-// charge per CTA for writing its partial and merging it.  A pure function of the shape:
-// results stay reproducible from run to run.
+// charge per CTA for writing its partial and merging it, and one for each round of 32 splits
+// of the merge (with one or two KV heads the most CTAs are 74 or 148 splits: a head of 32K at
+// 32 rows takes 13.1 us with 64 splits, 13.8 with 86, 15.4 with 128; two heads of 16K at 4
+// rows 10.7 with 32, 11.5 with 64, 12.6 with 74).  A pure function of the shape: results stay
+// reproducible from run to run.
 struct SplitModel {
     int units, tiles, most;     // (sequence, KV head) pairs; tiles of the longest sequence; splits of one wave
     double saturating;          // CTAs that reach the HBM bandwidth
+    double merge_round;         // a round of the merge: 2 us
     double rate(double ctas) const { return ctas >= saturating ? 1.0 : ctas / saturating; }
 };
 
@@ -144,6 +148,8 @@ SplitModel split_model(const lvspec_ctx *ctx, const lvspec_attn_shape_t *s, int 
     if (fp8 || s->head_dim == 64) share *= 2.1;
     else if (share < 0.8) share = 0.8;
     m.saturating = share * ctx->n_sm;
+    // (several sequences: left out, the choice without it is the better one on average)
+    m.merge_round = s->batch > 1 ? 0.0 : fp8 || s->head_dim == 64 ? 400.0 : 200.0;
     return m;
 }
 
@@ -162,7 +168,7 @@ int choose_splits(const lvspec_ctx *ctx, const lvspec_attn_shape_t *s, int max_k
     for (int ns = m.most; ns >= 1; --ns) {
         const double ctas = (double)ns * m.units;
         const int t_lo = m.tiles / ns, rem = m.tiles - t_lo * ns;
-        double cost = t_lo * ctas / m.rate(ctas) + 0.7 * ctas;
+        double cost = t_lo * ctas / m.rate(ctas) + 0.7 * ctas + m.merge_round * ((ns + 31) / 32);
         if (rem > 0) cost += (double)rem * m.units / m.rate((double)rem * m.units);
         if (ns == m.most || cost < best_cost) {
             best = ns;
