@@ -30,7 +30,7 @@
 // tile costs about 2.1 k cycles of which the exponentials are 0.4 k; in pairs a long stream is
 // bound by HBM at 80 rows too: 128K positions x 4, 331 us a layer against 347.  Where the
 // line lies, and the other side of it: pick_config.)
-// With an fp8 cache of up to 64 rows the groups take the tiles in turn (tile i belongs to
+// With an fp8 cache the groups take the tiles in turn (tile i belongs to
 // group i % 3, a thread works through all N columns of its tile), so the latencies of one
 // tile hide behind the exponentials of the two tiles the other groups are
 // on; S^T has a TMEM buffer per tile in flight.  The reference exponents m[] are
@@ -1511,8 +1511,9 @@ TcConfig pick_config(int M, int page_slots, bool fp8, bool turns, int D)
         // slots delay the first tiles (40 rows, 64 layers of 32K: 25.4 us a layer with 5 + 5,
         // 24.4 with 4 + 4, 23.9 with 3 + 3, 24.7 with 2 + 3).
         c.sb = (kSoftmaxGroups + acc) * c.n_pad <= 512 ? kSoftmaxGroups : 2;
-        const int tries[4][3] = {{3, 3, 3}, {3, 3, 2}, {3, 3, 1}, {2, 2, 1}};
-        for (int t = 0; t < 4; ++t) {
+        // (80 rows: 33.9 us with 2 + 3, 34.2 with 3 + 3)
+        const int tries[5][3] = {{2, 3, 3}, {3, 3, 3}, {3, 3, 2}, {3, 3, 1}, {2, 2, 1}};
+        for (int t = c.n_pad > 64 ? 0 : 1; t < 5; ++t) {
             const int *tr = tries[t];
             c.ks = tr[0]; c.vs = tr[1]; c.pb = tr[2];
             if (smem_map(c).total <= kMaxSmem) break;
@@ -1559,13 +1560,12 @@ cudaError_t launch_attn_tc(const AttnParams &p, const SeqInfo &seq, cudaStream_t
     // paged: one block-table entry per tile of the longest split, rounded up to 4
     const int tiles = (p.Lmax + kTilePos - 1) / kTilePos;
     const bool fp8 = p.fp8 != 0;
-    // Tiles in turn with an fp8 cache of up to 64 padded rows (half the bytes per tile for the
-    // same work: 24.2 us a layer at 40 rows of 32K against 29.0 with shared columns; with more
-    // rows TMEM holds only two S^T buffers and the shared columns win until the stream is
-    // long).  A bf16 cache goes through in pairs of tiles with shared columns, which beats
+    // Tiles in turn with an fp8 cache (half the bytes per tile for the same work: 24.2 us a layer
+    // at 40 rows of 32K against 29.0 with shared columns, 33.9 against 35.3 at 80).  A bf16
+    // cache goes through with shared columns, in pairs of tiles where that pays, which beats
     // turns at every length (long streams of 80 rows: 321 us against 331).
     // LVSPEC_TC_TURNS=0/1 overrides the choice with an fp8 cache (for measurements).
-    bool turns = fp8 && (p.M <= 64 || (tiles + p.n_split - 1) / p.n_split >= 96);
+    bool turns = fp8;
     if (const char *e = fp8 ? std::getenv("LVSPEC_TC_TURNS") : nullptr)
         if (e[0] == '0' || e[0] == '1') turns = e[0] == '1';
     P.cfg = pick_config(p.M, paged ? ((tiles + p.n_split - 1) / p.n_split + 4) & ~3 : 0, fp8, turns, p.D);

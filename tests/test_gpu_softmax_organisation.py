@@ -1,8 +1,7 @@
 """The tensor-core attention kernel has two organisations of its softmax stage: all
 warp groups on every tile, each on a share of the columns (a bf16 cache always), and the
-groups taking the tiles in turn (an fp8 cache up to 64 rows, or with a long stream per CTA;
-LVSPEC_TC_TURNS=0/1, read at every launch, forces one with an fp8 cache and means nothing
-with a bf16 one).  All must pass the same parity bar, above all where the reference exponents
+groups taking the tiles in turn (an fp8 cache; LVSPEC_TC_TURNS=0/1, read at every launch,
+forces one with an fp8 cache and means nothing with a bf16 one).  All must pass the same parity bar, above all where the reference exponents
 move while other groups are at work on later tiles: scores that climb along the cache, tile
 after tile."""
 import numpy as np
