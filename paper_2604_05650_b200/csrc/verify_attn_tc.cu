@@ -1494,8 +1494,9 @@ TcConfig pick_config(int M, int page_slots, bool fp8, bool turns, int D)
         // device, are enough for HBM, and more of them at the start of a launch only put later tiles
         // ahead of the first one's (40 rows, 16 tiles per CTA: 26.9 us with 2 + 2 slots,
         // 27.9 with 3 + 2 or 2 + 3).  Half-size tiles: 3 + 4 slots and two P^T buffers rather than
-        // 4 + 4 and one (120 rows of 32K at head_dim 64: 33.9 us a layer).  At 128 rows a second P^T buffer before a second K slot: 38.3 us
-        // a layer of 32K against 47.1.
+        // 4 + 4 and one (120 rows of 32K at head_dim 64: 33.9 us a layer, 128 rows 43.5 with one
+        // buffer).  At 128 rows a second P^T buffer before a second K slot: 37.3 us a layer of
+        // 32K against 47.1.
         c.sb = 512 / c.n_pad - acc;
         if (c.sb > 4) c.sb = 4;
         const int tries[5][3] = {{2, 2, 4}, {2, 2, 3}, {2, 2, 2}, {1, 2, 2}, {2, 2, 1}};
@@ -1509,9 +1510,9 @@ TcConfig pick_config(int M, int page_slots, bool fp8, bool turns, int D)
         // Tiles in turn (fp8 cache): an S^T buffer per softmax group when TMEM has the columns,
         // else two.  Three 16 KB slots each: a tile is half a bf16 tile's bytes, yet more
         // slots delay the first tiles (40 rows, 64 layers of 32K: 25.4 us a layer with 5 + 5,
-        // 24.4 with 4 + 4, 23.9 with 3 + 3, 24.7 with 2 + 3).
+        // 24.4 with 4 + 4, 23.9 with 3 + 3, 24.7 with 2 + 3).  Above 64 rows a tile takes longer:
+        // 80 rows 33.9 us with 2 + 3, 34.2 with 3 + 3.
         c.sb = (kSoftmaxGroups + acc) * c.n_pad <= 512 ? kSoftmaxGroups : 2;
-        // (80 rows: 33.9 us with 2 + 3, 34.2 with 3 + 3)
         const int tries[5][3] = {{2, 3, 3}, {3, 3, 3}, {3, 3, 2}, {3, 3, 1}, {2, 2, 1}};
         for (int t = c.n_pad > 64 ? 0 : 1; t < 5; ++t) {
             const int *tr = tries[t];
