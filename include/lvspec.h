@@ -29,7 +29,8 @@
  *     synchronising.  The return value reports argument and launch errors only.
  *     A call refused for its arguments (INVALID_ARG, UNSUPPORTED) has launched
  *     nothing.
- *   - A context owns scratch memory on its device and is not thread-safe.
+ *   - A context owns scratch memory on its device (among it a buffer of fixed size, 10 MB,
+ *     through which the attention kernel's CTAs pass their partials on) and is not thread-safe.
  *     Calls on one context must not overlap on the GPU with each other unless
  *     they are ordered on the same stream.
  *   - There is no CPU fallback: without a CUDA device lvspec_create fails.

@@ -27,6 +27,9 @@ struct lvspec_ctx {
     void *staging = nullptr;          // device copies for the *_host calls
     size_t staging_bytes = 0;
     uint64_t launches = 0;
+    void *exchange = nullptr;         // words of the merge inside the attention kernel, then its partials
+    size_t exchange_bytes = 0;
+    uint32_t merge_polls = 128;       // see AttnParams; about 100 us
     bool pdl = true;                  // programmatic dependent launch between the attention kernels
     std::string error;
 };
@@ -310,6 +313,31 @@ struct Fp8Cache {            // E4M3 codes with one scale per (sequence, KV head
     const float *k_scale = nullptr, *v_scale = nullptr;
 };
 
+constexpr size_t kMergeWordBytes = 4096;
+static_assert(kMergeWordBytes >= 8 * 256, "a word per CTA of the widest device");
+
+// Do this call's CTAs merge their splits themselves?  They wait for one another, so all have to run at
+// once: one CTA per SM, one wave.  A share is at most twelve rows (a warp each) and a head has at most 32
+// splits (a bit each); a head of more splits, or of more rows a split, goes to the merge kernel.
+bool merges_itself(const lvspec_ctx *ctx, const AttnParams &p, const SeqInfo &seq)
+{
+    if (p.n_split < 2 || p.n_split > kMergeSplits || p.B * p.Hkv * p.n_split > ctx->n_sm) return false;
+    for (int b = 0; b < p.B; ++b) {
+        const int tiles = (seq.kv_len[b] + 127) / 128;
+        if (p.M > kMergeRows * (tiles < p.n_split ? tiles : p.n_split)) return false;
+    }
+    return true;
+}
+
+// Nothing of the exchange buffer is anybody's: every word of its rows unwritten, no CTA arrived.
+cudaError_t reset_exchange(lvspec_ctx *ctx)
+{
+    cudaError_t e = cudaMemsetAsync(ctx->exchange, 0, kMergeWordBytes, ctx->stream);
+    if (e != cudaSuccess) return e;
+    return cudaMemsetAsync(static_cast<char *>(ctx->exchange) + kMergeWordBytes, 0xFF, ctx->exchange_bytes - kMergeWordBytes,
+                           ctx->stream);
+}
+
 lvspec_status_t run_attention(lvspec_ctx *ctx, const lvspec_attn_shape_t *s, const SeqInfo &seq,
                               int max_len, const void *q, const void *k, const void *v, void *out,
                               float *mass, int branch_len = 0, const PagedCache *paged = nullptr,
@@ -384,9 +412,17 @@ lvspec_status_t run_attention(lvspec_ctx *ctx, const lvspec_attn_shape_t *s, con
         *lse2 = p.lse2;
     }
 
+    const int kernel = resolve_kernel(s);
+    if (kernel == LVSPEC_KERNEL_TCGEN05 && merges_itself(ctx, p, seq)) {
+        p.merge = 1;
+        p.merge_polls = ctx->merge_polls;
+        p.merge_word = static_cast<unsigned long long *>(ctx->exchange);
+        p.part_o = reinterpret_cast<float *>(static_cast<char *>(ctx->exchange) + kMergeWordBytes);
+        p.part_stat = p.part_o + part_o_elems(p);
+    }
+
     int launches = 0;
     cudaError_t e;
-    const int kernel = resolve_kernel(s);
     if (kernel == LVSPEC_KERNEL_TCGEN05) {
         if (!attn_tc_supported(p))
             return fail(ctx, LVSPEC_ERR_UNSUPPORTED,
@@ -400,7 +436,7 @@ lvspec_status_t run_attention(lvspec_ctx *ctx, const lvspec_attn_shape_t *s, con
     ctx->launches += launches;
     if (e != cudaSuccess) return cuda_fail(ctx, "attention kernel launch", e);
     // with a single split the tensor-core kernel writes the results itself
-    if (kernel == LVSPEC_KERNEL_TCGEN05 && p.n_split == 1) return LVSPEC_OK;
+    if (kernel == LVSPEC_KERNEL_TCGEN05 && (p.n_split == 1 || p.merge)) return LVSPEC_OK;
     launches = 0;
     e = launch_attn_combine(p, ctx->stream, &launches);
     ctx->launches += launches;
@@ -535,6 +571,8 @@ lvspec_status_t lvspec_create(lvspec_ctx_t **out, int device)
         return LVSPEC_ERR_UNSUPPORTED;
     }
     ctx->n_sm = prop.multiProcessorCount;
+    // (0: every CTA that has to wait for a partial gives its share up; for tests)
+    if (const char *e = std::getenv("LVSPEC_MERGE_POLLS")) ctx->merge_polls = (uint32_t)std::strtoul(e, nullptr, 10);
     if (const char *e = std::getenv("LVSPEC_NO_PDL")) ctx->pdl = !(e[0] && e[0] != '0');
     const size_t small = sizeof(uint32_t) * (1 + LVSPEC_MAX_BATCH + LVSPEC_MAX_BATCH * LVSPEC_MAX_GAMMA);
     if ((e = cudaMalloc(reinterpret_cast<void **>(&ctx->status), small)) != cudaSuccess ||
@@ -554,6 +592,16 @@ lvspec_status_t lvspec_create(lvspec_ctx_t **out, int device)
         delete ctx;
         return st;
     }
+    ctx->exchange_bytes = kMergeWordBytes + (size_t)ctx->n_sm * LVSPEC_MAX_ROWS * (128 + 4) * sizeof(float);
+    if ((e = cudaMalloc(&ctx->exchange, ctx->exchange_bytes)) != cudaSuccess || (e = reset_exchange(ctx)) != cudaSuccess) {
+        g_create_error = std::string("exchange buffer: ") + cudaGetErrorString(e);
+        cudaFree(ctx->exchange);
+        cudaFree(ctx->scratch);
+        cudaFree(ctx->status);
+        cudaGetLastError();
+        delete ctx;
+        return LVSPEC_ERR_WORKSPACE;
+    }
     cudaDeviceSynchronize();
     *out = ctx;
     return LVSPEC_OK;
@@ -565,6 +613,7 @@ lvspec_status_t lvspec_destroy(lvspec_ctx_t *ctx)
     cudaSetDevice(ctx->device);
     cudaStreamSynchronize(ctx->stream);
     cudaFree(ctx->scratch);
+    cudaFree(ctx->exchange);
     cudaFree(ctx->staging);
     cudaFree(ctx->status);
     delete ctx;
@@ -588,8 +637,11 @@ lvspec_status_t lvspec_device_status(lvspec_ctx_t *ctx, uint32_t *flags)
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
     if (e != cudaSuccess) return cuda_fail(ctx, "reading the device status", e);
     *flags = h;
-    if (h & LVSPEC_DEV_WAIT_EXPIRED)
+    if (h & LVSPEC_DEV_WAIT_EXPIRED) {
+        // an attention call that gave up may have left words behind
+        if ((e = reset_exchange(ctx)) != cudaSuccess) return cuda_fail(ctx, "resetting the exchange buffer", e);
         return fail(ctx, LVSPEC_ERR_TIMEOUT, "a bounded device-side wait ran out");
+    }
     return LVSPEC_OK;
 }
 

@@ -12,7 +12,8 @@
 // records, records of 8 words follow from word 8):
 //   CTA records   {kind (1 attention, 2 merge), q pointer of the call, CTA index,
 //                  %globaltimer at CTA entry, past the prologue / the grid-dependency wait,
-//                  all K.Q^T issued (attention only), end of the CTA's work, unused}
+//                  all K.Q^T issued (attention only), end of the CTA's work or partials
+//                  written, merge inside the attention kernel: this CTA's arrival counted}
 //   tile records  of the one attention CTA (split 3, KV head 2, sequence 0), from word
 //                 8 + 8 * kTraceCtaRecords on: per role r (0 first softmax warp, 1 K.Q^T
 //                 issuer, 2 P.V issuer, 3 inside the first softmax warp's pass), tile i < 32, eight clock64 stamps at
@@ -80,6 +81,12 @@ struct AttnParams {
     float *part_stat;      // [B, Hkv, n_split, M, 4]: m (log2 units), l, l_vis, unused
     float *lse2;           // optional [B, gamma, Hq]: log2 of the softmax denominator, written by the combine
     uint32_t *status;      // device status word
+    // Merge inside the attention kernel (see verify_attn_tc.cu): part_o and part_stat are then in the
+    // context's exchange buffer, every word of which is kNoWord between calls, and merge_word has
+    // one word per (sequence, KV head): CTAs that have arrived, and in the upper half the shares given up
+    unsigned long long *merge_word;
+    uint32_t merge_polls;  // how often a CTA asks for the others' partials before it gives its share up
+    int32_t merge;
     int32_t B, gamma, Hq, Hkv, D, Lmax, G, M, n_split;
     int32_t pdl;           // launch programmatically dependent on the previous kernel
     int32_t branch_len;    // draft tokens per tree branch (= gamma for a plain chain)
@@ -108,6 +115,11 @@ __host__ __device__ inline bool draft_query_sees(int qi, int t, int branch_len)
 {
     return qi >= t && (t < 0 || (qi / branch_len) * branch_len <= t);
 }
+
+// Limits of the merge inside the attention kernel: splits of a head (a bit each in merge_word),
+// rows of a CTA's share (a warp each at most).
+constexpr int kMergeSplits = 32, kMergeRows = 12;
+constexpr uint32_t kNoWord = 0xFFFFFFFFu;    // a word of the exchange buffer nobody has written
 
 // Partial results of one KV split, rows r = g * G + hg.
 static inline size_t part_o_elems(const AttnParams &p)

@@ -380,6 +380,156 @@ __device__ __forceinline__ void softmax_share_bf16(uint32_t s_addr, int n_c, con
         }
     }
 }
+
+// ---- merge of the splits inside the attention kernel ---------------------------------------
+// Where all CTAs of a launch run at once and a head has at most 32 splits, no second kernel merges
+// them: every split's CTA merges an equal share of its head's rows.  Between the end of its stream
+// and its results a CTA then waits for its head's slowest CTA and one trip through L2, where a
+// merge kernel waits for the whole grid to complete (1.7 us), for its own data, and keeps the next
+// layer's launch waiting for a second completion (20 rows of 4K: 10.4 us a layer with the merge
+// kernel, 9.2 so; 40 rows of 32K 26.4 -> 25.3, 80 rows 28.8 -> 27.8, fp8 cache 21.8 -> 20.5).
+// The words themselves say that they have been written: a word of the exchange buffer nobody has
+// written is kNoWord, which no partial is, and whoever has read a word makes it kNoWord again
+// for the next launch.  So there is no fence and no flag between a partial and its reader, whose
+// first request for the data is also its first look whether they are there (statistics first and
+// rows once they are there, a request each: 0.3 us more; a flag behind a fence, 1.5 us more).
+// Nobody waits without end, since the CTAs it waits for may not run (other grids share the GPU):
+// after `merge_polls` requests a CTA gives its share up.  merge_word counts the CTAs of a head
+// whose partials are written, and its upper half has a bit for every share given up; both move in one
+// atomic operation, so either the one who gives up sees that all have arrived (and reads on) or the
+// last to arrive sees the bit, and merges that share itself by the same arithmetic.
+__device__ __forceinline__ bool all_there(const uint4 &x)
+{
+    return x.x != kNoWord && x.y != kNoWord && x.z != kNoWord && x.w != kNoWord;
+}
+// any value but the mark of a word nobody has written (a NaN's payload gives way)
+__device__ __forceinline__ uint32_t passable(float x) { return min(__float_as_uint(x), kNoWord - 1u); }
+
+struct MergedRow {
+    float m, l, lv;      // reference exponent, softmax sum, its part in the visual span
+    float4 o;            // this lane's four channels, over this warp's splits
+};
+// One warp's part of row r of a head whose first split is `unit0`: the splits first, first + step, ...
+// of n.  False when a word is still missing after `polls` requests.  kFlight: rows in flight per
+// lane, no more than there are: this code runs once, on cold instruction caches (twelve instead of
+// four cost 16 rows on 8 splits 0.9 us, eight instead of twelve cost 9 splits a warp 0.7 us).
+template <int kFlight>
+__device__ __forceinline__ bool merge_row(const AttnParams &p, size_t unit0, int r, int n, int first, int step,
+                                          int lane, uint32_t polls, MergedRow &res)
+{
+    const bool active = lane * 4 < p.D;
+    const float *stat = p.part_stat + ((unit0 + lane) * p.M + r) * 4;
+    const float *rows = p.part_o + ((unit0 + first) * p.M + r) * p.D + lane * 4;
+    const size_t stride = (size_t)step * p.M * p.D;
+    const int mine = (n - first + step - 1) / step;      // splits of this warp
+    uint4 st = make_uint4(0, 0, 0, 0), x[kFlight];
+    // statistics and the first rows travel together
+    if (lane < n) st = ld_relaxed_v4(stat);
+    auto fetch = [&](int k0) {
+#pragma unroll
+        for (int k = 0; k < kFlight; ++k)
+            if (active && k0 + k < mine) x[k] = ld_relaxed_v4(rows + (k0 + k) * stride);
+            else x[k] = make_uint4(0, 0, 0, 0);
+    };
+    fetch(0);
+    uint32_t tries = 0;
+    while (!__all_sync(0xffffffffu, all_there(st))) {
+        if (tries++ >= polls) return false;
+        if (!all_there(st)) st = ld_relaxed_v4(stat);
+#pragma unroll
+        for (int k = 0; k < kFlight; ++k)
+            if (!all_there(x[k])) x[k] = ld_relaxed_v4(rows + k * stride);
+    }
+    const float sm = __uint_as_float(st.x), sl = __uint_as_float(st.y), sv = __uint_as_float(st.z);
+    const float m_mine = lane < n && sl > 0.f ? sm : -INFINITY;
+    float m = m_mine;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    const float w = m_mine > -INFINITY ? exp2f(m_mine - m) : 0.f;
+    float l = w * sl, lv = w * sv;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        l += __shfl_xor_sync(0xffffffffu, l, o);
+        lv += __shfl_xor_sync(0xffffffffu, lv, o);
+    }
+    res.m = m; res.l = l; res.lv = lv;
+    res.o = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int k0 = 0; k0 < mine; k0 += kFlight) {
+        if (k0 > 0) fetch(k0);
+        for (;;) {
+            bool ok = true;
+#pragma unroll
+            for (int k = 0; k < kFlight; ++k) ok = ok && all_there(x[k]);
+            if (__all_sync(0xffffffffu, ok)) break;
+            if (tries++ >= polls) return false;
+#pragma unroll
+            for (int k = 0; k < kFlight; ++k)
+                if (!all_there(x[k])) x[k] = ld_relaxed_v4(rows + (k0 + k) * stride);
+        }
+#pragma unroll
+        for (int k = 0; k < kFlight; ++k) {
+            const float wk = __shfl_sync(0xffffffffu, w, (first + (k0 + k) * step) & 31);
+            if (k0 + k < mine && wk != 0.f) {
+                res.o.x = fmaf(wk, __uint_as_float(x[k].x), res.o.x);
+                res.o.y = fmaf(wk, __uint_as_float(x[k].y), res.o.y);
+                res.o.z = fmaf(wk, __uint_as_float(x[k].z), res.o.z);
+                res.o.w = fmaf(wk, __uint_as_float(x[k].w), res.o.w);
+            }
+        }
+    }
+    return true;
+}
+// The same for few registers and any number of rows: a row on all splits, in the order of the warps that
+// would share it (log2 `shift`), for the CTA that sees to shares others have given up.
+__device__ __forceinline__ bool merge_row_alone(const AttnParams &p, size_t unit0, int r, int n, int shift, int lane,
+                                                MergedRow &res)
+{
+    constexpr uint32_t kPolls = 4096;      // (all partials are there; a bound all the same)
+#pragma unroll 1
+    for (int k = 0; k < (1 << shift); ++k) {
+        MergedRow part;
+        if (!merge_row<4>(p, unit0, r, n, k, 1 << shift, lane, kPolls, part)) return false;
+        if (k > 0) {
+            part.o.x += res.o.x; part.o.y += res.o.y; part.o.z += res.o.z; part.o.w += res.o.w;
+        }
+        res = part;
+    }
+    return true;
+}
+// A share's rows [r0, r0 + rows) and log2 of the warps per row.
+struct Share {
+    int r0, rows, shift;
+    __device__ __forceinline__ Share(int split, int n, int M)
+    {
+        r0 = split * M / n;
+        rows = (split + 1) * M / n - r0;
+        shift = rows * 4 <= kSoftmaxWarps ? 2 : rows * 2 <= kSoftmaxWarps ? 1 : 0;
+    }
+};
+// Row r's results.
+__device__ __forceinline__ void write_row(const AttnParams &p, int b, int kvh, int r, int lane, const MergedRow &res)
+{
+    const int g = r / p.G, hg = r - g * p.G;
+    const size_t row = ((size_t)b * p.gamma + g) * p.Hq + kvh * p.G + hg;
+    const float inv = 1.f / res.l;
+    if (lane * 4 < p.D)
+        *reinterpret_cast<uint2 *>(p.out + row * p.D + lane * 4) =
+            make_uint2(pack_bf16x2(res.o.x * inv, res.o.y * inv), pack_bf16x2(res.o.z * inv, res.o.w * inv));
+    if (lane == 0) {
+        p.mass[row] = res.lv * inv;
+        if (p.lse2) p.lse2[row] = res.m + log2f(res.l);
+    }
+}
+// The words of row r that this warp has read are nobody's again.
+__device__ __forceinline__ void clear_row(const AttnParams &p, size_t unit0, int r, int n, int first, int step, int lane,
+                                          bool stats)
+{
+    const uint4 none = make_uint4(kNoWord, kNoWord, kNoWord, kNoWord);
+    if (lane * 4 < p.D)
+        for (int u = first; u < n; u += step) st_relaxed_v4(p.part_o + ((unit0 + u) * p.M + r) * p.D + lane * 4, none);
+    if (stats && lane < n) st_relaxed_v4(p.part_stat + ((unit0 + lane) * p.M + r) * 4, none);
+}
+
 // kFp8: E4M3 cache (tmap_q is not used: q is split into its two E4M3 tiles by the CTA).
 // kTurns: the softmax groups take the tiles in turn (fp8 cache only); otherwise all groups
 // work on every tile, each on a share of its columns, at most kC chunks of eight.
@@ -451,7 +601,7 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
             grid_launch_dependents();
         }
         __syncthreads();
-        for (int r = tid; r < M; r += kThreads)
+        for (int r = tid; !p.merge && r < M; r += kThreads)
             *reinterpret_cast<float4 *>(part_stat + r * 4) = make_float4(kMFloor, 0.f, 0.f, 0.f);
         return;
     }
@@ -1369,11 +1519,11 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                 }
                 if (c8 * 8 + 8 <= m_store) {
 #pragma unroll
-                    for (int k = 0; k < 8; ++k) po[k * D] = o8[k];
+                    for (int k = 0; k < 8; ++k) st_relaxed(po + k * D, passable(o8[k]));
                 } else {
 #pragma unroll
                     for (int k = 0; k < 8; ++k)
-                        if (c8 * 8 + k < m_store) po[k * D] = o8[k];
+                        if (c8 * 8 + k < m_store) st_relaxed(po + k * D, passable(o8[k]));
                 }
             }
             if (wq == 0) {
@@ -1390,14 +1540,65 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                         if (lane == k) { lk = a; lvk = c; }
                     }
                     if (lane < 8 && c8 * 8 + lane < M)
-                        *reinterpret_cast<float4 *>(part_stat + (c8 * 8 + lane) * 4) =
-                            make_float4(m_s[c8 * 8 + lane], lk, lvk, 0.f);
+                        st_relaxed_v4(part_stat + (c8 * 8 + lane) * 4,
+                                      make_uint4(passable(m_s[c8 * 8 + lane]), passable(lk), passable(lvk), 0u));
                 }
             }
         }
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(done_bar);
+
+        if (p.merge) {
+            // ------------------------------------------------------------ merge
+            const int n_eff = min(p.n_split, n_tiles);        // splits with a tile of their own
+            const Share share(split, n_eff, M);
+            const int shift = share.shift, rows = share.rows;
+            const int w = warp - kSoftmaxWarp0, slot = w >> shift, part = w & ((1 << shift) - 1);
+            const int r = share.r0 + slot;
+            const size_t unit0 = unit - split;
+            float4 *sums = reinterpret_cast<float4 *>(gbase + sm.k);   // the rings are empty by now
+            volatile uint32_t *verdict = epoch_s;
+            unsigned long long *word = p.merge_word + bh;
+            bool mine;
+            for (;;) {
+                MergedRow res;
+                const int each = (n_eff + (1 << shift) - 1) >> shift;      // splits of a warp
+                const bool got = slot >= rows ||
+                    (each <= 4 ? merge_row<4>(p, unit0, r, n_eff, part, 1 << shift, lane, p.merge_polls, res)
+                     : each <= 8 ? merge_row<8>(p, unit0, r, n_eff, part, 1 << shift, lane, p.merge_polls, res)
+                                 : merge_row<12>(p, unit0, r, n_eff, part, 1 << shift, lane, p.merge_polls, res));
+                if (part > 0 && slot < rows) sums[w * 32 + lane] = res.o;
+                uint32_t late;
+                asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 q, %2, 0;\n\tbar.red.or.pred p, %1, %3, q;\n\t"
+                             "selp.u32 %0, 1, 0, p;\n\t}"
+                             : "=r"(late) : "r"(kQBarrier), "r"((uint32_t)!got), "n"(kSoftmaxThreads) : "memory");
+                mine = true;
+                if (!late) {
+                    if (part == 0 && slot < rows) {
+                        for (int k = 1; k < (1 << shift); ++k) {
+                            const float4 o = sums[(w + k) * 32 + lane];
+                            res.o.x += o.x; res.o.y += o.y; res.o.z += o.z; res.o.w += o.w;
+                        }
+                        write_row(p, b, kvh, r, lane, res);
+                    }
+                    break;
+                }
+                // Some split's CTA is late, or not even running (the GPU is shared with another grid): this
+                // CTA leaves its share to the head's last one to arrive, unless that one has arrived.
+                if (w == 0 && lane == 0) {
+                    const unsigned long long bit = 1ull << (32 + split);
+                    const uint32_t arrived = (uint32_t)atomicOr(word, bit);
+                    if (arrived == 0) atomicAnd(word, ~bit);      // (all have, and the word is the next call's; or none has yet)
+                    *verdict = arrived == 0 || arrived >= (uint32_t)n_eff ? 1u : 0u;
+                }
+                asm volatile("bar.sync %0, %1;" ::"r"(kQBarrier), "r"(kSoftmaxThreads) : "memory");
+                mine = *verdict != 0;
+                asm volatile("bar.sync %0, %1;" ::"r"(kQBarrier), "r"(kSoftmaxThreads) : "memory");
+                if (!mine) break;
+            }
+            if (mine && slot < rows) clear_row(p, unit0, r, n_eff, part, 1 << shift, lane, part == 0);
+        }
     }
 
     // ------------------------------------------------------------------ teardown
@@ -1415,12 +1616,45 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
             if (*abort_flag || !all_done) atomicOr(p.status, LVSPEC_DEV_WAIT_EXPIRED);
             // this CTA is done but for freeing TMEM: a dependent launch may be scheduled
             // once every CTA has come this far (earlier, its CTAs would pile up on the
-            // few SMs this grid leaves idle)
-            grid_launch_dependents();
+            // few SMs this grid leaves idle; with the merge to come, later still)
+            if (!p.merge) grid_launch_dependents();
         }
         __syncwarp();
         tc_fence_after();
         tmem_dealloc(tmem_base, (uint32_t)cfg.tmem_cols);
+        if (p.merge) {
+            // this CTA's partials are written; the head's last one to say so sees to the shares that
+            // others have given up, and leaves the word as the next call expects it
+            const int n_eff = min(p.n_split, n_tiles);
+            unsigned long long *word = p.merge_word + bh;
+            unsigned long long before = 0;
+            if (lane == 0) {
+                __threadfence();
+                before = atomicAdd(word, 1ull);
+            }
+            before = __shfl_sync(0xffffffffu, before, 0);
+            if ((uint32_t)before == (uint32_t)n_eff - 1u) {
+                const size_t unit0 = unit - split;
+                for (uint32_t late = (uint32_t)(before >> 32); late != 0u; late &= late - 1u) {
+                    const Share share(__ffs(late) - 1, n_eff, M);
+#pragma unroll 1
+                    for (int r = share.r0; r < share.r0 + share.rows; ++r) {
+                        MergedRow res;
+                        if (merge_row_alone(p, unit0, r, n_eff, share.shift, lane, res)) {
+                            write_row(p, b, kvh, r, lane, res);
+                            clear_row(p, unit0, r, n_eff, 0, 1, lane, true);
+                        } else if (lane == 0) {
+                            atomicOr(p.status, LVSPEC_DEV_WAIT_EXPIRED);
+                        }
+                    }
+                }
+                if (lane == 0) atomicExch(word, 0ull);
+            }
+            if (lane == 0) grid_launch_dependents();
+#ifdef LVSPEC_TRACE
+            if (rec) rec[7] = lvspec_trace_now();
+#endif
+        }
     }
 }
 

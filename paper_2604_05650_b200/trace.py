@@ -7,7 +7,8 @@ shipped one; the shipped library carries no trace code), runs a few layers of th
 config's attention from one CUDA graph and prints
 
   * per layer, when its attention and merge CTAs became resident, got past their
-    prologue / dependency wait, issued their last K.Q^T and finished (%globaltimer,
+    prologue / dependency wait, issued their last K.Q^T, had their partials written and,
+    where they merge them themselves, counted their arrival (%globaltimer,
     microseconds from the first stamp; first / median / last CTA), and
   * per tile of one attention CTA, clock64 stamps of the first softmax warp and of the
     two MMA-issuing warps.
@@ -119,7 +120,8 @@ def main() -> None:
         A, C = R[(R[:, 0] == 1) & (lay == l)], R[(R[:, 0] == 2) & (lay == l)]
         if len(A):
             print(f"layer {l} attention ({len(A)} CTAs): resident {three(A[:, 3])} | past the prologue {three(A[:, 4])}"
-                  f" | last K.Q^T done {three(A[:, 5])} | end {three(A[:, 6])}")
+                  f" | last K.Q^T done {three(A[:, 5])} | end {three(A[:, 6])}"
+                  + (f" | merged {three(A[:, 7])}" if A[:, 7].all() else ""))
             late = A[np.argsort(A[:, 6])[-4:]]
             print("        last to finish (split, KV head: end, tiles done at): " + "; ".join(
                 f"{int(r[2]) % 1000}, {int(r[2]) // 1000 % 1000}: {us(r[6])}, {us(r[5])}" for r in late))

@@ -1,0 +1,93 @@
+"""Merge of the splits inside the attention kernel: a head of 2 to 32 splits whose CTAs all run at
+once, at most twelve rows a split.  On both sides of each limit against the oracle; and with
+LVSPEC_MERGE_POLLS=0, where every CTA that would have to wait gives its share to the last one to
+arrive, the same bits."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+# name: (B, Hkv, G, gamma, D, lengths, n_split); a launch merges its splits itself where it holds
+# B * Hkv * n_split <= SMs, n_split <= 32 and rows <= 12 * splits that have a tile
+CASES = {
+    "two-splits": ((1, 2, 2, 3, 128, [700], 2), True),
+    "rows-12-a-split": ((1, 2, 8, 9, 128, [900], 6), True),
+    "rows-13-a-split": ((1, 2, 6, 13, 128, [900], 6), False),
+    "128-rows": ((1, 1, 8, 16, 128, [3000], 11), True),
+    "three-warps-idle": ((1, 1, 5, 1, 128, [2500], 4), True),
+    "more-splits-than-rows": ((1, 2, 1, 3, 64, [4000], 31), True),
+    "32-splits": ((1, 4, 7, 8, 128, [4096 + 17], 32), True),
+    "33-splits": ((1, 2, 5, 4, 128, [4400], 33), False),
+    "splits-without-tiles": ((2, 2, 4, 5, 128, [2500, 300], 18), True),
+    "rows-of-the-shortest": ((2, 2, 5, 8, 128, [2500, 300], 18), False),
+    "head-dim-64": ((1, 2, 4, 4, 64, [1024], 8), True),
+}
+
+
+def _inputs(case, seed):
+    from paper_2604_05650_b200 import workloads as W
+    B, hkv, G, gamma, D, lens, ns = case
+    rng = np.random.default_rng(seed)
+    bf = lambda *s: W.f32_to_bf16_bits(rng.standard_normal(s).astype(np.float32))
+    cap = max(lens) + 5
+    q, k, v = bf(B, gamma, hkv * G, D), bf(B, hkv, cap, D), bf(B, hkv, cap, D)
+    return q, k, v, np.array(lens, np.int32), np.array([[n // 7, n // 2] for n in lens], np.int32), ns
+
+
+def _contexts(monkeypatch, polls=None):
+    from paper_2604_05650_b200 import binding
+    if polls is not None:
+        monkeypatch.setenv("LVSPEC_MERGE_POLLS", str(polls))
+    ctx = binding.Context(0)
+    monkeypatch.delenv("LVSPEC_MERGE_POLLS", raising=False)
+    return ctx
+
+
+@pytest.mark.parametrize("name", CASES)
+def test_both_sides_of_each_limit(name, oracle_mod, monkeypatch):
+    from gpu_util import assert_attention_close, run_attention
+    case, merged = CASES[name]
+    q, k, v, lens, span, ns = _inputs(case, 17)
+    ref = oracle_mod.verify_attention(q, k, v, lens, span)
+    waiting, giving_up = _contexts(monkeypatch), _contexts(monkeypatch, 0)
+    before = waiting.launch_count()
+    first = run_attention(waiting, q, k, v, lens, span, ns)
+    assert waiting.launch_count() - before == (1 if merged else 2)
+    assert_attention_close(*first, *ref)
+    # the exchange buffer is as it was: other shapes and the same one again, on both contexts
+    others = [_inputs(c, 3) for c, m in CASES.values() if m]
+    for ctx in (waiting, giving_up):
+        for _ in range(3):
+            out, mass = run_attention(ctx, q, k, v, lens, span, ns)
+            assert (out == first[0]).all() and (mass == first[1]).all()
+            for o in others[:4]:
+                run_attention(ctx, *o)
+        ctx.close()
+
+
+def test_two_contexts_share_the_gpu(monkeypatch):
+    """Attention calls of two contexts on two streams: grids whose CTAs may get SMs in any order.  (No
+    grid waits for another: a CTA that waits in vain leaves after about 100 us.)"""
+    import torch
+    from gpu_util import dev_bf16
+    from paper_2604_05650_b200 import binding
+    case = (1, 8, 5, 8, 128, [16384], 16)
+    q, k, v, lens, span, ns = _inputs(case, 5)
+    B, hkv, G, gamma, D = case[:5]
+    dq, dk, dv = dev_bf16(q), dev_bf16(k), dev_bf16(v)
+    shape = binding.attn_shape(B, gamma, hkv * G, hkv, D, k.shape[2], ns)
+    streams, ctxs, outs = [torch.cuda.Stream() for _ in range(2)], [], []
+    for s in streams:
+        ctxs.append(_contexts(monkeypatch))
+        ctxs[-1].set_stream(s)
+        outs.append([(torch.empty_like(dq), torch.empty((B, gamma, hkv * G), device="cuda")) for _ in range(40)])
+    torch.cuda.synchronize()
+    for i in range(40):
+        for ctx, o in zip(ctxs, outs):
+            ctx.verify_attention(shape, dq, dk, dv, lens, span, *o[i])
+    torch.cuda.synchronize()
+    for ctx, o in zip(ctxs, outs):
+        assert ctx.device_status() == 0
+        for out, mass in o:
+            assert torch.equal(out, outs[0][0][0]) and torch.equal(mass, outs[0][0][1])
+        ctx.close()
