@@ -133,7 +133,7 @@ __host__ __device__ inline SmemMap smem_map(const TcConfig &c)
     s.dl = o;   o += c.n_pad * 4;
     s.tmx = o;  o += 4 * c.n_pad * 4;
     s.bars = o; o += 8 * (2 * c.ks + 2 * c.vs + 4 * kHand + 4);
-    s.misc = o; o += 16 + 4 * kSoftmaxWarps;     // TMEM address, abort flag, epoch of m, committed tiles, per-warp maxima of |q|
+    s.misc = o; o += 16 + 4 * kSoftmaxWarps + 16;     // TMEM address, abort flag, epoch of m, committed tiles, per-warp maxima of |q|, arrival counted
     s.pages = o; o += 4 * c.page_slots;
     s.total = o;
     return s;
@@ -617,6 +617,7 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
     // how often the reference exponents m[] have been set or moved; tiles handed to the P.V issuer
     volatile uint32_t *epoch_s = reinterpret_cast<volatile uint32_t *>(gbase + sm.misc + 8);
     volatile uint32_t *committed_s = reinterpret_cast<volatile uint32_t *>(gbase + sm.misc + 12);
+    volatile uint32_t *arrived_s = reinterpret_cast<volatile uint32_t *>(gbase + sm.misc + 16 + 4 * kSoftmaxWarps);
 
     // barrier addresses
     const uint32_t bar0 = base + sm.bars;
@@ -719,6 +720,7 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                 *abort_flag = 0;
                 *epoch_s = 0;
                 *committed_s = 0;
+                *arrived_s = 0;
             }
             mbar_fence_init();
             fence_proxy_async_smem();
@@ -1561,6 +1563,7 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
             volatile uint32_t *verdict = epoch_s;
             unsigned long long *word = p.merge_word + bh;
             bool mine;
+            uint64_t since = 0;
             for (;;) {
                 MergedRow res;
                 const int each = (n_eff + (1 << shift) - 1) >> shift;      // splits of a warp
@@ -1586,11 +1589,27 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                 }
                 // Some split's CTA is late, or not even running (the GPU is shared with another grid): this
                 // CTA leaves its share to the head's last one to arrive, unless that one has arrived.
+                // Its own arrival comes first, so that a count of zero can only mean that all have and
+                // the word is the next call's again.
                 if (w == 0 && lane == 0) {
-                    const unsigned long long bit = 1ull << (32 + split);
-                    const uint32_t arrived = (uint32_t)atomicOr(word, bit);
-                    if (arrived == 0) atomicAnd(word, ~bit);      // (all have, and the word is the next call's; or none has yet)
-                    *verdict = arrived == 0 || arrived >= (uint32_t)n_eff ? 1u : 0u;
+                    uint32_t keep = 1u;
+                    if (*arrived_s) {
+                        const unsigned long long bit = 1ull << (32 + split);
+                        const uint32_t arrived = (uint32_t)atomicOr(word, bit);
+                        if (arrived == 0) atomicAnd(word, ~bit);
+                        keep = arrived == 0 || arrived >= (uint32_t)n_eff ? 1u : 0u;
+                    }
+                    if (keep && *abort_flag == 0) {
+                        // (the data are there or on their way: a bound all the same)
+                        const uint64_t now = global_timer_ns();
+                        if (since == 0) since = now;
+                        else if (now - since > 2000000000ull) *abort_flag = 1;
+                    }
+                    if (*abort_flag) {
+                        atomicOr(p.status, LVSPEC_DEV_WAIT_EXPIRED);
+                        keep = 0u;
+                    }
+                    *verdict = keep;
                 }
                 asm volatile("bar.sync %0, %1;" ::"r"(kQBarrier), "r"(kSoftmaxThreads) : "memory");
                 mine = *verdict != 0;
@@ -1631,6 +1650,7 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
             if (lane == 0) {
                 __threadfence();
                 before = atomicAdd(word, 1ull);
+                *arrived_s = 1;
             }
             before = __shfl_sync(0xffffffffu, before, 0);
             if ((uint32_t)before == (uint32_t)n_eff - 1u) {

@@ -108,6 +108,7 @@ def main() -> None:
     print("device status", ctx.device_status(), "| splits", ctx.attention_splits(shape, L),
           "| cache", "E4M3" if args.fp8 else "bf16")
     w = words.cpu().numpy()
+    lib.lvspec_trace_set_buffer(None)        # the buffer goes; kernels launched later must not write to it
     n = min(int(w[0]), CTA_RECORDS)
     R = w[8:8 + n * 8].reshape(n, 8)
     layer_of = {int(q.data_ptr()): i for i, q in enumerate(qs)}
