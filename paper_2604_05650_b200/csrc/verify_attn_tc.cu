@@ -629,12 +629,14 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
     // The hand-over barriers of tile i are those of index i % kRound, whatever the number of
     // S^T and P^T buffers: a parity wait tells a phase from its neighbours only, so whoever
     // waits for a phase must know the phase before it to be over, and the one after it not to
-    // be.  In turns (three barriers) each of them belongs to the tiles of one softmax group,
-    // which sees its phases in order.  With shared columns (four) every group waits for the
-    // product of tile i - pb before it writes tile i, and no product of a tile that is not yet
-    // handed over can end: with pb <= 4 no tile's phase is further than one from what a group
-    // may wait for.
-    constexpr int kRound = kTurns ? kSoftmaxGroups : kHand;
+    // be.  Products end in order, and no product of a tile that is not yet handed over can end.
+    // In turns a group has waited for the product of its tile before, i - 3 - pb, before it comes to
+    // tile i (pb <= 3: every phase it may wait for is the next one of its barrier), and the
+    // K.Q^T of tile i + 4 waits until the group has read tile i (at most four S^T buffers).
+    // With shared columns every group waits for the
+    // product of tile i - pb before it writes tile i: with pb <= 4 no tile's phase is further than
+    // one from what a group may wait for.
+    constexpr int kRound = kHand;
     auto s_full = [&](int i) { return bar1 + 8 * (i % kRound); };
     auto s_free = [&](int i) { return bar1 + 8 * (kHand + i % kRound); };
     auto p_full = [&](int i) { return bar1 + 8 * (2 * kHand + i % kRound); };
@@ -1761,12 +1763,15 @@ TcConfig pick_config(int M, int page_slots, bool fp8, bool turns, int D)
             if (smem_map(c).total <= kMaxSmem) break;
         }
     } else {
-        // Tiles in turn (fp8 cache): an S^T buffer per softmax group when TMEM has the columns,
-        // else two.  Three 16 KB slots each: a tile is half a bf16 tile's bytes, yet more
+        // Tiles in turn (fp8 cache): as many S^T buffers as TMEM has columns for, up to one more than
+        // there are softmax groups: the K.Q^T of a group's next tile is then done when the group
+        // comes to it (40 rows, 64 layers of 32K: 20.4 us a layer with four, 20.6 with three, 20.4 with
+        // five or six).  Three 16 KB slots each: a tile is half a bf16 tile's bytes, yet more
         // slots delay the first tiles (40 rows, 64 layers of 32K: 25.4 us a layer with 5 + 5,
         // 24.4 with 4 + 4, 23.9 with 3 + 3, 24.7 with 2 + 3).  Above 64 rows a tile takes longer:
         // 80 rows 33.9 us with 2 + 3, 34.2 with 3 + 3.
-        c.sb = (kSoftmaxGroups + acc) * c.n_pad <= 512 ? kSoftmaxGroups : 2;
+        c.sb = 512 / c.n_pad - acc;
+        if (c.sb > kHand) c.sb = kHand;
         const int tries[5][3] = {{2, 3, 3}, {3, 3, 3}, {3, 3, 2}, {3, 3, 1}, {2, 2, 1}};
         for (int t = c.n_pad > 64 ? 0 : 1; t < 5; ++t) {
             const int *tr = tries[t];
@@ -1779,7 +1784,7 @@ TcConfig pick_config(int M, int page_slots, bool fp8, bool turns, int D)
     if (const char *e = std::getenv("LVSPEC_TC_RING")) {
         int ks, vs, pb, sb;
         if (std::sscanf(e, "%d,%d,%d,%d", &ks, &vs, &pb, &sb) == 4 && ks >= 1 && ks <= 8 && vs >= 1 && vs <= 8 &&
-            pb >= 1 && sb >= 2 && pb <= (turns ? kSoftmaxGroups : kHand) && sb <= (turns ? kSoftmaxGroups : kHand)) {
+            pb >= 1 && sb >= 2 && pb <= (turns ? kSoftmaxGroups : kHand) && sb <= kHand) {
             c.ks = ks; c.vs = vs; c.pb = pb; c.sb = sb;
         }
     }
