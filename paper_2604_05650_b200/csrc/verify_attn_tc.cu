@@ -112,6 +112,7 @@ struct TcConfig {
     int step;         // tiles handed over at a time (all groups on every tile: 2 where the buffers allow)
     int pair_from;    // ... in a CTA of at least so many tiles; else one by one
     int tmem_cols;
+    uint32_t split_magic, group_magic;   // for divisions by n_split and G
     int page_slots;   // paged cache: pool pages of this split's tiles, one entry per tile
     int slot_bytes;   // one K or V tile: 32 KB bf16, 16 KB fp8
 };
@@ -143,6 +144,16 @@ struct TcParams {
     AttnParams a;
     TcConfig cfg;
 };
+
+// x / d with m = ceil(2^32 / d) from the host (0 for d = 1): the product is off by one at most for
+// x < 2^31.  A plain division is a hundred instructions on a cold instruction cache.
+uint32_t magic_of(uint32_t d) { return d > 1 ? 0xFFFFFFFFu / d + 1u : 0u; }
+__device__ __forceinline__ int div_by(int x, int d, uint32_t m)
+{
+    if (m == 0u) return x;
+    const int q = (int)__umulhi((uint32_t)x, m);
+    return q * d > x ? q - 1 : q;
+}
 
 // Position in a ring of n slots and the parity of the round: the per-tile loops count
 // instead of dividing.
@@ -405,43 +416,58 @@ __device__ __forceinline__ bool all_there(const uint4 &x)
 // any value but the mark of a word nobody has written (a NaN's payload gives way)
 __device__ __forceinline__ uint32_t passable(float x) { return min(__float_as_uint(x), kNoWord - 1u); }
 
+// A row of a head and one warp's part of its merge: the splits first, first + step, ... of n.
+struct MergePart {
+    float *stat, *rows;      // statistics of split `lane`; this lane's four channels of the first split's row
+    size_t stride;           // from one of the part's splits to the next
+    int n, mine, first, step;
+    size_t row;              // of the results
+    __device__ __forceinline__ MergePart(const AttnParams &p, uint32_t group_magic, int b, int kvh, int r, int n_, int first_,
+                                         int step_, int lane)
+        : n(n_), first(first_), step(step_)
+    {
+        const size_t unit0 = ((size_t)b * p.Hkv + kvh) * p.n_split;
+        stat = p.part_stat + ((unit0 + lane) * p.M + r) * 4;
+        rows = p.part_o + ((unit0 + first) * p.M + r) * p.D + lane * 4;
+        stride = (size_t)step * p.M * p.D;
+        mine = step == 4 ? (n - first + 3) >> 2 : step == 2 ? (n - first + 1) >> 1 : n - first;
+        const int g = div_by(r, p.G, group_magic), hg = r - g * p.G;
+        row = ((size_t)b * p.gamma + g) * p.Hq + kvh * p.G + hg;
+    }
+};
 struct MergedRow {
     float m, l, lv;      // reference exponent, softmax sum, its part in the visual span
     float4 o;            // this lane's four channels, over this warp's splits
 };
-// One warp's part of row r of a head whose first split is `unit0`: the splits first, first + step, ...
-// of n.  False when a word is still missing after `polls` requests.  kFlight: rows in flight per
+// False when a word is still missing after `polls` requests.  kFlight: rows in flight per
 // lane, no more than there are: this code runs once, on cold instruction caches (twelve instead of
 // four cost 16 rows on 8 splits 0.9 us, eight instead of twelve cost 9 splits a warp 0.7 us).
 template <int kFlight>
-__device__ __forceinline__ bool merge_row(const AttnParams &p, size_t unit0, int r, int n, int first, int step,
-                                          int lane, uint32_t polls, MergedRow &res)
+__device__ __forceinline__ bool merge_row(const AttnParams &p, const MergePart &t, int lane, uint32_t polls, MergedRow &res)
 {
     const bool active = lane * 4 < p.D;
-    const float *stat = p.part_stat + ((unit0 + lane) * p.M + r) * 4;
-    const float *rows = p.part_o + ((unit0 + first) * p.M + r) * p.D + lane * 4;
-    const size_t stride = (size_t)step * p.M * p.D;
-    const int mine = (n - first + step - 1) / step;      // splits of this warp
     uint4 st = make_uint4(0, 0, 0, 0), x[kFlight];
     // statistics and the first rows travel together
-    if (lane < n) st = ld_relaxed_v4(stat);
-    auto fetch = [&](int k0) {
+    if (lane < t.n) st = ld_relaxed_v4(t.stat);
+    const float *src = t.rows;
+    auto fetch = [&](int n) {
 #pragma unroll
-        for (int k = 0; k < kFlight; ++k)
-            if (active && k0 + k < mine) x[k] = ld_relaxed_v4(rows + (k0 + k) * stride);
-            else x[k] = make_uint4(0, 0, 0, 0);
+        for (int k = 0; k < kFlight; ++k) {
+            x[k] = make_uint4(0, 0, 0, 0);
+            if (active && k < n) x[k] = ld_relaxed_v4(src + k * t.stride);
+        }
     };
-    fetch(0);
+    fetch(t.mine);
     uint32_t tries = 0;
     while (!__all_sync(0xffffffffu, all_there(st))) {
         if (tries++ >= polls) return false;
-        if (!all_there(st)) st = ld_relaxed_v4(stat);
+        if (!all_there(st)) st = ld_relaxed_v4(t.stat);
 #pragma unroll
         for (int k = 0; k < kFlight; ++k)
-            if (!all_there(x[k])) x[k] = ld_relaxed_v4(rows + k * stride);
+            if (!all_there(x[k])) x[k] = ld_relaxed_v4(src + k * t.stride);
     }
     const float sm = __uint_as_float(st.x), sl = __uint_as_float(st.y), sv = __uint_as_float(st.z);
-    const float m_mine = lane < n && sl > 0.f ? sm : -INFINITY;
+    const float m_mine = lane < t.n && sl > 0.f ? sm : -INFINITY;
     float m = m_mine;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
@@ -454,8 +480,9 @@ __device__ __forceinline__ bool merge_row(const AttnParams &p, size_t unit0, int
     }
     res.m = m; res.l = l; res.lv = lv;
     res.o = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int k0 = 0; k0 < mine; k0 += kFlight) {
-        if (k0 > 0) fetch(k0);
+    int u = t.first;
+#pragma unroll 1
+    for (int left = t.mine; left > 0;) {
         for (;;) {
             bool ok = true;
 #pragma unroll
@@ -464,70 +491,57 @@ __device__ __forceinline__ bool merge_row(const AttnParams &p, size_t unit0, int
             if (tries++ >= polls) return false;
 #pragma unroll
             for (int k = 0; k < kFlight; ++k)
-                if (!all_there(x[k])) x[k] = ld_relaxed_v4(rows + (k0 + k) * stride);
+                if (!all_there(x[k])) x[k] = ld_relaxed_v4(src + k * t.stride);
         }
 #pragma unroll
-        for (int k = 0; k < kFlight; ++k) {
-            const float wk = __shfl_sync(0xffffffffu, w, (first + (k0 + k) * step) & 31);
-            if (k0 + k < mine && wk != 0.f) {
+        for (int k = 0; k < kFlight; ++k, u += t.step) {
+            // (a split of weight zero may hold anything, and a place beyond the last split holds zeros)
+            const float wk = __shfl_sync(0xffffffffu, w, u & 31);
+            if (k < left && wk != 0.f) {
                 res.o.x = fmaf(wk, __uint_as_float(x[k].x), res.o.x);
                 res.o.y = fmaf(wk, __uint_as_float(x[k].y), res.o.y);
                 res.o.z = fmaf(wk, __uint_as_float(x[k].z), res.o.z);
                 res.o.w = fmaf(wk, __uint_as_float(x[k].w), res.o.w);
             }
         }
-    }
-    return true;
-}
-// The same for few registers and any number of rows: a row on all splits, in the order of the warps that
-// would share it (log2 `shift`), for the CTA that sees to shares others have given up.
-__device__ __forceinline__ bool merge_row_alone(const AttnParams &p, size_t unit0, int r, int n, int shift, int lane,
-                                                MergedRow &res)
-{
-    constexpr uint32_t kPolls = 4096;      // (all partials are there; a bound all the same)
-#pragma unroll 1
-    for (int k = 0; k < (1 << shift); ++k) {
-        MergedRow part;
-        if (!merge_row<4>(p, unit0, r, n, k, 1 << shift, lane, kPolls, part)) return false;
-        if (k > 0) {
-            part.o.x += res.o.x; part.o.y += res.o.y; part.o.z += res.o.z; part.o.w += res.o.w;
-        }
-        res = part;
+        left -= kFlight;
+        src += kFlight * t.stride;
+        if (left > 0) fetch(left);
     }
     return true;
 }
 // A share's rows [r0, r0 + rows) and log2 of the warps per row.
 struct Share {
     int r0, rows, shift;
-    __device__ __forceinline__ Share(int split, int n, int M)
+    __device__ __forceinline__ Share(const AttnParams &p, uint32_t split_magic, int split, int n)
     {
-        r0 = split * M / n;
-        rows = (split + 1) * M / n - r0;
+        // (fewer splits than asked for, where a sequence has fewer tiles: the plain division)
+        r0 = n == p.n_split ? div_by(split * p.M, n, split_magic) : split * p.M / n;
+        rows = (n == p.n_split ? div_by(split * p.M + p.M, n, split_magic) : (split + 1) * p.M / n) - r0;
         shift = rows * 4 <= kSoftmaxWarps ? 2 : rows * 2 <= kSoftmaxWarps ? 1 : 0;
     }
 };
-// Row r's results.
-__device__ __forceinline__ void write_row(const AttnParams &p, int b, int kvh, int r, int lane, const MergedRow &res)
+// A row's results.
+__device__ __forceinline__ void write_row(const AttnParams &p, const MergePart &t, int lane, const MergedRow &res)
 {
-    const int g = r / p.G, hg = r - g * p.G;
-    const size_t row = ((size_t)b * p.gamma + g) * p.Hq + kvh * p.G + hg;
     const float inv = 1.f / res.l;
     if (lane * 4 < p.D)
-        *reinterpret_cast<uint2 *>(p.out + row * p.D + lane * 4) =
+        *reinterpret_cast<uint2 *>(p.out + t.row * p.D + lane * 4) =
             make_uint2(pack_bf16x2(res.o.x * inv, res.o.y * inv), pack_bf16x2(res.o.z * inv, res.o.w * inv));
     if (lane == 0) {
-        p.mass[row] = res.lv * inv;
-        if (p.lse2) p.lse2[row] = res.m + log2f(res.l);
+        p.mass[t.row] = res.lv * inv;
+        if (p.lse2) p.lse2[t.row] = res.m + log2f(res.l);
     }
 }
-// The words of row r that this warp has read are nobody's again.
-__device__ __forceinline__ void clear_row(const AttnParams &p, size_t unit0, int r, int n, int first, int step, int lane,
-                                          bool stats)
+// The words that this warp has read are nobody's again.
+__device__ __forceinline__ void clear_part(const AttnParams &p, const MergePart &t, int lane)
 {
     const uint4 none = make_uint4(kNoWord, kNoWord, kNoWord, kNoWord);
+    float *dst = t.rows;
     if (lane * 4 < p.D)
-        for (int u = first; u < n; u += step) st_relaxed_v4(p.part_o + ((unit0 + u) * p.M + r) * p.D + lane * 4, none);
-    if (stats && lane < n) st_relaxed_v4(p.part_stat + ((unit0 + lane) * p.M + r) * 4, none);
+#pragma unroll 4
+        for (int k = 0; k < t.mine; ++k, dst += t.stride) st_relaxed_v4(dst, none);
+    if (t.first == 0 && lane < t.n) st_relaxed_v4(t.stat, none);
 }
 
 // kFp8: E4M3 cache (tmap_q is not used: q is split into its two E4M3 tiles by the CTA).
@@ -584,7 +598,7 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
 
     // tiles [t_begin, t_begin + T) of this split: equal shares, sizes differ by at most one
     const int n_tiles = (L + kTilePos - 1) / kTilePos;
-    const int t_base = n_tiles / p.n_split, t_rem = n_tiles - t_base * p.n_split;
+    const int t_base = div_by(n_tiles, p.n_split, P.cfg.split_magic), t_rem = n_tiles - t_base * p.n_split;
     const int t_begin = split * t_base + min(split, t_rem);
     const int T = t_base + (split < t_rem ? 1 : 0);
 
@@ -728,6 +742,9 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
             fence_proxy_async_smem();
         }
         __syncwarp();
+        // The barriers are there: the other warps need not wait for the loads to be asked for (2.4 k cycles
+        // from here to the last one), nor this one for them.
+        asm volatile("bar.arrive 0, %0;" ::"n"(kThreads) : "memory");
         if (paged) {
             // the block table too may come from the kernel before this one: the warp reads
             // this split's entries (one per tile) after the wait, then lane 0 goes on
@@ -844,15 +861,17 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
         }
         fence_proxy_async_smem();
     }
-    // nobody polls a barrier while the grid before this one is still running
-    grid_dependency_wait();
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
+    if (warp != 0) {
+        // nobody polls a barrier while the grid before this one is still running
+        grid_dependency_wait();
+        tc_fence_before();
+        asm volatile("bar.sync 0, %0;" ::"n"(kThreads) : "memory");
+        tc_fence_after();
+    }
 #ifdef LVSPEC_TRACE
     if (rec) rec[4] = lvspec_trace_now();
 #endif
-    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t tmem_base = warp != 0 ? *tmem_slot : 0u;      // (the producer has no use for it)
     // accumulator columns: the S^T buffers, then O^T and the sums (fp8 cache: two columns per row)
     constexpr int kAccCols = kFp8 ? 2 : 1;
     const uint32_t tm_s0 = tmem_base, tm_o = tmem_base + cfg.sb * NP, tm_l = tm_o + kAccCols * NP;
@@ -1469,6 +1488,12 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
 
         // ---------------------------------------------------------------- epilogue
         // (every group takes its share of the columns)
+        // (what the merge needs to know is worked out ahead of the wait for the last product)
+        const int n_eff = min(p.n_split, n_tiles);        // splits with a tile of their own
+        const Share share(p, P.cfg.split_magic, split, n_eff);
+        const int shift = share.shift, rows = share.rows, each = (n_eff + (1 << shift) - 1) >> shift;   // each: splits of a warp
+        const int w = warp - kSoftmaxWarp0, slot = w >> shift, part = w & ((1 << shift) - 1);
+        const MergePart merge_part(p, P.cfg.group_magic, b, kvh, share.r0 + slot, n_eff, part, 1 << shift, lane);
         // the last P.V product has finished (and with it all before)
         mbar_wait(pv_done, 0, abort_flag);
         tc_fence_after();
@@ -1555,12 +1580,6 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
 
         if (p.merge) {
             // ------------------------------------------------------------ merge
-            const int n_eff = min(p.n_split, n_tiles);        // splits with a tile of their own
-            const Share share(split, n_eff, M);
-            const int shift = share.shift, rows = share.rows;
-            const int w = warp - kSoftmaxWarp0, slot = w >> shift, part = w & ((1 << shift) - 1);
-            const int r = share.r0 + slot;
-            const size_t unit0 = unit - split;
             float4 *sums = reinterpret_cast<float4 *>(gbase + sm.k);   // the rings are empty by now
             volatile uint32_t *verdict = epoch_s;
             unsigned long long *word = p.merge_word + bh;
@@ -1568,11 +1587,10 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
             uint64_t since = 0;
             for (;;) {
                 MergedRow res;
-                const int each = (n_eff + (1 << shift) - 1) >> shift;      // splits of a warp
                 const bool got = slot >= rows ||
-                    (each <= 4 ? merge_row<4>(p, unit0, r, n_eff, part, 1 << shift, lane, p.merge_polls, res)
-                     : each <= 8 ? merge_row<8>(p, unit0, r, n_eff, part, 1 << shift, lane, p.merge_polls, res)
-                                 : merge_row<12>(p, unit0, r, n_eff, part, 1 << shift, lane, p.merge_polls, res));
+                    (each <= 4 ? merge_row<4>(p, merge_part, lane, p.merge_polls, res)
+                     : each <= 8 ? merge_row<8>(p, merge_part, lane, p.merge_polls, res)
+                                 : merge_row<12>(p, merge_part, lane, p.merge_polls, res));
                 if (part > 0 && slot < rows) sums[w * 32 + lane] = res.o;
                 uint32_t late;
                 asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 q, %2, 0;\n\tbar.red.or.pred p, %1, %3, q;\n\t"
@@ -1585,7 +1603,7 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                             const float4 o = sums[(w + k) * 32 + lane];
                             res.o.x += o.x; res.o.y += o.y; res.o.z += o.z; res.o.w += o.w;
                         }
-                        write_row(p, b, kvh, r, lane, res);
+                        write_row(p, merge_part, lane, res);
                     }
                     break;
                 }
@@ -1618,7 +1636,7 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                 asm volatile("bar.sync %0, %1;" ::"r"(kQBarrier), "r"(kSoftmaxThreads) : "memory");
                 if (!mine) break;
             }
-            if (mine && slot < rows) clear_row(p, unit0, r, n_eff, part, 1 << shift, lane, part == 0);
+            if (mine && slot < rows) clear_part(p, merge_part, lane);
         }
     }
 
@@ -1656,15 +1674,30 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
             }
             before = __shfl_sync(0xffffffffu, before, 0);
             if ((uint32_t)before == (uint32_t)n_eff - 1u) {
-                const size_t unit0 = unit - split;
+#pragma unroll 1
                 for (uint32_t late = (uint32_t)(before >> 32); late != 0u; late &= late - 1u) {
-                    const Share share(__ffs(late) - 1, n_eff, M);
+                    const Share share(p, P.cfg.split_magic, __ffs(late) - 1, n_eff);
+                    const int parts = 1 << share.shift;
+                    constexpr uint32_t kPolls = 4096;      // (all partials are there; a bound all the same)
 #pragma unroll 1
                     for (int r = share.r0; r < share.r0 + share.rows; ++r) {
+                        // by the same arithmetic, part after part
                         MergedRow res;
-                        if (merge_row_alone(p, unit0, r, n_eff, share.shift, lane, res)) {
-                            write_row(p, b, kvh, r, lane, res);
-                            clear_row(p, unit0, r, n_eff, 0, 1, lane, true);
+                        bool ok = true;
+#pragma unroll 1
+                        for (int k = 0; k < parts && ok; ++k) {
+                            MergedRow of_part;
+                            ok = merge_row<4>(p, MergePart(p, P.cfg.group_magic, b, kvh, r, n_eff, k, parts, lane), lane, kPolls,
+                                              of_part);
+                            if (k > 0) {
+                                of_part.o.x += res.o.x; of_part.o.y += res.o.y; of_part.o.z += res.o.z; of_part.o.w += res.o.w;
+                            }
+                            res = of_part;
+                        }
+                        const MergePart whole(p, P.cfg.group_magic, b, kvh, r, n_eff, 0, 1, lane);
+                        if (ok) {
+                            write_row(p, whole, lane, res);
+                            clear_part(p, whole, lane);
                         } else if (lane == 0) {
                             atomicOr(p.status, LVSPEC_DEV_WAIT_EXPIRED);
                         }
@@ -1829,6 +1862,8 @@ cudaError_t launch_attn_tc(const AttnParams &p, const SeqInfo &seq, cudaStream_t
     if (const char *e = fp8 ? std::getenv("LVSPEC_TC_TURNS") : nullptr)
         if (e[0] == '0' || e[0] == '1') turns = e[0] == '1';
     P.cfg = pick_config(p.M, paged ? ((tiles + p.n_split - 1) / p.n_split + 4) & ~3 : 0, fp8, turns, p.D);
+    P.cfg.split_magic = magic_of((uint32_t)p.n_split);
+    P.cfg.group_magic = magic_of((uint32_t)p.G);
     if (smem_map(P.cfg).total > kMaxSmem || P.cfg.tmem_cols > 512) return cudaErrorInvalidConfiguration;
     CUtensorMap mk, mv, mq;
     const int map_len = paged ? p.page_size : p.Lmax;
