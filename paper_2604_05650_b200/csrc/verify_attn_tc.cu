@@ -121,7 +121,7 @@ struct TcConfig {
 struct SmemMap {
     uint32_t k, v, q, p, a2, m, dl, tmx, bars, misc, pages, total;
 };
-__host__ __device__ inline SmemMap smem_map(const TcConfig &c)
+inline SmemMap smem_map(const TcConfig &c)
 {
     SmemMap s;
     uint32_t o = 0;
@@ -141,8 +141,9 @@ __host__ __device__ inline SmemMap smem_map(const TcConfig &c)
 }
 
 struct TcParams {
-    AttnParams a;
     TcConfig cfg;
+    SmemMap sm;     // worked out on the host: in the kernel it was thirty instructions of the cold start
+    AttnParams a;
 };
 
 // x / d with m = ceil(2^32 / d) from the host (0 for d = 1): the product is off by one at most for
@@ -563,7 +564,7 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
     const bool paged = P.a.page_size > 0;
     extern __shared__ uint8_t smem_raw[];
     const AttnParams &p = P.a;
-    const TcConfig cfg = P.cfg;
+    const TcConfig &cfg = P.cfg;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 #ifdef LVSPEC_TRACE
     unsigned long long *rec = nullptr;      // this CTA's record (one thread writes it)
@@ -622,7 +623,7 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
 
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t *gbase = smem_raw + (base - smem_u32(smem_raw));
-    const SmemMap sm = smem_map(cfg);
+    const SmemMap &sm = P.sm;
     float *m_s = reinterpret_cast<float *>(gbase + sm.m);
     float *dl_s = reinterpret_cast<float *>(gbase + sm.dl);
     float *tmx_s = reinterpret_cast<float *>(gbase + sm.tmx);
@@ -738,7 +739,6 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                 *committed_s = 0;
                 *arrived_s = 0;
             }
-            mbar_fence_init();
             fence_proxy_async_smem();
         }
         __syncwarp();
@@ -1865,6 +1865,7 @@ cudaError_t launch_attn_tc(const AttnParams &p, const SeqInfo &seq, cudaStream_t
     P.cfg.split_magic = magic_of((uint32_t)p.n_split);
     P.cfg.group_magic = magic_of((uint32_t)p.G);
     if (smem_map(P.cfg).total > kMaxSmem || P.cfg.tmem_cols > 512) return cudaErrorInvalidConfiguration;
+    P.sm = smem_map(P.cfg);
     CUtensorMap mk, mv, mq;
     const int map_len = paged ? p.page_size : p.Lmax;
     const int map_outer = paged ? p.n_pages : p.B;
