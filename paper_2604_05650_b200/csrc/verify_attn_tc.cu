@@ -399,7 +399,7 @@ __device__ __forceinline__ void softmax_share_bf16(uint32_t s_addr, int n_c, con
 // and its results a CTA then waits for its head's slowest CTA and one trip through L2, where a
 // merge kernel waits for the whole grid to complete (1.7 us), for its own data, and keeps the next
 // layer's launch waiting for a second completion (20 rows of 4K: 10.4 us a layer with the merge
-// kernel, 9.2 so; 40 rows of 32K 26.4 -> 25.3, 80 rows 28.8 -> 27.8, fp8 cache 21.8 -> 20.5).
+// kernel, 8.9 so; 40 rows of 32K 26.4 -> 25.5, 80 rows 28.8 -> 28.0, fp8 cache 21.8 -> 20.6).
 // The words themselves say that they have been written: a word of the exchange buffer nobody has
 // written is kNoWord, which no partial is, and whoever has read a word makes it kNoWord again
 // for the next launch.  So there is no fence and no flag between a partial and its reader, whose
@@ -645,8 +645,8 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
     // S^T and P^T buffers: a parity wait tells a phase from its neighbours only, so whoever
     // waits for a phase must know the phase before it to be over, and the one after it not to
     // be.  Products end in order, and no product of a tile that is not yet handed over can end.
-    // In turns a group has waited for the product of its tile before, i - 3 - pb, before it comes to
-    // tile i (pb <= 3: every phase it may wait for is the next one of its barrier), and the
+    // In turns a group has waited for the product of tile i - 3 - pb before it comes to tile i, and so
+    // for all before it (pb <= 4: every phase it may wait for is the next one of its barrier), and the
     // K.Q^T of tile i + 4 waits until the group has read tile i (at most four S^T buffers).
     // With shared columns every group waits for the
     // product of tile i - pb before it writes tile i: with pb <= 4 no tile's phase is further than
@@ -1799,14 +1799,15 @@ TcConfig pick_config(int M, int page_slots, bool fp8, bool turns, int D)
         // Tiles in turn (fp8 cache): as many S^T buffers as TMEM has columns for, up to one more than
         // there are softmax groups: the K.Q^T of a group's next tile is then done when the group
         // comes to it (40 rows, 64 layers of 32K: 20.4 us a layer with four, 20.6 with three, 20.4 with
-        // five or six).  Three 16 KB slots each: a tile is half a bf16 tile's bytes, yet more
-        // slots delay the first tiles (40 rows, 64 layers of 32K: 25.4 us a layer with 5 + 5,
-        // 24.4 with 4 + 4, 23.9 with 3 + 3, 24.7 with 2 + 3).  Above 64 rows a tile takes longer:
-        // 80 rows 33.9 us with 2 + 3, 34.2 with 3 + 3.
+        // five or six).  A fourth P^T buffer too: with three a group waited for the product of its tile
+        // before, which is in the queue behind two others'.  Then also more slots of 16 KB (us a layer of 32K, 40 rows:
+        // 19.8 with 3 + 3 slots and three P^T buffers, 19.5 with 3 + 3 and four, 19.1 with 4 + 4, 19.3 with 5 + 4;
+        // 56 rows of 64K: 25.6, 24.8, 25.1; 80 rows: 33.3 with 2 + 3 and three, 33.6 with 3 + 3, 33.4 with a fourth P^T
+        // buffer, 33.8 with more slots).
         c.sb = 512 / c.n_pad - acc;
         if (c.sb > kHand) c.sb = kHand;
-        const int tries[5][3] = {{2, 3, 3}, {3, 3, 3}, {3, 3, 2}, {3, 3, 1}, {2, 2, 1}};
-        for (int t = c.n_pad > 64 ? 0 : 1; t < 5; ++t) {
+        const int tries[6][3] = {{4, 4, 4}, {3, 3, 4}, {2, 3, 3}, {3, 3, 2}, {3, 3, 1}, {2, 2, 1}};
+        for (int t = c.n_pad > 64 ? 2 : c.n_pad > 48 ? 1 : 0; t < 6; ++t) {
             const int *tr = tries[t];
             c.ks = tr[0]; c.vs = tr[1]; c.pb = tr[2];
             if (smem_map(c).total <= kMaxSmem) break;
@@ -1817,7 +1818,7 @@ TcConfig pick_config(int M, int page_slots, bool fp8, bool turns, int D)
     if (const char *e = std::getenv("LVSPEC_TC_RING")) {
         int ks, vs, pb, sb;
         if (std::sscanf(e, "%d,%d,%d,%d", &ks, &vs, &pb, &sb) == 4 && ks >= 1 && ks <= 8 && vs >= 1 && vs <= 8 &&
-            pb >= 1 && sb >= 2 && pb <= (turns ? kSoftmaxGroups : kHand) && sb <= kHand) {
+            pb >= 1 && sb >= 2 && pb <= kHand && sb <= kHand) {
             c.ks = ks; c.vs = vs; c.pb = pb; c.sb = sb;
         }
     }

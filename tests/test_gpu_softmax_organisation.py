@@ -251,3 +251,10 @@ def test_fp8_turns_with_fewer_buffers(ctx, oracle_mod, monkeypatch, ring):
     monkeypatch.setenv("LVSPEC_TC_RING", ring)
     F8._check(ctx, oracle_mod, F8._case(37, 1, 8, 40, 8, 4096, [4001], [[256, 3000]]), n_split=1)
     _check_fp8_moving(ctx, oracle_mod, F8._case(38, 2, 4, 8, 2, 2304, [2304, 700], [[100, 2000], [0, 650]], k_gain=6.0), 2)
+
+
+@pytest.mark.parametrize("rows", [20, 50, 55, 65])
+def test_fp8_rings_wrap(ctx, oracle_mod, rows):
+    """Tiles in turn with the buffer counts of each range of padded rows (32, 64, 64, 80), in
+    streams of 19 and 6 tiles: every ring and every hand-over barrier goes round several times."""
+    F8._check(ctx, oracle_mod, F8._case(36, 2, rows // 5, 10, 2, 2560, [2400, 700], [[128, 2000], [0, 500]]), n_split=1)
