@@ -574,9 +574,14 @@ lvspec_status_t lvspec_create(lvspec_ctx_t **out, int device)
     // (0: every CTA that has to wait for a partial gives its share up; for tests)
     if (const char *e = std::getenv("LVSPEC_MERGE_POLLS")) ctx->merge_polls = (uint32_t)std::strtoul(e, nullptr, 10);
     if (const char *e = std::getenv("LVSPEC_NO_PDL")) ctx->pdl = !(e[0] && e[0] != '0');
-    const size_t small = sizeof(uint32_t) * (1 + LVSPEC_MAX_BATCH + LVSPEC_MAX_BATCH * LVSPEC_MAX_GAMMA);
-    if ((e = cudaMalloc(reinterpret_cast<void **>(&ctx->status), small)) != cudaSuccess ||
-        (e = cudaMemset(ctx->status, 0, small)) != cudaSuccess) {
+    // status word and counters, then the exchange buffer, in one allocation
+    const size_t counted = sizeof(uint32_t) * (1 + LVSPEC_MAX_BATCH + LVSPEC_MAX_BATCH * LVSPEC_MAX_GAMMA);
+    const size_t small = (counted + 255) & ~size_t(255);
+    ctx->exchange_bytes = kMergeWordBytes + (size_t)ctx->n_sm * LVSPEC_MAX_ROWS * (128 + 4) * sizeof(float);
+    if ((e = cudaMalloc(reinterpret_cast<void **>(&ctx->status), small + ctx->exchange_bytes)) == cudaSuccess)
+        ctx->exchange = reinterpret_cast<char *>(ctx->status) + small;
+    if (e != cudaSuccess || (e = cudaMemset(ctx->status, 0, small)) != cudaSuccess ||
+        (e = reset_exchange(ctx)) != cudaSuccess) {
         g_create_error = std::string("status allocation: ") + cudaGetErrorString(e);
         cudaFree(ctx->status);      // null when the allocation itself failed
         cudaGetLastError();
@@ -592,16 +597,6 @@ lvspec_status_t lvspec_create(lvspec_ctx_t **out, int device)
         delete ctx;
         return st;
     }
-    ctx->exchange_bytes = kMergeWordBytes + (size_t)ctx->n_sm * LVSPEC_MAX_ROWS * (128 + 4) * sizeof(float);
-    if ((e = cudaMalloc(&ctx->exchange, ctx->exchange_bytes)) != cudaSuccess || (e = reset_exchange(ctx)) != cudaSuccess) {
-        g_create_error = std::string("exchange buffer: ") + cudaGetErrorString(e);
-        cudaFree(ctx->exchange);
-        cudaFree(ctx->scratch);
-        cudaFree(ctx->status);
-        cudaGetLastError();
-        delete ctx;
-        return LVSPEC_ERR_WORKSPACE;
-    }
     cudaDeviceSynchronize();
     *out = ctx;
     return LVSPEC_OK;
@@ -613,7 +608,6 @@ lvspec_status_t lvspec_destroy(lvspec_ctx_t *ctx)
     cudaSetDevice(ctx->device);
     cudaStreamSynchronize(ctx->stream);
     cudaFree(ctx->scratch);
-    cudaFree(ctx->exchange);
     cudaFree(ctx->staging);
     cudaFree(ctx->status);
     delete ctx;
