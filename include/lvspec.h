@@ -103,7 +103,9 @@ typedef struct {
  * "programmatically dependent" on the kernel before them in the stream (their
  * set-up overlaps that kernel's tail; they still wait for it to finish before they
  * read any input).  The environment variable LVSPEC_NO_PDL=1, read here, makes
- * them plain launches.  The relevance score's kernels are always launched so; the
+ * them plain launches; LVSPEC_MERGE_POLLS=n, read here too, is how often an attention CTA
+ * asks for the partials of its head's other CTAs before it leaves its rows to the last of them
+ * (128; 0 for tests).  The relevance score's kernels are always launched so; the
  * plain attention kernel and lvspec_loose_accept_static never. */
 lvspec_status_t lvspec_create(lvspec_ctx_t **ctx, int device);
 
