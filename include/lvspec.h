@@ -56,7 +56,7 @@ typedef enum {
 } lvspec_status_t;
 
 /* Bits of the device status word (lvspec_device_status). */
-#define LVSPEC_DEV_WAIT_EXPIRED 0x1u /* a bounded barrier wait gave up; results invalid */
+#define LVSPEC_DEV_WAIT_EXPIRED 0x1u /* a bounded wait gave up; that call's results are invalid */
 #define LVSPEC_DEV_NAN_LOGIT    0x2u /* a NaN logit was seen (it was ranked as -inf) */
 
 #define LVSPEC_MAX_BATCH 128   /* sequences per call */
@@ -118,7 +118,10 @@ lvspec_status_t lvspec_set_stream(lvspec_ctx_t *ctx, void *cuda_stream);
 
 /* Synchronises the stream, reads and clears the device status word.
  * `flags` (host) receives the LVSPEC_DEV_* bits.  Returns LVSPEC_ERR_TIMEOUT if
- * LVSPEC_DEV_WAIT_EXPIRED is set, LVSPEC_ERR_CUDA if the sync failed. */
+ * LVSPEC_DEV_WAIT_EXPIRED is set, LVSPEC_ERR_CUDA if the sync failed.  After an
+ * expired wait later calls are right, but until this call has reported it the
+ * attention merges its splits the slow way (the buffer they pass through is not
+ * trusted; this call puts it in order). */
 lvspec_status_t lvspec_device_status(lvspec_ctx_t *ctx, uint32_t *flags);
 /* The same call under the name "last device status": what the kernels launched
  * since the previous reading have reported. */
@@ -183,7 +186,8 @@ lvspec_status_t lvspec_reserve(lvspec_ctx_t *ctx, size_t workspace_bytes);
  * raises LVSPEC_DEV_WAIT_EXPIRED and lets the kernel return, so that a lost
  * arrival cannot hang the GPU.  This call enqueues one warp that waits, through
  * the same code but with a limit of `limit_ms` milliseconds (1..2000), on a
- * barrier nothing ever completes.  Afterwards lvspec_device_status reports
+ * barrier nothing ever completes, and leaves the buffer of the splits' partials as
+ * an attention call that gave up may leave it.  Afterwards lvspec_device_status reports
  * LVSPEC_ERR_TIMEOUT once, and the context is as usable as before. */
 lvspec_status_t lvspec_selftest_wait_expiry(lvspec_ctx_t *ctx, int32_t limit_ms);
 

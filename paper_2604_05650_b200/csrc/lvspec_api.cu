@@ -988,6 +988,10 @@ lvspec_status_t lvspec_selftest_wait_expiry(lvspec_ctx_t *ctx, int32_t limit_ms)
     int launches = 0;
     e = launch_wait_expiry(ctx->status, (unsigned long long)limit_ms * 1000000ull, ctx->stream, &launches);
     ctx->launches += launches;
+    // words left behind, as by an attention call that gave up
+    if (e == cudaSuccess)
+        e = cudaMemsetAsync(static_cast<char *>(ctx->exchange) + kMergeWordBytes, 0, ctx->exchange_bytes - kMergeWordBytes,
+                            ctx->stream);
     if (e != cudaSuccess) return cuda_fail(ctx, "self-test kernel launch", e);
     return LVSPEC_OK;
 }

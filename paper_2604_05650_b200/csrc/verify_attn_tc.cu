@@ -134,7 +134,7 @@ inline SmemMap smem_map(const TcConfig &c)
     s.dl = o;   o += c.n_pad * 4;
     s.tmx = o;  o += 4 * c.n_pad * 4;
     s.bars = o; o += 8 * (2 * c.ks + 2 * c.vs + 4 * kHand + 4);
-    s.misc = o; o += 16 + 4 * kSoftmaxWarps + 16;     // TMEM address, abort flag, epoch of m, committed tiles, per-warp maxima of |q|, arrival counted
+    s.misc = o; o += 16 + 4 * kSoftmaxWarps + 16;     // TMEM address, abort flag, epoch of m, committed tiles, per-warp maxima of |q|, arrival counted, exchange buffer in doubt
     s.pages = o; o += 4 * c.page_slots;
     s.total = o;
     return s;
@@ -410,6 +410,10 @@ __device__ __forceinline__ void softmax_share_bf16(uint32_t s_addr, int n_c, con
 // whose partials are written, and its upper half has a bit for every share given up; both move in one
 // atomic operation, so either the one who gives up sees that all have arrived (and reads on) or the
 // last to arrive sees the bit, and merges that share itself by the same arithmetic.
+// A CTA that leaves because a wait has run out may leave words behind that nobody makes kNoWord again.
+// It has raised LVSPEC_DEV_WAIT_EXPIRED, and while that stands (lvspec_device_status puts the buffer
+// in order and takes it back) a word that has been written need not be this launch's: CTAs then
+// read nothing before all of their head's have arrived, and give their shares up until then.
 __device__ __forceinline__ bool all_there(const uint4 &x)
 {
     return x.x != kNoWord && x.y != kNoWord && x.z != kNoWord && x.w != kNoWord;
@@ -633,6 +637,7 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
     volatile uint32_t *epoch_s = reinterpret_cast<volatile uint32_t *>(gbase + sm.misc + 8);
     volatile uint32_t *committed_s = reinterpret_cast<volatile uint32_t *>(gbase + sm.misc + 12);
     volatile uint32_t *arrived_s = reinterpret_cast<volatile uint32_t *>(gbase + sm.misc + 16 + 4 * kSoftmaxWarps);
+    volatile uint32_t *doubt_s = arrived_s + 1;      // (the first softmax thread's)
 
     // barrier addresses
     const uint32_t bar0 = base + sm.bars;
@@ -1092,6 +1097,9 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
         }
     } else {
         // ------------------------------------------------------------ softmax warps
+        // (read while nothing else is to be done: the first S^T is a tile's load and products away)
+        if (warp == kSoftmaxWarp0 && lane == 0)
+            *doubt_s = p.merge ? *static_cast<volatile uint32_t *>(p.status) & LVSPEC_DEV_WAIT_EXPIRED : 0u;
         const int grp = (warp - kSoftmaxWarp0) >> 2;    // tiles grp, grp + 3, ... are this group's
         const int bar_id = 1 + grp;
         const int wq = warp & 3;                        // TMEM lane quarter of this warp
@@ -1583,7 +1591,7 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
             float4 *sums = reinterpret_cast<float4 *>(gbase + sm.k);   // the rings are empty by now
             volatile uint32_t *verdict = epoch_s;
             unsigned long long *word = p.merge_word + bh;
-            bool mine;
+            bool mine, doubt = w == 0 && lane == 0 && *doubt_s != 0u;
             uint64_t since = 0;
             for (;;) {
                 MergedRow res;
@@ -1595,7 +1603,7 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                 uint32_t late;
                 asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 q, %2, 0;\n\tbar.red.or.pred p, %1, %3, q;\n\t"
                              "selp.u32 %0, 1, 0, p;\n\t}"
-                             : "=r"(late) : "r"(kQBarrier), "r"((uint32_t)!got), "n"(kSoftmaxThreads) : "memory");
+                             : "=r"(late) : "r"(kQBarrier), "r"((uint32_t)(!got || doubt)), "n"(kSoftmaxThreads) : "memory");
                 mine = true;
                 if (!late) {
                     if (part == 0 && slot < rows) {
@@ -1618,6 +1626,7 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                         const uint32_t arrived = (uint32_t)atomicOr(word, bit);
                         if (arrived == 0) atomicAnd(word, ~bit);
                         keep = arrived == 0 || arrived >= (uint32_t)n_eff ? 1u : 0u;
+                        if (keep) doubt = false;       // every word there is from this launch now
                     }
                     if (keep && *abort_flag == 0) {
                         // (the data are there or on their way: a bound all the same)

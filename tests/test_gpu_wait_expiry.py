@@ -37,3 +37,49 @@ def test_expired_wait_is_reported_and_the_context_stays_usable(oracle_mod):
             ctx.selftest_wait_expiry(0)
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("polls", [None, 0])
+def test_calls_after_an_expired_wait_are_right(polls, monkeypatch):
+    """An expired wait may leave words in the buffer through which the splits' partials go.  The calls
+    after it must not take them for their own, whether or not the status has been read."""
+    import torch
+    from paper_2604_05650_b200 import binding
+    from gpu_util import dev_bf16
+    if polls is not None:
+        monkeypatch.setenv("LVSPEC_MERGE_POLLS", str(polls))
+    ctx = binding.Context(0)
+    ctx.set_stream(torch.cuda.current_stream().cuda_stream)
+    calls = []
+    # the widest merging launch first; (KV heads, G, gamma, D, length, splits)
+    for hkv, G, gamma, D, L, ns in ((4, 7, 8, 128, 4113, 32), (2, 8, 9, 128, 900, 6), (2, 4, 4, 64, 1024, 8)):
+        rng = np.random.default_rng(ns)
+        bf = lambda *s: dev_bf16(W.f32_to_bf16_bits(rng.standard_normal(s).astype(np.float32)))
+        calls.append((binding.attn_shape(1, gamma, hkv * G, hkv, D, L, ns),
+                      bf(1, gamma, hkv * G, D), bf(1, hkv, L, D), bf(1, hkv, L, D), [L], [[9, L // 2]]))
+
+    def results():
+        res = []
+        for shape, q, k, v, lens, span in calls:       # one after the other, no synchronisation between
+            out, mass = torch.empty_like(q), torch.empty(q.shape[:3], device="cuda")
+            ctx.verify_attention(shape, q, k, v, lens, span, out, mass)
+            res += [out, mass]
+        return res
+
+    try:
+        first = results()
+        assert ctx.device_status_code() == (binding.OK, 0)
+        assert all(torch.isfinite(x.float()).all() for x in first)
+        ctx.selftest_wait_expiry(1)
+        for _ in range(5):
+            for a, b in zip(first, results()):
+                assert torch.equal(a, b)
+        assert ctx.device_status_code() == (binding.ERR_TIMEOUT, binding.DEV_WAIT_EXPIRED)
+        before = ctx.launch_count()
+        for _ in range(5):
+            for a, b in zip(first, results()):
+                assert torch.equal(a, b)
+        assert ctx.launch_count() - before == 5 * len(calls)       # all of them merge inside the launch
+        assert ctx.device_status_code() == (binding.OK, 0)
+    finally:
+        ctx.close()
