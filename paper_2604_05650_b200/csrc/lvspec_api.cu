@@ -633,7 +633,9 @@ lvspec_status_t lvspec_device_status(lvspec_ctx_t *ctx, uint32_t *flags)
     *flags = h;
     if (h & LVSPEC_DEV_WAIT_EXPIRED) {
         // an attention call that gave up may have left words behind
-        if ((e = reset_exchange(ctx)) != cudaSuccess) return cuda_fail(ctx, "resetting the exchange buffer", e);
+        // (done before this returns: the caller may go on on another stream)
+        if ((e = reset_exchange(ctx)) != cudaSuccess || (e = cudaStreamSynchronize(ctx->stream)) != cudaSuccess)
+            return cuda_fail(ctx, "resetting the exchange buffer", e);
         return fail(ctx, LVSPEC_ERR_TIMEOUT, "a bounded device-side wait ran out");
     }
     return LVSPEC_OK;

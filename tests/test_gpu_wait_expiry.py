@@ -83,3 +83,20 @@ def test_calls_after_an_expired_wait_are_right(polls, monkeypatch):
         assert ctx.device_status_code() == (binding.OK, 0)
     finally:
         ctx.close()
+
+
+def test_reading_the_status_leaves_nothing_on_the_stream():
+    """A caller may go on on another stream once the status has been read: what the reading puts in
+    order is in order by then."""
+    import torch
+    from paper_2604_05650_b200 import binding
+    ctx = binding.Context(0)
+    stream = torch.cuda.Stream()
+    ctx.set_stream(stream)
+    try:
+        for _ in range(20):
+            ctx.selftest_wait_expiry(1)
+            assert ctx.device_status_code() == (binding.ERR_TIMEOUT, binding.DEV_WAIT_EXPIRED)
+            assert stream.query()
+    finally:
+        ctx.close()
