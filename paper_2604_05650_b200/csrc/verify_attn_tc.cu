@@ -1622,6 +1622,7 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                 if (w == 0 && lane == 0) {
                     uint32_t keep = 1u;
                     if (*arrived_s) {
+                        __threadfence_block();      // with the one ahead of arrived_s: this CTA's arrival is in the word
                         const unsigned long long bit = 1ull << (32 + split);
                         const uint32_t arrived = (uint32_t)atomicOr(word, bit);
                         if (arrived == 0) atomicAnd(word, ~bit);
@@ -1679,7 +1680,6 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
             if (lane == 0) {
                 __threadfence();
                 before = atomicAdd(word, 1ull);
-                *arrived_s = 1;
             }
             before = __shfl_sync(0xffffffffu, before, 0);
             if ((uint32_t)before == (uint32_t)n_eff - 1u) {
@@ -1714,7 +1714,14 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                 }
                 if (lane == 0) atomicExch(word, 0ull);
             }
-            if (lane == 0) grid_launch_dependents();
+            if (lane == 0) {
+                grid_launch_dependents();
+                // The arrival comes before whatever the softmax warps do to the word once they see this.  All
+                // are threads of one CTA: its scope is enough (a fence for the device holds the CTA's end up,
+                // 0.3 us a layer of 4K or 16K).
+                __threadfence_block();
+                *arrived_s = 1;
+            }
 #ifdef LVSPEC_TRACE
             if (rec) rec[7] = lvspec_trace_now();
 #endif
