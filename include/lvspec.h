@@ -105,9 +105,13 @@ typedef struct {
  * read any input).  The environment variable LVSPEC_NO_PDL=1, read here, makes
  * them plain launches; LVSPEC_MERGE_POLLS=n, read here too, is how often an attention CTA
  * asks for the partials of its head's other CTAs before it leaves its rows to the last of them
- * (128; 0 for tests).  The relevance score's kernels are always launched so; the
+ * (lvspec_merge_polls).  The relevance score's kernels are always launched so; the
  * plain attention kernel and lvspec_loose_accept_static never. */
 lvspec_status_t lvspec_create(lvspec_ctx_t **ctx, int device);
+
+/* The number of requests that LVSPEC_MERGE_POLLS=`text` stands for: 0..4096, what is larger
+ * counting as 4096 (about 1.3 ms); 128 if `text` is NULL (not set) or not a number. */
+int32_t lvspec_merge_polls(const char *text);
 
 /* Synchronises the context's stream, frees its scratch memory and the context. */
 lvspec_status_t lvspec_destroy(lvspec_ctx_t *ctx);

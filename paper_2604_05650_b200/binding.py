@@ -35,7 +35,7 @@ EXPORTS = (
     "lvspec_verify_attention_spans", "lvspec_last_device_status",
     "lvspec_attention_workspace_bytes", "lvspec_accept_workspace_bytes",
     "lvspec_relevance_workspace_bytes", "lvspec_workspace_capacity", "lvspec_reserve",
-    "lvspec_verify_attention_fp8", "lvspec_verify_attention_strided",
+    "lvspec_verify_attention_fp8", "lvspec_verify_attention_strided", "lvspec_merge_polls",
 )
 
 
@@ -77,6 +77,8 @@ def load_library(path: Optional[str] = None) -> ctypes.CDLL:
     S = ctypes.POINTER(AttnShape)
     T = ctypes.POINTER(Thresholds)
     lib.lvspec_create.argtypes = [ctypes.POINTER(vp), ctypes.c_int]
+    lib.lvspec_merge_polls.argtypes = [ctypes.c_char_p]
+    lib.lvspec_merge_polls.restype = i32
     lib.lvspec_destroy.argtypes = [vp]
     lib.lvspec_set_stream.argtypes = [vp, vp]
     lib.lvspec_device_status.argtypes = [vp, ctypes.POINTER(ctypes.c_uint32)]

@@ -29,7 +29,7 @@ struct lvspec_ctx {
     uint64_t launches = 0;
     void *exchange = nullptr;         // words of the merge inside the attention kernel, then its partials
     size_t exchange_bytes = 0;
-    uint32_t merge_polls = 128;       // see AttnParams; about 100 us
+    uint32_t merge_polls = 128;       // see AttnParams
     bool pdl = true;                  // programmatic dependent launch between the attention kernels
     std::string error;
 };
@@ -532,6 +532,18 @@ int lvspec_trace_set_buffer(unsigned long long *device_words)
 }
 #endif
 
+int32_t lvspec_merge_polls(const char *text)
+{
+    // 0: every CTA that has to wait for a partial gives its share up.  4096: over a millisecond.  The polls
+    // look at no clock, so their number is the bound of the wait.
+    constexpr int32_t kUnset = 128, kMost = 4096;
+    if (!text || text[0] < '0' || text[0] > '9') return kUnset;
+    char *end = nullptr;
+    const unsigned long n = std::strtoul(text, &end, 10);
+    if (*end) return kUnset;
+    return n < (unsigned long)kMost ? (int32_t)n : kMost;
+}
+
 lvspec_status_t lvspec_create(lvspec_ctx_t **out, int device)
 {
     if (!out) {
@@ -571,8 +583,7 @@ lvspec_status_t lvspec_create(lvspec_ctx_t **out, int device)
         return LVSPEC_ERR_UNSUPPORTED;
     }
     ctx->n_sm = prop.multiProcessorCount;
-    // (0: every CTA that has to wait for a partial gives its share up; for tests)
-    if (const char *e = std::getenv("LVSPEC_MERGE_POLLS")) ctx->merge_polls = (uint32_t)std::strtoul(e, nullptr, 10);
+    ctx->merge_polls = (uint32_t)lvspec_merge_polls(std::getenv("LVSPEC_MERGE_POLLS"));
     if (const char *e = std::getenv("LVSPEC_NO_PDL")) ctx->pdl = !(e[0] && e[0] != '0');
     // status word and counters, then the exchange buffer, in one allocation
     const size_t counted = sizeof(uint32_t) * (1 + LVSPEC_MAX_BATCH + LVSPEC_MAX_BATCH * LVSPEC_MAX_GAMMA);

@@ -68,3 +68,11 @@ def test_product_package_does_not_import_the_oracle():
                 text = open(os.path.join(dirpath, fn)).read()
                 assert not re.search(r"^\s*(from|import)\s+oracle\b", text, flags=re.M), fn
                 assert "lvspec_oracle" not in text, fn
+
+
+@pytest.mark.parametrize("text, polls", [
+    (None, 128), (b"0", 0), (b"1", 1), (b"128", 128), (b"4096", 4096), (b"4097", 4096), (b"4294967295", 4096),
+    (b"4294967296", 4096), (b"99999999999999999999999", 4096), (b"", 128), (b"-1", 128), (b" 7", 128), (b"+7", 128),
+    (b"7x", 128), (b"many", 128), (b"0x10", 128)])
+def test_merge_polls_are_bounded(lib, text, polls):
+    assert lib.lvspec_merge_polls(text) == polls
