@@ -31,6 +31,7 @@ struct lvspec_ctx {
     size_t exchange_bytes = 0;
     uint32_t merge_polls = 128;       // see AttnParams
     bool pdl = true;                  // programmatic dependent launch between the attention kernels
+    bool gpu_shared = false;          // other work runs on the GPU beside this context's
     std::string error;
 };
 
@@ -318,10 +319,13 @@ static_assert(kMergeWordBytes >= 8 * 256, "a word per CTA of the widest device")
 
 // Do this call's CTAs merge their splits themselves?  They wait for one another, so all have to run at
 // once: one CTA per SM, one wave.  A share is at most twelve rows (a warp each) and a head has at most 32
-// splits (a bit each); a head of more splits, or of more rows a split, goes to the merge kernel.
+// splits (a bit each); a head of more splits, or of more rows a split, goes to the merge kernel.  So does
+// all on a shared GPU: a CTA that waits for its head's others holds its SM meanwhile, and CTAs that start as
+// SMs come free wait long.  Two contexts' passes at once, us a pass, merge inside / merge kernel: 64 layers of
+// 4K 464 / 320, of 32K 1600 / 1435.
 bool merges_itself(const lvspec_ctx *ctx, const AttnParams &p, const SeqInfo &seq)
 {
-    if (p.n_split < 2 || p.n_split > kMergeSplits || p.B * p.Hkv * p.n_split > ctx->n_sm) return false;
+    if (ctx->gpu_shared || p.n_split < 2 || p.n_split > kMergeSplits || p.B * p.Hkv * p.n_split > ctx->n_sm) return false;
     for (int b = 0; b < p.B; ++b) {
         const int tiles = (seq.kv_len[b] + 127) / 128;
         if (p.M > kMergeRows * (tiles < p.n_split ? tiles : p.n_split)) return false;
@@ -629,6 +633,13 @@ lvspec_status_t lvspec_set_stream(lvspec_ctx_t *ctx, void *cuda_stream)
 {
     if (!ctx) return LVSPEC_ERR_INVALID_ARG;
     ctx->stream = static_cast<cudaStream_t>(cuda_stream);
+    return LVSPEC_OK;
+}
+
+lvspec_status_t lvspec_set_gpu_shared(lvspec_ctx_t *ctx, int32_t shared)
+{
+    if (!ctx) return LVSPEC_ERR_INVALID_ARG;
+    ctx->gpu_shared = shared != 0;
     return LVSPEC_OK;
 }
 

@@ -91,3 +91,18 @@ def test_two_contexts_share_the_gpu(monkeypatch):
         for out, mass in o:
             assert torch.equal(out, outs[0][0][0]) and torch.equal(mass, outs[0][0][1])
         ctx.close()
+
+
+@pytest.mark.parametrize("name", [n for n, (c, merged) in CASES.items() if merged])
+def test_on_a_shared_gpu_a_kernel_merges(name, oracle_mod, monkeypatch):
+    from gpu_util import assert_attention_close, run_attention
+    q, k, v, lens, span, ns = _inputs(CASES[name][0], 29)
+    ref = oracle_mod.verify_attention(q, k, v, lens, span)
+    ctx = _contexts(monkeypatch)
+    for shared, launches in ((True, 2), (False, 1), (True, 2)):
+        ctx.set_gpu_shared(shared)
+        before = ctx.launch_count()
+        got = run_attention(ctx, q, k, v, lens, span, ns)
+        assert ctx.launch_count() - before == launches
+        assert_attention_close(*got, *ref)
+    ctx.close()
