@@ -554,12 +554,17 @@ __device__ __forceinline__ void clear_part(const AttnParams &p, const MergePart 
 // work on every tile, each on a share of its columns, at most kC chunks of eight.
 // Draft trees and page pools are run-time cases (a mask range per position, a look-up per
 // tile): as template cases they gave nothing.
-template <bool kFp8, bool kTurns, int kC>
+// kMerge: the launch may merge its splits itself.  With a bf16 cache a case of its own, because that code
+// takes registers (128 a thread against 104 to 116): without it another kernel's CTAs find room beside this one's.
+// With an fp8 cache it is 128 either way, and one instance decides by p.merge.
+template <bool kFp8, bool kTurns, int kC, bool kMerge>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUtensorMap tmap_k,
                const __grid_constant__ CUtensorMap tmap_v, const __grid_constant__ CUtensorMap tmap_q)
 {
     static_assert(kFp8 || !kTurns, "a bf16 cache does not go through in turns");
+    static_assert(kMerge || !kFp8, "one instance per organisation of an fp8 cache");
+    auto merges = [&] { return kFp8 ? P.a.merge != 0 : kMerge; };     // (asked anew: a register less)
     // bytes of one K or V tile: two 64-channel boxes at head_dim 128 (bf16), one box at
     // head_dim 64 and for an fp8 tile of 128 channels
     const uint32_t kSlot = (uint32_t)P.cfg.slot_bytes;
@@ -620,7 +625,7 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
             grid_launch_dependents();
         }
         __syncthreads();
-        for (int r = tid; !p.merge && r < M; r += kThreads)
+        for (int r = tid; !merges() && r < M; r += kThreads)
             *reinterpret_cast<float4 *>(part_stat + r * 4) = make_float4(kMFloor, 0.f, 0.f, 0.f);
         return;
     }
@@ -1098,8 +1103,8 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
     } else {
         // ------------------------------------------------------------ softmax warps
         // (read while nothing else is to be done: the first S^T is a tile's load and products away)
-        if (warp == kSoftmaxWarp0 && lane == 0)
-            *doubt_s = p.merge ? *static_cast<volatile uint32_t *>(p.status) & LVSPEC_DEV_WAIT_EXPIRED : 0u;
+        if (kMerge && warp == kSoftmaxWarp0 && lane == 0)
+            *doubt_s = merges() ? *static_cast<volatile uint32_t *>(p.status) & LVSPEC_DEV_WAIT_EXPIRED : 0u;
         const int grp = (warp - kSoftmaxWarp0) >> 2;    // tiles grp, grp + 3, ... are this group's
         const int bar_id = 1 + grp;
         const int wq = warp & 3;                        // TMEM lane quarter of this warp
@@ -1554,13 +1559,17 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
 #pragma unroll
                     for (int k = 0; k < 8; ++k) o8[k] *= v_scale;
                 }
+                auto put = [&](int k) {
+                    if constexpr (kMerge) st_relaxed(po + k * D, passable(o8[k]));
+                    else po[k * D] = o8[k];
+                };
                 if (c8 * 8 + 8 <= m_store) {
 #pragma unroll
-                    for (int k = 0; k < 8; ++k) st_relaxed(po + k * D, passable(o8[k]));
+                    for (int k = 0; k < 8; ++k) put(k);
                 } else {
 #pragma unroll
                     for (int k = 0; k < 8; ++k)
-                        if (c8 * 8 + k < m_store) st_relaxed(po + k * D, passable(o8[k]));
+                        if (c8 * 8 + k < m_store) put(k);
                 }
             }
             if (wq == 0) {
@@ -1576,9 +1585,12 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                         const float c = __shfl_sync(0xffffffffu, lsum[k], 1);
                         if (lane == k) { lk = a; lvk = c; }
                     }
-                    if (lane < 8 && c8 * 8 + lane < M)
-                        st_relaxed_v4(part_stat + (c8 * 8 + lane) * 4,
-                                      make_uint4(passable(m_s[c8 * 8 + lane]), passable(lk), passable(lvk), 0u));
+                    if (lane < 8 && c8 * 8 + lane < M) {
+                        const float mk = m_s[c8 * 8 + lane];
+                        float *ps = part_stat + (c8 * 8 + lane) * 4;
+                        if constexpr (kMerge) st_relaxed_v4(ps, make_uint4(passable(mk), passable(lk), passable(lvk), 0u));
+                        else *reinterpret_cast<float4 *>(ps) = make_float4(mk, lk, lvk, 0.f);
+                    }
                 }
             }
         }
@@ -1586,7 +1598,7 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
         __syncwarp();
         if (lane == 0) mbar_arrive(done_bar);
 
-        if (p.merge) {
+        if (merges()) {
             // ------------------------------------------------------------ merge
             float4 *sums = reinterpret_cast<float4 *>(gbase + sm.k);   // the rings are empty by now
             volatile uint32_t *verdict = epoch_s;
@@ -1666,12 +1678,12 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
             // this CTA is done but for freeing TMEM: a dependent launch may be scheduled
             // once every CTA has come this far (earlier, its CTAs would pile up on the
             // few SMs this grid leaves idle; with the merge to come, later still)
-            if (!p.merge) grid_launch_dependents();
+            if (!merges()) grid_launch_dependents();
         }
         __syncwarp();
         tc_fence_after();
         tmem_dealloc(tmem_base, (uint32_t)cfg.tmem_cols);
-        if (p.merge) {
+        if (merges()) {
             // this CTA's partials are written; the head's last one to say so sees to the shares that
             // others have given up, and leaves the word as the next call expects it
             const int n_eff = min(p.n_split, n_tiles);
@@ -1895,9 +1907,11 @@ cudaError_t launch_attn_tc(const AttnParams &p, const SeqInfo &seq, cudaStream_t
     const bool tree = p.branch_len != p.gamma;
     if ((tree && paged) || (fp8 && (tree || paged))) return cudaErrorNotSupported;
     const int share = ((p.M + 7) / 8 + kSoftmaxGroups - 1) / kSoftmaxGroups;    // column chunks of a softmax group
-    auto kernel = fp8 ? (turns ? attn_tc_kernel<true, true, 1> : attn_tc_kernel<true, false, 4>)
-                  : share <= 2 ? attn_tc_kernel<false, false, 2>
-                  : share <= 4 ? attn_tc_kernel<false, false, 4> : attn_tc_kernel<false, false, kMaxChunks>;
+    auto kernel = fp8 ? (turns ? attn_tc_kernel<true, true, 1, true> : attn_tc_kernel<true, false, 4, true>)
+                  : p.merge ? (share <= 2 ? attn_tc_kernel<false, false, 2, true>
+                               : share <= 4 ? attn_tc_kernel<false, false, 4, true> : attn_tc_kernel<false, false, kMaxChunks, true>)
+                  : share <= 2 ? attn_tc_kernel<false, false, 2, false>
+                  : share <= 4 ? attn_tc_kernel<false, false, 4, false> : attn_tc_kernel<false, false, kMaxChunks, false>;
     cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
     cudaLaunchConfig_t cfg = {};
