@@ -139,6 +139,11 @@ lvspec_status_t lvspec_device_status(lvspec_ctx_t *ctx, uint32_t *flags);
  * since the previous reading have reported. */
 lvspec_status_t lvspec_last_device_status(lvspec_ctx_t *ctx, uint32_t *flags);
 
+/* Synchronises the stream and gives the number of shares of a head's rows that an attention CTA has left
+ * to another one, having waited in vain, since the context was created or an expired wait was last
+ * reported.  Zero while nothing else runs on the GPU; much more: see lvspec_set_gpu_shared. */
+lvspec_status_t lvspec_merge_handed_over(lvspec_ctx_t *ctx, uint64_t *shares);
+
 /* Text of the last error recorded on this context (never NULL; valid until the
  * next call on the context).  `ctx` may be NULL: then the text describes why
  * the last lvspec_create on this thread failed. */

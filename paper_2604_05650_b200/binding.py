@@ -36,7 +36,7 @@ EXPORTS = (
     "lvspec_attention_workspace_bytes", "lvspec_accept_workspace_bytes",
     "lvspec_relevance_workspace_bytes", "lvspec_workspace_capacity", "lvspec_reserve",
     "lvspec_verify_attention_fp8", "lvspec_verify_attention_strided", "lvspec_merge_polls",
-    "lvspec_set_gpu_shared",
+    "lvspec_set_gpu_shared", "lvspec_merge_handed_over",
 )
 
 
@@ -82,6 +82,7 @@ def load_library(path: Optional[str] = None) -> ctypes.CDLL:
     lib.lvspec_merge_polls.restype = i32
     lib.lvspec_destroy.argtypes = [vp]
     lib.lvspec_set_stream.argtypes = [vp, vp]
+    lib.lvspec_merge_handed_over.argtypes = [vp, ctypes.POINTER(u64)]
     lib.lvspec_set_gpu_shared.argtypes = [vp, i32]
     lib.lvspec_device_status.argtypes = [vp, ctypes.POINTER(ctypes.c_uint32)]
     lib.lvspec_last_device_status.argtypes = [vp, ctypes.POINTER(ctypes.c_uint32)]
@@ -202,6 +203,11 @@ class Context:
     def set_gpu_shared(self, shared: bool = True) -> None:
         """Other work runs on the GPU beside this context's: see ``lvspec_set_gpu_shared``."""
         self._check(self._lib.lvspec_set_gpu_shared(self._h, int(bool(shared))))
+
+    def merge_handed_over(self) -> int:
+        n = ctypes.c_uint64(0)
+        self._check(self._lib.lvspec_merge_handed_over(self._h, ctypes.byref(n)))
+        return int(n.value)
 
     def device_status(self) -> int:
         flags = ctypes.c_uint32(0)

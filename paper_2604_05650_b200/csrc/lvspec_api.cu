@@ -314,8 +314,8 @@ struct Fp8Cache {            // E4M3 codes with one scale per (sequence, KV head
     const float *k_scale = nullptr, *v_scale = nullptr;
 };
 
-constexpr size_t kMergeWordBytes = 4096;
-static_assert(kMergeWordBytes >= 8 * 256, "a word per CTA of the widest device");
+constexpr size_t kMergeWordBytes = 8 * kMergeWords;
+static_assert(kMergeCountWord >= 256, "a word per CTA of the widest device");
 
 // Do this call's CTAs merge their splits themselves?  They wait for one another, so all have to run at
 // once: one CTA per SM, one wave.  A share is at most twelve rows (a warp each) and a head has at most 32
@@ -660,6 +660,19 @@ lvspec_status_t lvspec_device_status(lvspec_ctx_t *ctx, uint32_t *flags)
             return cuda_fail(ctx, "resetting the exchange buffer", e);
         return fail(ctx, LVSPEC_ERR_TIMEOUT, "a bounded device-side wait ran out");
     }
+    return LVSPEC_OK;
+}
+
+lvspec_status_t lvspec_merge_handed_over(lvspec_ctx_t *ctx, uint64_t *shares)
+{
+    if (!ctx || !shares) return LVSPEC_ERR_INVALID_ARG;
+    cudaSetDevice(ctx->device);
+    unsigned long long n = 0;
+    cudaError_t e = cudaMemcpyAsync(&n, static_cast<unsigned long long *>(ctx->exchange) + kMergeCountWord, sizeof n,
+                                    cudaMemcpyDeviceToHost, ctx->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
+    if (e != cudaSuccess) return cuda_fail(ctx, "reading the count of shares handed over", e);
+    *shares = n;
     return LVSPEC_OK;
 }
 

@@ -119,6 +119,8 @@ __host__ __device__ inline bool draft_query_sees(int qi, int t, int branch_len)
 // Limits of the merge inside the attention kernel: splits of a head (a bit each in merge_word),
 // rows of a CTA's share (a warp each at most).
 constexpr int kMergeSplits = 32, kMergeRows = 12;
+constexpr int kMergeWords = 512;             // words ahead of the exchange buffer's rows: one per head, ...
+constexpr int kMergeCountWord = kMergeWords - 1;     // ... and how many shares were given up
 constexpr uint32_t kNoWord = 0xFFFFFFFFu;    // a word of the exchange buffer nobody has written
 
 // Partial results of one KV split, rows r = g * G + hg.

@@ -1104,7 +1104,7 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
         // ------------------------------------------------------------ softmax warps
         // (read while nothing else is to be done: the first S^T is a tile's load and products away)
         if (kMerge && warp == kSoftmaxWarp0 && lane == 0)
-            *doubt_s = merges() ? *static_cast<volatile uint32_t *>(p.status) & LVSPEC_DEV_WAIT_EXPIRED : 0u;
+            *doubt_s = *static_cast<volatile uint32_t *>(p.status) & LVSPEC_DEV_WAIT_EXPIRED;
         const int grp = (warp - kSoftmaxWarp0) >> 2;    // tiles grp, grp + 3, ... are this group's
         const int bar_id = 1 + grp;
         const int wq = warp & 3;                        // TMEM lane quarter of this warp
@@ -1639,7 +1639,8 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                         const uint32_t arrived = (uint32_t)atomicOr(word, bit);
                         if (arrived == 0) atomicAnd(word, ~bit);
                         keep = arrived == 0 || arrived >= (uint32_t)n_eff ? 1u : 0u;
-                        if (keep) doubt = false;       // every word there is from this launch now
+                        if (!keep) atomicAdd(p.merge_word + kMergeCountWord, 1ull);
+                        else doubt = false;            // every word there is from this launch now
                     }
                     if (keep && *abort_flag == 0) {
                         // (the data are there or on their way: a bound all the same)
