@@ -127,9 +127,12 @@ int resolve_kernel(const lvspec_attn_shape_t *s)
 // their CTA count reaches, the uneven last round at the bandwidth of its few CTAs, and a
 // charge per CTA for writing its partial and merging it, and one for each round of 32 splits
 // of the merge (with one or two KV heads the most CTAs are 74 or 148 splits: a head of 32K at
-// 32 rows takes 13.1 us with 64 splits, 13.8 with 86, 15.4 with 128; two heads of 16K at 4
-// rows 10.7 with 32, 11.5 with 64, 12.6 with 74).  A pure function of the shape: results stay
-// reproducible from run to run.
+// 32 rows takes 12.5 us with 32 splits, 12.3 with 64, 13.1 with 86, 14.7 with 128; two heads of 16K
+// at 4 rows 8.9 with 32, 10.9 with 64, 11.9 with 74).  The charge is that of a round of the merge
+// kernel; what more than 32 splits cost by leaving the merge inside the launch (merges_itself) is not
+// in it: one head of 16K at 8 rows takes 9.8 us with the 64 splits it gets, 8.8 with 32, two heads of
+// 32K at 40 rows 14.0 with 64, 13.7 with 32.  A pure function of the shape: results stay reproducible
+// from run to run.
 struct SplitModel {
     int units, tiles, most;     // (sequence, KV head) pairs; tiles of the longest sequence; splits of one wave
     double saturating;          // CTAs that reach the HBM bandwidth
@@ -852,8 +855,8 @@ lvspec_status_t lvspec_verify_attention_spans(lvspec_ctx_t *ctx, const lvspec_at
     if (st != LVSPEC_OK) return st;
     cudaError_t e = cudaSetDevice(ctx->device);
     if (e != cudaSuccess) return cuda_fail(ctx, "cudaSetDevice", e);
-    // the log2 denominators come from the combine kernel: at least two splits where the
-    // tensor-core kernel would otherwise finish alone (the plain kernel always combines)
+    // the log2 denominators come from the merge of the splits, in the launch or in a kernel of its own:
+    // at least two splits where the tensor-core kernel would otherwise finish alone (the plain kernel always merges)
     lvspec_attn_shape_t s = *shape;
     if (resolve_kernel(&s) == LVSPEC_KERNEL_TCGEN05 && s.n_split == 0 && choose_splits(ctx, &s, max_len) < 2) {
         if (max_len > 128) s.n_split = 2;

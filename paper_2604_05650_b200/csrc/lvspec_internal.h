@@ -79,7 +79,7 @@ struct AttnParams {
     float *mass;           // [B, gamma, Hq]
     float *part_o;         // [B, Hkv, n_split, M, D] fp32, unnormalised
     float *part_stat;      // [B, Hkv, n_split, M, 4]: m (log2 units), l, l_vis, unused
-    float *lse2;           // optional [B, gamma, Hq]: log2 of the softmax denominator, written by the combine
+    float *lse2;           // optional [B, gamma, Hq]: log2 of the softmax denominator, written by whoever merges the splits
     uint32_t *status;      // device status word
     // Merge inside the attention kernel (see verify_attn_tc.cu): part_o and part_stat are then in the
     // context's exchange buffer, every word of which is kNoWord between calls, and merge_word has

@@ -4,7 +4,7 @@
 // spans they run on the hull [first start, last end), and this kernel takes off
 // what the positions between the spans hold: for every gap position j and query
 // row, p_j = exp2(scale * <q, k_j> - lse2), with lse2 the log2 of the row's softmax
-// denominator that the combine kernel leaves behind.  Gap positions are few (a few
+// denominator that the merge of the splits leaves behind.  Gap positions are few (a few
 // text tokens per frame), only the layer whose mass feeds the rule needs it, and
 // all of them lie before the draft slots, so every draft query sees them.
 //

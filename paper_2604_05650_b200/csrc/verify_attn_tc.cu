@@ -655,13 +655,16 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
     // S^T and P^T buffers: a parity wait tells a phase from its neighbours only, so whoever
     // waits for a phase must know the phase before it to be over, and the one after it not to
     // be.  Products end in order, and no product of a tile that is not yet handed over can end.
-    // In turns a group has waited for the product of tile i - 3 - pb before it comes to tile i, and so
-    // for all before it (pb <= 4: every phase it may wait for is the next one of its barrier), and the
-    // K.Q^T of tile i + 4 waits until the group has read tile i (at most four S^T buffers).
-    // With shared columns every group waits for the
-    // product of tile i - pb before it writes tile i: with pb <= 4 no tile's phase is further than
-    // one from what a group may wait for.
+    // Whoever writes tile i has first waited for the product of tile i - pb, in turns as with
+    // shared columns, and only then waits for that of tile i - 1 (ahead of a rescale, or of zeroing V
+    // rows): with pb <= 4 the phase before that one, tile i - 5's, is over by then, while tile i - 4
+    // being done a turn ago is nothing that could be relied on.  The wait for tile i - pb itself comes
+    // after the one for tile i - 3 - pb (in turns, a turn ago) or i - 1 - pb (shared columns).  The K.Q^T of
+    // tile i + 4 waits until tile i has been read (at most four S^T buffers).
     constexpr int kRound = kHand;
+    static_assert(kHand == 4, "as many S^T and P^T buffers at most: see above");
+    static_assert(kMergeRows <= kSoftmaxWarps, "a warp per row of a share");
+    static_assert(kMergeSplits <= 32, "a bit of the word's upper half and a lane per split");
     auto s_full = [&](int i) { return bar1 + 8 * (i % kRound); };
     auto s_free = [&](int i) { return bar1 + 8 * (kHand + i % kRound); };
     auto p_full = [&](int i) { return bar1 + 8 * (2 * kHand + i % kRound); };
@@ -1190,7 +1193,7 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                 const bool tail = pos0 + kTilePos > L - gamma;
                 const Seen seen = seen_by(tail ? pos - L + gamma : -1, G, gamma, p.branch_len);
                 // P^T goes straight to shared memory: the P.V product that read this buffer last is done
-                // (tile i - pb; this group saw tile i - 3 - pb's product done a turn ago)
+                // (tile i - pb).  This wait stays ahead of those for tile i - 1 below: see kRound.
                 if (i >= cfg.pb) mbar_wait(p_free(i - cfg.pb), hand_parity(i - cfg.pb), abort_flag);
                 if (warp == kSoftmaxWarp0) LVSPEC_TILE_TS(tile_tr, 0, i, 2);     // P buffer free
                 uint8_t *prow = gbase + sm.p + pb * (NP * 256) + row * 16;
@@ -1258,8 +1261,7 @@ attn_tc_kernel(const TcParams P, const SeqInfo seq, const __grid_constant__ CUte
                     }
                     if (i > 0) {
                         // O^T and the sums were accumulated under the old m: rescale them once
-                        // the P.V product of tile i - 1 has finished (tile i - 1 is committed, so
-                        // its group has seen the product of tile i - 4 or a later one done)
+                        // the P.V product of tile i - 1 has finished (that of tile i - pb has: see kRound)
                         mbar_wait(p_free(i - 1), hand_parity(i - 1), abort_flag);
                         tc_fence_after();
                         // (fp8 cache: accumulator columns 2n and 2n + 1 belong to row n)
@@ -1827,12 +1829,12 @@ TcConfig pick_config(int M, int page_slots, bool fp8, bool turns, int D)
     } else {
         // Tiles in turn (fp8 cache): as many S^T buffers as TMEM has columns for, up to one more than
         // there are softmax groups: the K.Q^T of a group's next tile is then done when the group
-        // comes to it (40 rows, 64 layers of 32K: 20.4 us a layer with four, 20.6 with three, 20.4 with
-        // five or six).  A fourth P^T buffer too: with three a group waited for the product of its tile
-        // before, which is in the queue behind two others'.  Then also more slots of 16 KB (us a layer of 32K, 40 rows:
-        // 19.8 with 3 + 3 slots and three P^T buffers, 19.5 with 3 + 3 and four, 19.1 with 4 + 4, 19.3 with 5 + 4;
-        // 56 rows of 64K: 25.6, 24.8, 25.1; 80 rows: 33.3 with 2 + 3 and three, 33.6 with 3 + 3, 33.4 with a fourth P^T
-        // buffer, 33.8 with more slots).
+        // comes to it.  A fourth P^T buffer too: with three a group waited for the product of its tile
+        // before, which is in the queue behind two others'.  Then also more slots of 16 KB.  us a layer, by
+        // K + V slots / P^T buffers / S^T buffers:
+        //   40 rows of 32K: 3 + 3 / 3 / 3 19.4, 3 + 3 / 3 / 4 19.2, 3 + 3 / 4 / 4 19.0, 4 + 4 / 4 / 4 18.5, 5 + 4 / 4 / 4 18.6
+        //   56 rows of 64K: 23.9, 23.7, 23.0, 23.4, does not fit
+        //   80 rows of 32K (two S^T buffers): 2 + 3 / 3 30.9, 2 + 3 / 4 31.0, 3 + 3 / 3 31.2, 3 + 3 / 4 31.5
         c.sb = 512 / c.n_pad - acc;
         if (c.sb > kHand) c.sb = kHand;
         const int tries[6][3] = {{4, 4, 4}, {3, 3, 4}, {2, 3, 3}, {3, 3, 2}, {3, 3, 1}, {2, 2, 1}};

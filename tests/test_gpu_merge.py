@@ -67,7 +67,7 @@ def test_both_sides_of_each_limit(name, oracle_mod, monkeypatch):
 
 def test_two_contexts_share_the_gpu(monkeypatch):
     """Attention calls of two contexts on two streams: grids whose CTAs may get SMs in any order.  (No
-    grid waits for another: a CTA that waits in vain leaves after about 100 us.)"""
+    grid waits for another: a CTA that waits in vain leaves after some 40 us.)"""
     import torch
     from gpu_util import dev_bf16
     from paper_2604_05650_b200 import binding
