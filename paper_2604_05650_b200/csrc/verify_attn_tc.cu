@@ -1885,8 +1885,8 @@ cudaError_t launch_attn_tc(const AttnParams &p, const SeqInfo &seq, cudaStream_t
     // paged: one block-table entry per tile of the longest split, rounded up to 4
     const int tiles = (p.Lmax + kTilePos - 1) / kTilePos;
     const bool fp8 = p.fp8 != 0;
-    // Tiles in turn with an fp8 cache (half the bytes per tile for the same work: 24.2 us a layer
-    // at 40 rows of 32K against 29.0 with shared columns, 33.9 against 35.3 at 80).  A bf16
+    // Tiles in turn with an fp8 cache (half the bytes per tile for the same work: 18.4 us a layer
+    // at 40 rows of 32K against 23.5 with shared columns, 30.6 against 34.3 at 80).  A bf16
     // cache goes through with shared columns, in pairs of tiles where that pays, which beats
     // turns at every length (long streams of 80 rows: 321 us against 331).
     // LVSPEC_TC_TURNS=0/1 overrides the choice with an fp8 cache (for measurements).

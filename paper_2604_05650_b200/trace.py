@@ -105,7 +105,7 @@ def main() -> None:
         graph.replay()
         torch.cuda.synchronize()
     ctx.set_stream(stream.cuda_stream)
-    print("device status", ctx.device_status(), "| splits", ctx.attention_splits(shape, L),
+    print("device status", ctx.device_status(), "| splits", ctx.attention_splits(shape, L, args.fp8),
           "| cache", "E4M3" if args.fp8 else "bf16")
     w = words.cpu().numpy()
     lib.lvspec_trace_set_buffer(None)        # the buffer goes; kernels launched later must not write to it
